@@ -37,7 +37,8 @@ struct DevCtrl {
   int32_t K;
   int32_t total_events;
   unsigned counters[2];
-  unsigned pad[2];
+  unsigned ticket;       // blocks of k_group_count done
+  unsigned pad;
   double out[survgpu::OUT_COUNT];
   unsigned long long timing[survgpu::PH_COUNT];
   survgpu::GraphCtl gctl;
@@ -244,32 +245,32 @@ int stage_data(const surv_data* d, int prec, surv_workspace* ws, cudaStream_t s,
   return SURV_OK;
 }
 
-// Validation kernels on the staged data and the tie-group count: *K after a
-// synchronisation (ctrl zeroed here; prep errors mapped to return codes).
+// Validation kernels on the staged data and the tie-group count: *K and the
+// number of events after a synchronisation (ctrl zeroed here; prep errors mapped to return codes).
 // CSC values that are all exactly 1 are dropped from st (the kernels then
 // take every nonzero as 1, an indicator matrix): the arithmetic is the same
 // bit for bit (x e = e, x^2 = x, delta x = delta) and the values are not read
 // again.
 int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, Staged& st, DevCtrl* ctrl,
-                       surv_workspace* ws, cudaStream_t s, void** blockcnt, int32_t* K, int64_t* launches) {
+                       surv_workspace* ws, cudaStream_t s, void** cnt, int32_t* K, int32_t* events,
+                       int64_t* launches) {
   CUDA_TRY(cudaMemsetAsync(ctrl, 0, sizeof(DevCtrl), s));
-  CUDA_TRY(survgpu::prep_check_times(st.time, st.status, n, model, &ctrl->perr, s));
+  int rc;
+  if ((rc = ensure(ws, surv_workspace::BLOCKCNT, survgpu::prep_count_bytes(n), cnt))) return rc;
+  CUDA_TRY(survgpu::prep_group_count(st.time, st.status, n, model, *cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events,
+                                     &ctrl->ticket, s));
   ++*launches;
   if (layout == SURV_CSC)
     CUDA_TRY(survgpu::prep_check_csc(st.colptr, st.rowidx, st.vals, prec, p, n, &ctrl->perr, s));
   else
     CUDA_TRY(survgpu::prep_check_dense(st.vals, prec, st.ld, n, p, &ctrl->perr, s));
   ++*launches;
-  const int64_t nb = survgpu::prep_end_blocks(n);
-  int rc;
-  if ((rc = ensure(ws, surv_workspace::BLOCKCNT, 4 * (size_t)nb, blockcnt))) return rc;
-  CUDA_TRY(survgpu::prep_count_ends(st.time, n, static_cast<int32_t*>(*blockcnt), &ctrl->K, s));
-  *launches += 2;
   DevCtrl hc;
   CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   if ((rc = map_prep_error(hc.perr))) return rc;
   *K = hc.K;
+  *events = hc.total_events;
   if (layout == SURV_CSC && st.vals && !(hc.perr & survgpu::PREP_VALUES_NOT_ONE)) st.vals = nullptr;
   return SURV_OK;
 }
@@ -363,9 +364,10 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   DevCtrl* ctrl = static_cast<DevCtrl*>(ctrl_v);
   const int32_t* time_p = stg.time;
   const int8_t* status_p = stg.status;
-  void* blockcnt = nullptr;
-  int32_t K = 0;
-  if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &blockcnt, &K, &launches))) return rc;
+  void* cnt = nullptr;
+  int32_t K = 0, events = 0;
+  if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches))) return rc;
+  if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   const void* vals_d = stg.vals;  // null for indicator CSC data (all values 1)
   DevCtrl hc;
 
@@ -436,10 +438,10 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     S.multi = (int64_t)K >= 2 * (int64_t)nwarps ? 1 : 0;
   }
 
-  CUDA_TRY(survgpu::prep_write_ends(time_p, n, static_cast<const int32_t*>(blockcnt), static_cast<int32_t*>(gend), s));
-  CUDA_TRY(survgpu::prep_group_stats(static_cast<int32_t*>(gend), K, status_p, n, static_cast<int32_t*>(dk),
-                                     static_cast<int32_t*>(ck), &ctrl->total_events, s));
-  launches += 2;
+  CUDA_TRY(survgpu::prep_group_write(time_p, status_p, n, cnt, K, static_cast<int32_t*>(gend),
+                                     static_cast<int32_t*>(dk), static_cast<int32_t*>(ck), nwarps, rows_per_warp,
+                                     static_cast<int32_t*>(wk0), s));
+  ++launches;
   if (model == SURV_FG) {
     CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk),
                               static_cast<float2*>(Gkff), s));
@@ -456,9 +458,6 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     CUDA_TRY(survgpu::prep_dtx_dense(vals_d, prec, ld, n, status_p, p, static_cast<double*>(dTx), s));
     ++launches;
   }
-  CUDA_TRY(survgpu::prep_warp_groups(static_cast<int32_t*>(gend), K, n, nwarps, rows_per_warp,
-                                     static_cast<int32_t*>(wk0), s));
-  ++launches;
   CUDA_TRY(cudaMemcpyAsync(beta, beta_h.data(), 8 * (size_t)p, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(pen, pen_h.data(), 8 * (size_t)p, cudaMemcpyHostToDevice, s));
   CUDA_TRY(survgpu::prep_fill_f64(static_cast<double*>(width), 1.0, p, s));
@@ -491,9 +490,6 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     const unsigned long long big = ~0ull;
     CUDA_TRY(cudaMemcpyAsync(&ctrl->timing[survgpu::PH_PASS_MIN], &big, sizeof(big), cudaMemcpyHostToDevice, s));
   }
-  CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaStreamSynchronize(s));
-  if (hc.total_events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
 
   // ---------------------------------------------------------- CCD kernel
   CcdParams P;
@@ -653,29 +649,25 @@ int lambda_max_impl(const surv_data* d, const double* pf_in, double* out, void* 
   void* ctrl_v = nullptr;
   if ((rc = ensure(&ws, W::CTRL, sizeof(DevCtrl), &ctrl_v))) return rc;
   DevCtrl* ctrl = static_cast<DevCtrl*>(ctrl_v);
-  void* blockcnt = nullptr;
-  int32_t K = 0;
-  if ((rc = validate_and_count(SURV_COX, layout, prec, n, p, stg, ctrl, &ws, s, &blockcnt, &K, &launches))) return rc;
-  void *gend, *dk, *ck, *lam, *r, *g;
+  void* cnt = nullptr;
+  int32_t K = 0, events = 0;
+  if ((rc = validate_and_count(SURV_COX, layout, prec, n, p, stg, ctrl, &ws, s, &cnt, &K, &events, &launches))) return rc;
+  if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
+  void *gend, *dk, *lam, *r, *g;
   if ((rc = ensure(&ws, W::GEND, 4 * (size_t)K, &gend))) return rc;
   if ((rc = ensure(&ws, W::DK, 4 * (size_t)K, &dk))) return rc;
-  if ((rc = ensure(&ws, W::CK, 4 * (size_t)K, &ck))) return rc;
   if ((rc = ensure(&ws, W::LM_LAM, 8 * (size_t)K, &lam))) return rc;
   if ((rc = ensure(&ws, W::LM_R, 8 * (size_t)n, &r))) return rc;
   if ((rc = ensure(&ws, W::LM_G, 8 * (size_t)(p + 1), &g))) return rc;
-  CUDA_TRY(survgpu::prep_write_ends(stg.time, n, static_cast<const int32_t*>(blockcnt), static_cast<int32_t*>(gend), s));
-  CUDA_TRY(survgpu::prep_group_stats(static_cast<int32_t*>(gend), K, stg.status, n, static_cast<int32_t*>(dk),
-                                     static_cast<int32_t*>(ck), &ctrl->total_events, s));
+  CUDA_TRY(survgpu::prep_group_write(stg.time, stg.status, n, cnt, K, static_cast<int32_t*>(gend),
+                                     static_cast<int32_t*>(dk), nullptr, 0, 32, nullptr, s));
   double* gd = static_cast<double*>(g);
   CUDA_TRY(survgpu::lambda_max_device(layout, prec, stg.colptr, stg.rowidx, stg.vals, stg.ld, n, p, stg.status,
                                       static_cast<const int32_t*>(gend), static_cast<const int32_t*>(dk), K, pf_d,
                                       static_cast<double*>(lam), static_cast<double*>(r), gd, gd + p, s));
-  DevCtrl hc;
   double v = 0.0;
-  CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaMemcpyAsync(&v, gd + p, sizeof(double), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  if (hc.total_events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   *out = v;
   return SURV_OK;
 }
@@ -787,9 +779,9 @@ int cv_impl(const surv_data* d, const int8_t* fold_id, int nfolds, const double*
   void* ctrl_v = nullptr;
   if ((rc = ensure(ws, W::CTRL, sizeof(DevCtrl), &ctrl_v))) return rc;
   DevCtrl* ctrl = static_cast<DevCtrl*>(ctrl_v);
-  void* blockcnt = nullptr;
-  int32_t K = 0;
-  if ((rc = validate_and_count(SURV_COX, layout, prec, n, p, stg, ctrl, ws, s, &blockcnt, &K, &launches))) return rc;
+  void* cnt = nullptr;
+  int32_t K = 0, events = 0;
+  if ((rc = validate_and_count(SURV_COX, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches))) return rc;
   const void* fold_v = nullptr;
   if ((rc = device_view(ws, W::CV_FOLD, fold_id, (size_t)n, s, &fold_v))) return rc;
   const int8_t* fold_d = static_cast<const int8_t*>(fold_v);
@@ -801,13 +793,12 @@ int cv_impl(const surv_data* d, const int8_t* fold_id, int nfolds, const double*
   // batches would be as many as the slowest fit needs (measured slower:
   // 180 against 237 fits/s at N = 10^6, 200 fits)
   const int RC = M, NPART = 3;
-  void *gend, *dk, *ck, *wk0, *woff = nullptr, *dkf, *dtxf, *cvc_v;
+  void *gend, *dk, *wk0, *woff = nullptr, *dkf, *dtxf, *cvc_v;
   void *e, *eta, *rec, *wt, *agg, *part, *gctl, *beta, *width, *pen, *out, *fits, *den, *held, *mean;
   const size_t rec_f = pad((size_t)K * RC, 8), wt_f = pad((size_t)RC * nwarps_alloc, 8);
   const size_t agg_f = pad((size_t)survgpu::kRep * RC * Galloc, 8), part_f = pad((size_t)NPART * Galloc, 8);
   if ((rc = ensure(ws, W::GEND, 4 * (size_t)K, &gend))) return rc;
   if ((rc = ensure(ws, W::DK, 4 * (size_t)K, &dk))) return rc;
-  if ((rc = ensure(ws, W::CK, 4 * (size_t)K, &ck))) return rc;
   if ((rc = ensure(ws, W::WK0, 4 * (size_t)(nwarps_alloc + 1), &wk0))) return rc;
   if (layout == SURV_CSC && (rc = ensure(ws, W::WOFF, 4 * (size_t)p * (nwarps_alloc + 1), &woff))) return rc;
   if ((rc = ensure(ws, W::CV_DK, 4 * (size_t)nfolds * K, &dkf))) return rc;
@@ -832,25 +823,22 @@ int cv_impl(const surv_data* d, const int8_t* fold_id, int nfolds, const double*
 
   CUDA_TRY(cudaMemsetAsync(cvc, 0, sizeof(CvCtrl), s));
   CUDA_TRY(survgpu::cv_check_folds(fold_d, n, nfolds, &cvc->perr, s));
-  CUDA_TRY(survgpu::prep_write_ends(stg.time, n, static_cast<const int32_t*>(blockcnt), static_cast<int32_t*>(gend), s));
-  CUDA_TRY(survgpu::prep_group_stats(static_cast<int32_t*>(gend), K, stg.status, n, static_cast<int32_t*>(dk),
-                                     static_cast<int32_t*>(ck), &ctrl->total_events, s));
+  CUDA_TRY(survgpu::prep_group_write(stg.time, stg.status, n, cnt, K, static_cast<int32_t*>(gend),
+                                     static_cast<int32_t*>(dk), nullptr, 0, 32, nullptr, s));
   CUDA_TRY(survgpu::cv_fold_stats(static_cast<int32_t*>(gend), K, stg.status, fold_d, nfolds,
                                   static_cast<int32_t*>(dkf), cvc->events, s));
   CUDA_TRY(survgpu::cv_dtx(layout == SURV_CSC ? 0 : 1, prec, stg.colptr, stg.rowidx, stg.vals, stg.ld, n, p,
                            stg.status, fold_d, nfolds, static_cast<double*>(dtxf), s));
-  launches += 5;
+  launches += 4;
   std::vector<double> pen_h((size_t)F * p);
   for (int f = 0; f < F; ++f)
     for (int64_t j = 0; j < p; ++j) pen_h[(size_t)f * p + j] = lam_h[f / nfolds] * pf_h[j];
   CUDA_TRY(cudaMemcpyAsync(pen, pen_h.data(), 8 * pen_h.size(), cudaMemcpyHostToDevice, s));
   CvCtrl hcv;
-  DevCtrl hc;
   CUDA_TRY(cudaMemcpyAsync(&hcv, cvc, sizeof(CvCtrl), cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   if (hcv.perr & survgpu::PREP_FOLD) { set_error("fold_id outside [0, %d)", nfolds); return SURV_E_INVALID; }
-  if (hc.total_events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
+  if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   for (int k = 0; k < nfolds; ++k)
     if (hcv.events[k] <= 0) { set_error("no events outside fold %d", k); return SURV_E_NO_EVENTS; }
 
@@ -1122,15 +1110,14 @@ int surv_groups(const int32_t* time, const int8_t* status, int64_t n, int64_t ma
   int rc;
   if ((rc = device_view(&ws, W::TIME, time, 4 * (size_t)n, s, &time_d))) return rc;
   if ((rc = device_view(&ws, W::STATUS, status, (size_t)n, s, &status_d))) return rc;
-  void *ctrl_v, *blockcnt;
+  void *ctrl_v, *cnt;
   if ((rc = ensure(&ws, W::CTRL, sizeof(DevCtrl), &ctrl_v))) return rc;
   DevCtrl* ctrl = static_cast<DevCtrl*>(ctrl_v);
   CUDA_TRY(cudaMemsetAsync(ctrl, 0, sizeof(DevCtrl), s));
   const int32_t* tp = static_cast<const int32_t*>(time_d);
   const int8_t* sp = static_cast<const int8_t*>(status_d);
-  CUDA_TRY(survgpu::prep_check_times(tp, sp, n, 1, &ctrl->perr, s));
-  if ((rc = ensure(&ws, W::BLOCKCNT, 4 * (size_t)survgpu::prep_end_blocks(n), &blockcnt))) return rc;
-  CUDA_TRY(survgpu::prep_count_ends(tp, n, static_cast<int32_t*>(blockcnt), &ctrl->K, s));
+  if ((rc = ensure(&ws, W::BLOCKCNT, survgpu::prep_count_bytes(n), &cnt))) return rc;
+  CUDA_TRY(survgpu::prep_group_count(tp, sp, n, 1, cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket, s));
   DevCtrl hc;
   CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
@@ -1144,9 +1131,8 @@ int surv_groups(const int32_t* time, const int8_t* status, int64_t n, int64_t ma
   if ((rc = ensure(&ws, W::DK, 4 * (size_t)K, &dk))) return rc;
   if ((rc = ensure(&ws, W::CK, 4 * (size_t)K, &ck))) return rc;
   if ((rc = ensure(&ws, W::GK, 8 * (size_t)K, &Gk))) return rc;
-  CUDA_TRY(survgpu::prep_write_ends(tp, n, static_cast<const int32_t*>(blockcnt), static_cast<int32_t*>(gend), s));
-  CUDA_TRY(survgpu::prep_group_stats(static_cast<int32_t*>(gend), K, sp, n, static_cast<int32_t*>(dk),
-                                     static_cast<int32_t*>(ck), &ctrl->total_events, s));
+  CUDA_TRY(survgpu::prep_group_write(tp, sp, n, cnt, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
+                                     static_cast<int32_t*>(ck), 0, 32, nullptr, s));
   CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), nullptr, s));
   if (gend_out) CUDA_TRY(cudaMemcpyAsync(gend_out, gend, 4 * (size_t)K, cudaMemcpyDefault, s));
   if (dk_out) CUDA_TRY(cudaMemcpyAsync(dk_out, dk, 4 * (size_t)K, cudaMemcpyDefault, s));

@@ -234,21 +234,22 @@ cudaError_t run_sn_graph(const CcdParams& P, const SnParams& S, cudaStream_t s, 
 cudaError_t time_one_sweep(int model, int layout, int prec, const CcdParams& P, cudaStream_t s, float* ms);
 
 // ---- prep kernels (prep.cu) --------------------------------------------
-cudaError_t prep_check_times(const int32_t* time, const int8_t* status, int64_t n, int model,
-                             unsigned* perr, cudaStream_t s);
 cudaError_t prep_check_csc(const int64_t* col_ptr, const int32_t* row_idx, const void* values, int prec,
                            int64_t p, int64_t n, unsigned* perr, cudaStream_t s);
 cudaError_t prep_check_dense(const void* X, int prec, int64_t ld, int64_t n, int64_t p, unsigned* perr,
                              cudaStream_t s);
 cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr, cudaStream_t s);
-// Count tie groups: writes per-block counts into blockcnt [nblocks] and K into *K_dev.
-int64_t prep_end_blocks(int64_t n);
-cudaError_t prep_count_ends(const int32_t* time, int64_t n, int32_t* blockcnt, int32_t* K_dev, cudaStream_t s);
-cudaError_t prep_write_ends(const int32_t* time, int64_t n, const int32_t* blockoff, int32_t* gend, cudaStream_t s);
-// dk, ck [K] (zeroed here): events and censored subjects per group, n subjects;
-// *total_events (zeroed by the caller) += all events
-cudaError_t prep_group_stats(const int32_t* gend, int32_t K, const int8_t* status, int64_t n, int32_t* dk,
-                             int32_t* ck, int32_t* total_events, cudaStream_t s);
+// Tie groups.  prep_group_count checks times and status codes (*perr) and
+// writes *K, *total_events (subjects with status 1) and its block counts
+// into cnt (prep_count_bytes(n) bytes); *ticket is a zeroed word.
+// prep_group_write then fills gend, dk and ck (ck may be null) and, with
+// wk0, the first group of each warp's rows.
+size_t prep_count_bytes(int64_t n);
+cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
+                             unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s);
+cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
+                             int32_t* gend, int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rows_per_warp,
+                             int32_t* wk0, cudaStream_t s);
 cudaError_t prep_km(const int32_t* gend, const int32_t* ck, int32_t K, double* Gk, float2* Gkff, cudaStream_t s);
 cudaError_t prep_w2(const int32_t* gend, int32_t K, const int8_t* status, const double* Gk, void* w2, int prec,
                     cudaStream_t s);

@@ -499,7 +499,7 @@ struct NllCtrl {
   unsigned perr;
   int32_t K;
   int32_t total_events;
-  int32_t pad;
+  unsigned ticket;
 };
 
 #define NLL_TRY(expr)        \
@@ -536,16 +536,16 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   using W = surv_workspace;
-  void *ctrl_v, *blk, *gend, *dk, *ck, *wk0, *Y, *Bcat, *rec, *wt, *den;
+  void *ctrl_v, *blk, *gend, *dk, *wk0, *Y, *Bcat, *rec, *wt, *den;
   NLL_TRY(ws_ensure(ws, W::NLL_CTRL, sizeof(NllCtrl), &ctrl_v));
   NllCtrl* ctrl = static_cast<NllCtrl*>(ctrl_v);
   NLL_TRY(cuda_err(cudaMemsetAsync(ctrl, 0, sizeof(NllCtrl), s), "memset"));
   const int32_t* time = static_cast<const int32_t*>(d->time);
   const int8_t* status = static_cast<const int8_t*>(d->status);
-  NLL_TRY(cuda_err(prep_check_times(time, status, n, 0, &ctrl->perr, s), "check times"));
-  const int64_t nb = prep_end_blocks(n);
-  NLL_TRY(ws_ensure(ws, W::NLL_BLK, 4 * (size_t)nb, &blk));
-  NLL_TRY(cuda_err(prep_count_ends(time, n, static_cast<int32_t*>(blk), &ctrl->K, s), "count ends"));
+  NLL_TRY(ws_ensure(ws, W::NLL_BLK, prep_count_bytes(n), &blk));
+  NLL_TRY(cuda_err(prep_group_count(time, status, n, 0, blk, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket,
+                                    s),
+                   "count groups"));
   NllCtrl hc;
   unsigned prev_err = 0;
   NLL_TRY(cuda_err(cudaMemcpyAsync(&hc, ctrl, sizeof(hc), cudaMemcpyDeviceToHost, s), "copy"));
@@ -565,12 +565,6 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   const int K = hc.K;
   NLL_TRY(ws_ensure(ws, W::NLL_GEND, 4 * (size_t)K, &gend));
   NLL_TRY(ws_ensure(ws, W::NLL_DK, 4 * (size_t)K, &dk));
-  NLL_TRY(ws_ensure(ws, W::GK, 4 * (size_t)K, &ck));
-  NLL_TRY(cuda_err(prep_write_ends(time, n, static_cast<const int32_t*>(blk), static_cast<int32_t*>(gend), s),
-                   "write ends"));
-  NLL_TRY(cuda_err(prep_group_stats(static_cast<int32_t*>(gend), K, status, n, static_cast<int32_t*>(dk),
-                                    static_cast<int32_t*>(ck), &ctrl->total_events, s),
-                   "group stats"));
   // row partition of the scan kernels: two CTAs of 16 warps per SM
   int dev = 0, sms = 0;
   NLL_TRY(cuda_err(cudaGetDevice(&dev), "device"));
@@ -580,8 +574,9 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   const int64_t wpw = (nwords + nwarps - 1) / nwarps;
   const int64_t rpw = wpw * 32;
   NLL_TRY(ws_ensure(ws, W::NLL_WK0, 4 * (size_t)(nwarps + 1), &wk0));
-  NLL_TRY(cuda_err(prep_warp_groups(static_cast<int32_t*>(gend), K, n, nwarps, rpw, static_cast<int32_t*>(wk0), s),
-                   "warp groups"));
+  NLL_TRY(cuda_err(prep_group_write(time, status, n, blk, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
+                                    nullptr, nwarps, rpw, static_cast<int32_t*>(wk0), s),
+                   "write groups"));
   // eta = X B_hi + X B_lo on the tensor cores (nll_tc.cu).  Bcat^T holds the
   // split in 2 Cp rows, Cp = C rounded up to 16 (at least 32); X and Bcat^T
   // rows have a pitch of ld = p rounded up to 8 elements (16 bytes)

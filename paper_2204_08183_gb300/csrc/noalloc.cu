@@ -34,7 +34,8 @@ struct Ctrl {
   int32_t K;
   int32_t total_events;
   unsigned counters[2];
-  unsigned pad[2];
+  unsigned ticket;
+  unsigned pad;
   double out[survgpu::OUT_COUNT];
   unsigned long long timing[survgpu::PH_COUNT];
 };
@@ -193,10 +194,10 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   for (int64_t q = 0; q < p; ++q)
     if (!std::isfinite(beta_h[q])) { snprintf(g_err, sizeof(g_err), "non-finite beta"); return SURV_E_NONFINITE; }
 
-  void *ctrl_v, *blockcnt, *e, *eta, *w2 = nullptr, *wk0, *woff = nullptr, *dTx, *beta_d, *width, *pen, *slots;
+  void *ctrl_v, *cnt, *e, *eta, *w2 = nullptr, *wk0, *woff = nullptr, *dTx, *beta_d, *width, *pen, *slots;
   TAKE(ctrl_v, sizeof(Ctrl));
   Ctrl* ctrl = static_cast<Ctrl*>(ctrl_v);
-  TAKE(blockcnt, 4 * (size_t)survgpu::prep_end_blocks(n));
+  TAKE(cnt, survgpu::prep_count_bytes(n));
   TAKE(e, tsz * (size_t)n);
   TAKE(eta, 8 * (size_t)n);
   if (model == SURV_FG) TAKE(w2, tsz * (size_t)n);
@@ -213,18 +214,17 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   TRY(cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), s));
   const int32_t* tp = static_cast<const int32_t*>(static_cast<const void*>(d->time));
   const int8_t* sp = d->status;
-  TRY(survgpu::prep_check_times(tp, sp, n, model, &ctrl->perr, s));
+  TRY(survgpu::prep_group_count(tp, sp, n, model, cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket, s));
   if (csc) {
     TRY(survgpu::prep_check_csc(d->col_ptr, d->row_idx, d->values, prec, p, n, &ctrl->perr, s));
   } else {
     TRY(survgpu::prep_check_dense(d->values, prec, n, n, p, &ctrl->perr, s));
   }
-  TRY(survgpu::prep_count_ends(tp, n, static_cast<int32_t*>(blockcnt), &ctrl->K, s));
   Ctrl hc;
   TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
   TRY(cudaStreamSynchronize(s));
   if ((rc = map_prep(hc.perr))) return rc;
-  const int32_t K = hc.K;
+  const int32_t K = hc.K, events = hc.total_events;
 
   void *gend, *dk, *ck, *Gk, *Gkff, *rec;
   TAKE(gend, 4 * (size_t)K);
@@ -234,9 +234,9 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   TAKE(Gkff, 8 * (size_t)K);
   TAKE(rec, 8 * (size_t)K * M);
 
-  TRY(survgpu::prep_write_ends(tp, n, static_cast<const int32_t*>(blockcnt), static_cast<int32_t*>(gend), s));
-  TRY(survgpu::prep_group_stats(static_cast<int32_t*>(gend), K, sp, n, static_cast<int32_t*>(dk),
-                                static_cast<int32_t*>(ck), &ctrl->total_events, s));
+  if (events <= 0) { snprintf(g_err, sizeof(g_err), "no events"); return SURV_E_NO_EVENTS; }
+  TRY(survgpu::prep_group_write(tp, sp, n, cnt, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
+                                static_cast<int32_t*>(ck), nwarps, rows_per_warp, static_cast<int32_t*>(wk0), s));
   if (model == SURV_FG) {
     TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk),
                          static_cast<float2*>(Gkff), s));
@@ -248,7 +248,6 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   } else {
     TRY(survgpu::prep_dtx_dense(d->values, prec, n, n, sp, p, static_cast<double*>(dTx), s));
   }
-  TRY(survgpu::prep_warp_groups(static_cast<int32_t*>(gend), K, n, nwarps, rows_per_warp, static_cast<int32_t*>(wk0), s));
   TRY(cudaMemcpyAsync(beta_d, beta_h, 8 * (size_t)p, cudaMemcpyHostToDevice, s));
   TRY(survgpu::prep_fill_f64(static_cast<double*>(width), 1.0, p, s));
   TRY(survgpu::prep_fill_f64(static_cast<double*>(pen), 0.0, p, s));
@@ -269,9 +268,6 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
     TRY(survgpu::prep_eta_exp(prec, n, eta, e, s));
   }
   TRY(cudaMemsetAsync(slots, 0, 2 * slot_bytes, s));
-  TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
-  TRY(cudaStreamSynchronize(s));
-  if (hc.total_events <= 0) { snprintf(g_err, sizeof(g_err), "no events"); return SURV_E_NO_EVENTS; }
 
   survgpu::CcdParams P;
   std::memset(&P, 0, sizeof(P));
