@@ -35,3 +35,20 @@ def test_groups_at_block_edges(lib, n, n_times, offset):
     else:   # the chunked product: below (2 L + 12 + K) u relative of the sequential one
         K = len(ref)
         np.testing.assert_allclose(Gk, G, rtol=(2 * -(-K // 1024) + 12 + K) * 2.0 ** -53)
+
+
+# tiles of the sort hold 4096 elements; the spans need 0, 1, 8, 9, 17 and 32
+# key bits: 0 to 4 passes of equal digits
+@pytest.mark.parametrize("span", [1, 2, 256, 257, 100_000, 2**32])
+@pytest.mark.parametrize("n", [1, 33, 4095, 4096, 4097, 70_001])
+def test_sort_at_tile_edges_and_key_spans(lib, n, span):
+    import torch
+    rng = np.random.default_rng(n + span)
+    lo = -(span // 2)
+    time = rng.integers(lo, lo + span, n).astype(np.int32)
+    time[0], time[-1] = lo, lo + span - 1
+    ref = oracle.sort_desc(time).astype(np.int32)
+    t = torch.from_numpy(time).cuda()
+    np.testing.assert_array_equal(binding.surv_sort_desc(t).cpu().numpy(), ref)
+    binding.surv_sort_desc(t, perm=t)   # the order written over the times
+    np.testing.assert_array_equal(t.cpu().numpy(), ref)
