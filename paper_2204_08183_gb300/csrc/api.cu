@@ -253,17 +253,27 @@ int stage_data(const surv_data* d, int prec, surv_workspace* ws, cudaStream_t s,
 // again.
 int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, Staged& st, DevCtrl* ctrl,
                        surv_workspace* ws, cudaStream_t s, void** cnt, int32_t* K, int32_t* events,
-                       int64_t* launches) {
+                       int64_t* launches, survgpu::PrepColumns* cols = nullptr, int* cols_nb = nullptr) {
   CUDA_TRY(cudaMemsetAsync(ctrl, 0, sizeof(DevCtrl), s));
   int rc;
   if ((rc = ensure(ws, surv_workspace::BLOCKCNT, survgpu::prep_count_bytes(n), cnt))) return rc;
   CUDA_TRY(survgpu::prep_group_count(st.time, st.status, n, model, *cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events,
                                      &ctrl->ticket, s));
   ++*launches;
+  int64_t longest = n;
+  if (layout == SURV_CSC) {
+    longest = 0;
+    for (int64_t j = 0; j < p; ++j) longest = std::max(longest, st.colptr_h[j + 1] - st.colptr_h[j]);
+  }
+  const int nb = survgpu::prep_col_blocks(longest, p);
+  if (cols) {
+    if ((rc = ensure(ws, surv_workspace::DTX_PART, 8 * (size_t)p * nb, &cols->part))) return rc;
+    *cols_nb = nb;
+  }
   if (layout == SURV_CSC)
-    CUDA_TRY(survgpu::prep_check_csc(st.colptr, st.rowidx, st.vals, prec, p, n, &ctrl->perr, s));
+    CUDA_TRY(survgpu::prep_check_csc(st.colptr, st.rowidx, st.vals, prec, p, n, nb, cols, &ctrl->perr, s));
   else
-    CUDA_TRY(survgpu::prep_check_dense(st.vals, prec, st.ld, n, p, &ctrl->perr, s));
+    CUDA_TRY(survgpu::prep_check_dense(st.vals, prec, st.ld, n, p, nb, cols, &ctrl->perr, s));
   ++*launches;
   DevCtrl hc;
   CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
@@ -366,13 +376,25 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   const int8_t* status_p = stg.status;
   void* cnt = nullptr;
   int32_t K = 0, events = 0;
-  if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches))) return rc;
+  survgpu::PrepColumns cols;
+  int cols_nb = 0;
+  void *woff = nullptr, *wk0 = nullptr;
+  cols.status = status_p;
+  cols.nwarps = nwarps;
+  cols.rows_per_warp = rows_per_warp;
+  if (layout == SURV_CSC) {
+    if ((rc = ensure(ws, W::WOFF, 4 * (size_t)p * (nwarps + 1), &woff))) return rc;
+    cols.woff = static_cast<int32_t*>(woff);
+  }
+  if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches, &cols,
+                               &cols_nb)))
+    return rc;
   if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   const void* vals_d = stg.vals;  // null for indicator CSC data (all values 1)
   DevCtrl hc;
 
   // ---------------------------------------------------------- tables
-  void *gend, *dk, *ck, *Gk, *rec, *e, *eta, *w2 = nullptr, *wk0, *woff = nullptr, *dTx, *beta, *width, *pen, *slots;
+  void *gend, *dk, *ck, *Gk, *rec, *e, *eta, *w2 = nullptr, *dTx, *beta, *width, *pen, *slots;
   constexpr size_t accsz = 8;  // an accumulator: ff (2 floats) or double
   if ((rc = ensure(ws, W::GEND, 4 * (size_t)K, &gend))) return rc;
   if ((rc = ensure(ws, W::DK, 4 * (size_t)K, &dk))) return rc;
@@ -397,7 +419,6 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   if ((rc = ensure(ws, W::ETA, 8 * (size_t)n, &eta))) return rc;
   if (model == SURV_FG && (rc = ensure(ws, W::W2, tsz * (size_t)n, &w2))) return rc;
   if ((rc = ensure(ws, W::WK0, 4 * (size_t)(nwarps + 1), &wk0))) return rc;
-  if (layout == SURV_CSC && (rc = ensure(ws, W::WOFF, 4 * (size_t)p * (nwarps + 1), &woff))) return rc;
   if ((rc = ensure(ws, W::DTX, 8 * (size_t)p, &dTx))) return rc;
   if ((rc = ensure(ws, W::BETA, 8 * (size_t)p, &beta))) return rc;
   if ((rc = ensure(ws, W::WIDTH, 8 * (size_t)p, &width))) return rc;
@@ -443,25 +464,17 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
                                      static_cast<int32_t*>(wk0), s));
   ++launches;
   if (model == SURV_FG) {
-    CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk),
-                              static_cast<float2*>(Gkff), s));
-    CUDA_TRY(survgpu::prep_w2(static_cast<int32_t*>(gend), K, status_p, static_cast<double*>(Gk), w2, prec, s));
-    launches += 2;
+    CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), s));
+    // the records are not in use yet: scratch for 1 / G
+    CUDA_TRY(survgpu::prep_weights(time_p, status_p, n, cnt, K, static_cast<double*>(Gk), static_cast<float2*>(Gkff),
+                                   rec, w2, prec, s));
+    launches += 4;
   }
-  if (layout == SURV_CSC) {
-    CUDA_TRY(survgpu::prep_dtx_csc(static_cast<const int64_t*>(colptr_d), static_cast<const int32_t*>(rowidx_d),
-                                   vals_d, prec, status_p, p, static_cast<double*>(dTx), s));
-    CUDA_TRY(survgpu::prep_warp_offsets(static_cast<const int64_t*>(colptr_d), static_cast<const int32_t*>(rowidx_d),
-                                        p, n, nwarps, rows_per_warp, static_cast<int32_t*>(woff), s));
-    launches += 2;
-  } else {
-    CUDA_TRY(survgpu::prep_dtx_dense(vals_d, prec, ld, n, status_p, p, static_cast<double*>(dTx), s));
-    ++launches;
-  }
+  CUDA_TRY(survgpu::prep_coord_init(cols.part, prec, cols_nb, p, static_cast<double*>(dTx),
+                                    static_cast<double*>(width), s));
+  ++launches;
   CUDA_TRY(cudaMemcpyAsync(beta, beta_h.data(), 8 * (size_t)p, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(pen, pen_h.data(), 8 * (size_t)p, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(survgpu::prep_fill_f64(static_cast<double*>(width), 1.0, p, s));
-  ++launches;
   bool any_beta = false;
   for (double b : beta_h) any_beta |= (b != 0.0);
   if (!any_beta) {
@@ -1133,7 +1146,7 @@ int surv_groups(const int32_t* time, const int8_t* status, int64_t n, int64_t ma
   if ((rc = ensure(&ws, W::GK, 8 * (size_t)K, &Gk))) return rc;
   CUDA_TRY(survgpu::prep_group_write(tp, sp, n, cnt, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
                                      static_cast<int32_t*>(ck), 0, 32, nullptr, s));
-  CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), nullptr, s));
+  CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), s));
   if (gend_out) CUDA_TRY(cudaMemcpyAsync(gend_out, gend, 4 * (size_t)K, cudaMemcpyDefault, s));
   if (dk_out) CUDA_TRY(cudaMemcpyAsync(dk_out, dk, 4 * (size_t)K, cudaMemcpyDefault, s));
   if (Gk_out) CUDA_TRY(cudaMemcpyAsync(Gk_out, Gk, 8 * (size_t)K, cudaMemcpyDefault, s));

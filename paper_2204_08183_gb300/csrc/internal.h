@@ -234,10 +234,24 @@ cudaError_t run_sn_graph(const CcdParams& P, const SnParams& S, cudaStream_t s, 
 cudaError_t time_one_sweep(int model, int layout, int prec, const CcdParams& P, cudaStream_t s, float* ms);
 
 // ---- prep kernels (prep.cu) --------------------------------------------
-cudaError_t prep_check_csc(const int64_t* col_ptr, const int32_t* row_idx, const void* values, int prec,
-                           int64_t p, int64_t n, unsigned* perr, cudaStream_t s);
-cudaError_t prep_check_dense(const void* X, int prec, int64_t ld, int64_t n, int64_t p, unsigned* perr,
-                             cudaStream_t s);
+// One pass over X: checks (*perr) and, with `out`, the partial sums of
+// delta^T X_j (part: p x nb accumulators of 8 bytes, nb = prep_col_blocks of
+// the longest column) and, for CSC, the offsets of each warp's first row.
+struct PrepColumns {
+  const int8_t* status = nullptr;
+  void* part = nullptr;
+  int32_t nwarps = 0;
+  int64_t rows_per_warp = 0;   // a multiple of 32
+  int32_t* woff = nullptr;     // [p][nwarps + 1] (CSC)
+};
+int prep_col_blocks(int64_t longest, int64_t p);
+cudaError_t prep_check_csc(const int64_t* col_ptr, const int32_t* row_idx, const void* values, int prec, int64_t p,
+                           int64_t n, int nb, const PrepColumns* out, unsigned* perr, cudaStream_t s);
+cudaError_t prep_check_dense(const void* X, int prec, int64_t ld, int64_t n, int64_t p, int nb,
+                             const PrepColumns* out, unsigned* perr, cudaStream_t s);
+// delta^T X_j from the partial sums; trust-region widths 1.
+cudaError_t prep_coord_init(const void* part, int prec, int nb, int64_t p, double* dTx, double* width,
+                            cudaStream_t s);
 cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr, cudaStream_t s);
 // Tie groups.  prep_group_count checks times and status codes (*perr) and
 // writes *K, *total_events (subjects with status 1) and its block counts
@@ -250,13 +264,11 @@ cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t 
 cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
                              int32_t* gend, int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rows_per_warp,
                              int32_t* wk0, cudaStream_t s);
-cudaError_t prep_km(const int32_t* gend, const int32_t* ck, int32_t K, double* Gk, float2* Gkff, cudaStream_t s);
-cudaError_t prep_w2(const int32_t* gend, int32_t K, const int8_t* status, const double* Gk, void* w2, int prec,
-                    cudaStream_t s);
-cudaError_t prep_dtx_csc(const int64_t* col_ptr, const int32_t* row_idx, const void* values, int prec,
-                         const int8_t* status, int64_t p, double* dTx, cudaStream_t s);
-cudaError_t prep_dtx_dense(const void* X, int prec, int64_t ld, int64_t n, const int8_t* status, int64_t p,
-                           double* dTx, cudaStream_t s);
+// G(t_k); then its float-float form, 1 / G(t_k) in the working precision (inv:
+// K values of scratch) and W (cnt: the counts of prep_group_count).
+cudaError_t prep_km(const int32_t* gend, const int32_t* ck, int32_t K, double* Gk, cudaStream_t s);
+cudaError_t prep_weights(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
+                         const double* Gk, float2* Gkff, void* inv, void* w2, int prec, cudaStream_t s);
 cudaError_t prep_warp_groups(const int32_t* gend, int32_t K, int64_t n, int32_t nwarps, int64_t rows_per_warp,
                              int32_t* wk0, cudaStream_t s);
 cudaError_t prep_warp_offsets(const int64_t* col_ptr, const int32_t* row_idx, int64_t p, int64_t n,

@@ -7,6 +7,7 @@
 // life of the process.  Host code must not use the symbol `g_scratch` as an
 // address (it names a host-side shadow); the device address comes from
 // cudaGetSymbolAddress, once per device, cached below.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -215,10 +216,24 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   const int32_t* tp = static_cast<const int32_t*>(static_cast<const void*>(d->time));
   const int8_t* sp = d->status;
   TRY(survgpu::prep_group_count(tp, sp, n, model, cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket, s));
+  // partial sums of delta^T X_j: in the exchange slots, which are zeroed
+  // after they have been summed
+  survgpu::PrepColumns cols;
+  cols.status = sp;
+  cols.part = slots;
+  cols.nwarps = nwarps;
+  cols.rows_per_warp = rows_per_warp;
+  cols.woff = static_cast<int32_t*>(woff);
+  int64_t longest = csc ? 0 : n;
+  for (int64_t q = 0; csc && q < p; ++q) longest = std::max(longest, colptr_h[q + 1] - colptr_h[q]);
+  static_assert(2 * 4 * survgpu::kSlotWords * 2 >= 8 * 32, "at least 32 partial sums a CTA");
+  const int64_t room = (int64_t)(2 * slot_bytes / 8) / p;
+  if (room < 1) { snprintf(g_err, sizeof(g_err), "too many covariates for this device's grid"); return SURV_E_INVALID; }
+  const int nb = (int)std::min<int64_t>(survgpu::prep_col_blocks(longest, p), room);
   if (csc) {
-    TRY(survgpu::prep_check_csc(d->col_ptr, d->row_idx, d->values, prec, p, n, &ctrl->perr, s));
+    TRY(survgpu::prep_check_csc(d->col_ptr, d->row_idx, d->values, prec, p, n, nb, &cols, &ctrl->perr, s));
   } else {
-    TRY(survgpu::prep_check_dense(d->values, prec, n, n, p, &ctrl->perr, s));
+    TRY(survgpu::prep_check_dense(d->values, prec, n, n, p, nb, &cols, &ctrl->perr, s));
   }
   Ctrl hc;
   TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
@@ -238,18 +253,13 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   TRY(survgpu::prep_group_write(tp, sp, n, cnt, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
                                 static_cast<int32_t*>(ck), nwarps, rows_per_warp, static_cast<int32_t*>(wk0), s));
   if (model == SURV_FG) {
-    TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk),
-                         static_cast<float2*>(Gkff), s));
-    TRY(survgpu::prep_w2(static_cast<int32_t*>(gend), K, sp, static_cast<double*>(Gk), w2, prec, s));
+    TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), s));
+    // the records are not in use yet: scratch for 1 / G
+    TRY(survgpu::prep_weights(tp, sp, n, cnt, K, static_cast<double*>(Gk), static_cast<float2*>(Gkff), rec, w2, prec,
+                              s));
   }
-  if (csc) {
-    TRY(survgpu::prep_dtx_csc(d->col_ptr, d->row_idx, d->values, prec, sp, p, static_cast<double*>(dTx), s));
-    TRY(survgpu::prep_warp_offsets(d->col_ptr, d->row_idx, p, n, nwarps, rows_per_warp, static_cast<int32_t*>(woff), s));
-  } else {
-    TRY(survgpu::prep_dtx_dense(d->values, prec, n, n, sp, p, static_cast<double*>(dTx), s));
-  }
+  TRY(survgpu::prep_coord_init(slots, prec, nb, p, static_cast<double*>(dTx), static_cast<double*>(width), s));
   TRY(cudaMemcpyAsync(beta_d, beta_h, 8 * (size_t)p, cudaMemcpyHostToDevice, s));
-  TRY(survgpu::prep_fill_f64(static_cast<double*>(width), 1.0, p, s));
   TRY(survgpu::prep_fill_f64(static_cast<double*>(pen), 0.0, p, s));
   bool any_beta = false;
   for (int64_t q = 0; q < p; ++q) any_beta |= beta_h[q] != 0.0;

@@ -8,6 +8,7 @@
 // Integer work (ends, counts) is exact; G(t_k) is a sequential FP64 product
 // from the smallest time upward in a single thread, so its rounding follows
 // one fixed order.
+#include <algorithm>
 #include <climits>
 #include <cuda_bf16.h>
 #include <cmath>
@@ -28,33 +29,186 @@ inline unsigned grid_for(int64_t count, int threads, unsigned cap = 65535u * 32u
   return (unsigned)g;
 }
 
-template <typename T>
-__global__ void k_check_csc(const int64_t* col_ptr, const int32_t* row_idx, const T* values, int64_t p,
-                            int64_t n, unsigned* perr) {
+// Blocks of a column of `len` stored values: contiguous chunks of at least
+// kColChunk, at most kMaxColBlocks (a partial sum each).
+constexpr int kColThreads = 256;
+constexpr int kColChunk = 4096;
+constexpr int kMaxColBlocks = 512;
+
+// Partial sum of one block in a fixed order (thread 0 stores it).
+template <typename A>
+__device__ __forceinline__ void block_partial(A v, A* dst) {
+  __shared__ A s_w[kColThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  v = warp_sum(v);
+  if (lane == 0) s_w[w] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    A a = s_w[0];
+    for (int q = 1; q < kColThreads / 32; ++q) a = acc_add(a, s_w[q]);
+    *dst = a;
+  }
+}
+
+// One pass over the stored entries of CSC column blockIdx.y: row indices in
+// range and increasing, values finite and (flag) all 1.  With FULL it also
+// leaves the block's share of delta^T X_j in part[j][blockIdx.x] and the
+// column's offsets at the warps' first rows in woff[j][.]: entry i is the
+// first at or after the first row of every warp after its predecessor's
+// warp, up to its own.  Three kernels did this before, two of them reading
+// the row indices again, one with a block per column and one with a binary
+// search per (column, warp): 248 us at 5 x 10^7 entries of 100 columns,
+// against 118 us for the one pass over 400 MB.
+template <typename T, bool FULL>
+__global__ void __launch_bounds__(kColThreads) k_check_csc(const int64_t* col_ptr, const int32_t* row_idx,
+                                                           const T* values, int64_t p, int64_t n,
+                                                           const int8_t* status, int32_t nwarps, uint32_t wpw,
+                                                           typename AccOf<T>::type* part, int32_t* woff,
+                                                           unsigned* perr) {
+  using A = typename AccOf<T>::type;
+  constexpr int U = 4;
+  const int lane = threadIdx.x & 31;
+  const float inv_wpw = 1.f / (float)wpw;
   unsigned bits = 0;
   for (int64_t j = blockIdx.y; j < p; j += gridDim.y) {
     const int64_t a = col_ptr[j], b = col_ptr[j + 1];
-    for (int64_t i = a + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < b;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t r = row_idx[i];
-      if (r < 0 || r >= n) bits |= PREP_INDEX;
-      if (i > a && row_idx[i - 1] >= r) bits |= PREP_INDEX;
-      if (values && !isfinite(values[i])) bits |= PREP_NONFINITE;
-      if (values && values[i] != T(1)) bits |= PREP_VALUES_NOT_ONE;
+    A acc;
+    acc_zero(acc);
+    // the warp that holds row r: r / 32 / wpw by a float quotient, corrected
+    auto warp_of = [&](int32_t r) {
+      const uint32_t x = (uint32_t)r >> 5;
+      uint32_t q = (uint32_t)((float)x * inv_wpw);
+      const int32_t rem = (int32_t)(x - q * wpw);
+      if (rem < 0) --q;
+      else if (rem >= (int32_t)wpw) ++q;
+      return (int32_t)q;
+    };
+    int32_t* wo = FULL ? woff + j * (nwarps + 1) : nullptr;
+    if (FULL && blockIdx.x == 0 && a == b)
+      for (int g = threadIdx.x; g <= nwarps; g += kColThreads) wo[g] = 0;
+    // whole rounds of U x kColThreads entries per block (every lane takes part)
+    for (int64_t i0 = a + (int64_t)blockIdx.x * (U * kColThreads); i0 < b; i0 += (int64_t)gridDim.x * (U * kColThreads)) {
+      int32_t r[U], rp[U];
+      T v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = i0 + u * kColThreads + threadIdx.x;
+        r[u] = i < b ? row_idx[i] : -1;
+        rp[u] = (lane == 0 && i < b && i > a) ? row_idx[i - 1] : -1;
+        v[u] = (values && i < b) ? values[i] : T(1);
+      }
+      int8_t st[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) st[u] = (FULL && r[u] >= 0 && r[u] < n) ? status[r[u]] : (int8_t)0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = i0 + u * kColThreads + threadIdx.x;
+        const int32_t up = __shfl_up_sync(0xffffffffu, r[u], 1);
+        const int32_t prev = lane == 0 ? rp[u] : up;
+        if (i >= b) continue;
+        bool good = r[u] >= 0 && r[u] < n;
+        if (i > a && prev >= r[u]) good = false;
+        if (!good) bits |= PREP_INDEX;
+        if (values) {
+          if (!isfinite(v[u])) bits |= PREP_NONFINITE;
+          if (v[u] != T(1)) bits |= PREP_VALUES_NOT_ONE;
+        }
+        if (FULL) {
+          if (st[u] == 1) acc = acc_add_v(acc, v[u]);
+          if (good && (i == a || prev >= 0)) {
+            const int32_t g1 = warp_of(r[u]);
+            const int32_t g0 = i > a ? warp_of(prev) + 1 : 0;
+            for (int32_t g = g0; g <= g1; ++g) wo[g] = (int32_t)(i - a);
+            if (i == b - 1)
+              for (int32_t g = g1 + 1; g <= nwarps; ++g) wo[g] = (int32_t)(b - a);
+          }
+        }
+      }
+    }
+    if (FULL) {
+      __syncthreads();   // the previous column's partial has been read
+      block_partial<A>(acc, part + j * gridDim.x + blockIdx.x);
     }
   }
   if (bits) atomicOr(perr, bits);
 }
 
+// Dense column blockIdx.y: finite values and, with part, the block's share of
+// delta^T X_j.  Four rows a load (16 bytes of FP32) where base and pitch
+// allow it.  Bound by the bytes of X; one block per column left two thirds
+// of the chip idle (1.2 ms for 1 GB of 50 columns, after a check pass of
+// 0.45 ms with a 64-bit division per element).
 template <typename T>
-__global__ void k_check_dense(const T* X, int64_t ld, int64_t n, int64_t p, unsigned* perr) {
+__global__ void __launch_bounds__(kColThreads) k_check_dense(const T* X, int64_t ld, int64_t n, int64_t p,
+                                                             const int8_t* status, typename AccOf<T>::type* part,
+                                                             unsigned* perr) {
+  using A = typename AccOf<T>::type;
+  constexpr int U = 4;
   unsigned bits = 0;
-  const int64_t total = n * p;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = t / n, i = t - j * n;
-    if (!isfinite(X[j * ld + i])) bits |= PREP_NONFINITE;
+  const bool vec = (((uintptr_t)X & 15) | ((uintptr_t)(ld * sizeof(T)) & 15) | ((uintptr_t)status & 3)) == 0;
+  const int64_t quads = (n + 3) >> 2;
+  for (int64_t j = blockIdx.y; j < p; j += gridDim.y) {
+    const T* x = X + j * ld;
+    A acc;
+    acc_zero(acc);
+    for (int64_t q0 = (int64_t)blockIdx.x * (U * kColThreads) + threadIdx.x; q0 < quads;
+         q0 += (int64_t)gridDim.x * (U * kColThreads)) {
+      T v[U][4];
+      uint32_t st[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = (q0 + u * kColThreads) * 4;
+        st[u] = 0;
+        if (vec && i + 4 <= n) {
+          if constexpr (sizeof(T) == 4) {
+            const float4 f = __ldcs(reinterpret_cast<const float4*>(x + i));
+            v[u][0] = f.x, v[u][1] = f.y, v[u][2] = f.z, v[u][3] = f.w;
+          } else {
+            const double2 f = __ldcs(reinterpret_cast<const double2*>(x + i));
+            const double2 g = __ldcs(reinterpret_cast<const double2*>(x + i + 2));
+            v[u][0] = f.x, v[u][1] = f.y, v[u][2] = g.x, v[u][3] = g.y;
+          }
+          if (part) st[u] = *reinterpret_cast<const uint32_t*>(status + i);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            v[u][e] = i + e < n ? x[i + e] : T(0);
+            if (part && i + e < n) st[u] |= (uint32_t)(uint8_t)status[i + e] << (8 * e);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (!isfinite(v[u][e])) bits |= PREP_NONFINITE;
+          if ((st[u] >> (8 * e) & 255u) == 1u) acc = acc_add_v(acc, v[u][e]);
+        }
+    }
+    if (part) {
+      __syncthreads();
+      block_partial<A>(acc, part + j * gridDim.x + blockIdx.x);
+    }
   }
   if (bits) atomicOr(perr, bits);
+}
+
+// delta^T X_j from its nb partial sums (one warp a column, fixed order), and
+// the initial trust-region width.
+template <typename A>
+__global__ void __launch_bounds__(kColThreads) k_coord_init(const A* part, int nb, int64_t p, double* dTx,
+                                                            double* width) {
+  const int lane = threadIdx.x & 31;
+  const int64_t j = ((int64_t)blockIdx.x * kColThreads + threadIdx.x) >> 5;
+  if (j >= p) return;   // the whole warp
+  A a;
+  acc_zero(a);
+  for (int q = lane; q < nb; q += 32) a = acc_add(a, part[j * nb + q]);
+  a = warp_sum(a);
+  if (lane == 0) {
+    dTx[j] = acc_to_d(a);
+    width[j] = 1.0;
+  }
 }
 
 __global__ void k_check_finite(const double* v, int64_t count, unsigned* perr) {
@@ -294,23 +448,43 @@ __global__ void k_km_factor(const int32_t* gend, const int32_t* ck, int32_t K, d
     f[k] = 1.0 - (double)ck[k] / (double)((int64_t)gend[k] + 1);
 }
 
-__device__ __forceinline__ void km_put(double* Gk, float2* Gkff, int64_t k, double v) {
-  Gk[k] = v;
-  if (Gkff) {
-    const ff q = d_to_ff(v);
-    Gkff[k] = make_float2(q.hi, q.lo);
-  }
-}
-
-// Gk holds the factors on entry and G(t_k) on exit (one block).
-__global__ void __launch_bounds__(kKmThreads) k_km_product(int32_t K, double* Gk, float2* Gkff) {
+// Gk holds the factors on entry and G(t_k) on exit (one block).  The ordered
+// product is a chain of dependent FP64 multiplications by one thread, so its
+// operands come from shared memory, eight ahead of their use, and nothing
+// else stands in the chain (out of global memory, with the float-float copies
+// written on the way, 1000 groups took 225 us and 3,650 groups 318).
+__global__ void __launch_bounds__(kKmThreads) k_km_product(int32_t K, double* Gk) {
   if (K <= kKmSerial) {
-    if (threadIdx.x != 0) return;
-    double acc = 1.0;
-    for (int64_t k = (int64_t)K - 1; k >= 0; --k) {
-      acc = acc * Gk[k];
-      km_put(Gk, Gkff, k, acc);
+    __shared__ double s_f[kKmSerial];
+    for (int k = threadIdx.x; k < K; k += kKmThreads) s_f[k] = Gk[k];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double acc = 1.0;
+      int k = K - 1;
+      double f[8];
+      if (k >= 7) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = s_f[k - u];
+      }
+      for (; k >= 7; k -= 8) {
+        double nx[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) nx[u] = k - 8 - u >= 0 ? s_f[k - 8 - u] : 1.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          acc = acc * f[u];
+          s_f[k - u] = acc;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = nx[u];
+      }
+      for (; k >= 0; --k) {
+        acc = acc * s_f[k];
+        s_f[k] = acc;
+      }
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < K; k += kKmThreads) Gk[k] = s_f[k];
     return;
   }
   __shared__ double s_w[32];
@@ -344,79 +518,75 @@ __global__ void __launch_bounds__(kKmThreads) k_km_product(int32_t K, double* Gk
   double acc = later_warps * in_warp;   // product of the chunks after this one
   for (int64_t k = b - 1; k >= a; --k) {
     acc = acc * Gk[k];
-    km_put(Gk, Gkff, k, acc);
+    Gk[k] = acc;
   }
 }
 
+// G(t_k) as float-float and 1 / G(t_k) in the working precision.
 template <typename T>
-__global__ void k_w2(const int32_t* gend, int32_t K, const int8_t* status, const double* Gk, T* w2) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < K; k += nwarp) {
-    const int64_t a = k == 0 ? 0 : (int64_t)gend[k - 1] + 1, b = gend[k];
-    const T inv = (T)(1.0 / Gk[k]);
-    for (int64_t i = a + lane; i <= b; i += 32) w2[i] = status[i] == 2 ? inv : T(0);
+__global__ void k_km_finish(int32_t K, const double* Gk, float2* Gkff, T* inv) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x) {
+    const ff q = d_to_ff(Gk[k]);
+    Gkff[k] = make_float2(q.hi, q.lo);
+    inv[k] = (T)(1.0 / Gk[k]);
   }
 }
 
+// W_r = I(status_r = 2) / G(y_r), rows in the blocks of k_group_count (a
+// row's group is the number of group ends before it): 5 bytes read and one
+// value written a subject, whatever the group sizes.  (A warp per group left
+// the largest of 1000 groups to one warp: 384 us for 5 x 10^6 subjects.)
 template <typename T>
-__device__ __forceinline__ void block_sum_store(typename AccOf<T>::type v, double* dst) {
-  using A = typename AccOf<T>::type;
-  __shared__ A s[32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  v = warp_sum(v);
-  if (lane == 0) s[w] = v;
+__global__ void __launch_bounds__(kGrpThreads) k_w2(const int32_t* time, const int8_t* status, int64_t n, int64_t nb,
+                                                    const int32_t* cnt, const T* inv, T* w2) {
+  __shared__ unsigned s_w[kGrpThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const bool vec = quad_aligned(time, status);
+  const int64_t r0 = (int64_t)blockIdx.x * kGrpRows + w * (128 * kGrpRounds) + lane * 4;
+  RowQuad q[kGrpRounds];
+  unsigned c = 0;
+#pragma unroll
+  for (int it = 0; it < kGrpRounds; ++it) {
+    q[it] = load_quad(time, status, n, r0 + 128 * it, vec, 2);
+    c += (unsigned)__popc(q[it].end);
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) s_w[w] = c;
   __syncthreads();
-  if (w == 0) {
-    A u;
-    acc_zero(u);
-    if (lane < (int)(blockDim.x >> 5)) u = s[lane];
-    u = warp_sum(u);
-    if (lane == 0) *dst = acc_to_d(u);
-  }
-}
-
-// delta^T X_j over the nonzeros of column j (one block per column)
-template <typename T>
-__global__ void k_dtx_csc(const int64_t* col_ptr, const int32_t* row_idx, const T* values, const int8_t* status,
-                          double* dTx) {
-  using A = typename AccOf<T>::type;
-  const int64_t j = blockIdx.x;
-  const int64_t a = col_ptr[j], b = col_ptr[j + 1];
-  const int64_t NT = blockDim.x;
-  A acc;
-  acc_zero(acc);
-  // eight independent gathers in flight per thread
-  int64_t i = a + threadIdx.x;
-  for (; i + 7 * NT < b; i += 8 * NT) {
-    int32_t r[8];
-    T v[8];
+  int32_t k0 = cnt[blockIdx.x];
+  for (int v = 0; v < w; ++v) k0 += (int32_t)s_w[v];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      r[u] = row_idx[i + u * NT];
-      v[u] = values ? values[i + u * NT] : T(1);
+  for (int it = 0; it < kGrpRounds; ++it) {
+    const int mine = __popc(q[it].end);
+    int incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += v;
     }
-    int8_t st[8];
+    int32_t k = k0 + incl - mine;
+    k0 += __shfl_sync(0xffffffffu, incl, 31);
+    const int64_t i0 = r0 + 128 * it;
+    T v[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) st[u] = status[r[u]];
+    for (int u = 0; u < 4; ++u) {
+      const bool comp = i0 + u < n && !((q[it].ev | q[it].ce) >> u & 1u);   // status 2 (0 and 1 are the others)
+      v[u] = comp ? inv[k] : T(0);
+      k += (int)(q[it].end >> u & 1u);
+    }
+    if (i0 + 4 <= n) {   // w2 is the library's own, 256-byte aligned
+      if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(w2 + i0) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+        *reinterpret_cast<double2*>(w2 + i0) = make_double2(v[0], v[1]);
+        *reinterpret_cast<double2*>(w2 + i0 + 2) = make_double2(v[2], v[3]);
+      }
+    } else {
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (st[u] == 1) acc = acc_add_v(acc, v[u]);
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < n) w2[i0 + u] = v[u];
+    }
   }
-  for (; i < b; i += NT)
-    if (status[row_idx[i]] == 1) acc = acc_add_v(acc, values ? values[i] : T(1));
-  block_sum_store<T>(acc, dTx + j);
-}
-
-template <typename T>
-__global__ void k_dtx_dense(const T* X, int64_t ld, int64_t n, const int8_t* status, double* dTx) {
-  using A = typename AccOf<T>::type;
-  const int64_t j = blockIdx.x;
-  A acc;
-  acc_zero(acc);
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x)
-    if (status[i] == 1) acc = acc_add_v(acc, X[j * ld + i]);
-  block_sum_store<T>(acc, dTx + j);
 }
 
 // first group whose end is at or after the warp's first row
@@ -533,12 +703,26 @@ __device__ __forceinline__ float to_wide<float, __nv_bfloat16>(__nv_bfloat16 v) 
 template <>
 __device__ __forceinline__ double to_wide<double, __nv_bfloat16>(__nv_bfloat16 v) { return (double)__bfloat162float(v); }
 
+// column blockIdx.y of a dense matrix, widened to the working precision and
+// padded to the pitch ld with zeros
 template <typename S, typename D>
 __global__ void k_convert_dense(const S* src, int64_t n, int64_t p, D* dst, int64_t ld) {
-  const int64_t total = ld * p;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = t / ld, i = t - j * ld;
-    dst[t] = i < n ? to_wide<D>(src[j * n + i]) : D(0);
+  constexpr int U = 4;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = blockIdx.y; j < p; j += gridDim.y) {
+    const S* x = src + j * n;
+    D* y = dst + j * ld;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < ld; i0 += U * stride) {
+      D v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = i0 + u * stride;
+        v[u] = i < n ? to_wide<D>(x[i]) : D(0);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * stride < ld) y[i0 + u * stride] = v[u];
+    }
   }
 }
 
@@ -550,21 +734,46 @@ __global__ void k_convert_vec(const S* src, int64_t count, D* dst) {
 
 }  // namespace
 
+int prep_col_blocks(int64_t longest, int64_t p) {
+  const int64_t most = std::max<int64_t>(1, std::min<int64_t>(kMaxColBlocks, 65536 / std::max<int64_t>(1, p)));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(most, (longest + kColChunk - 1) / kColChunk));
+}
+
 cudaError_t prep_check_csc(const int64_t* col_ptr, const int32_t* row_idx, const void* values, int prec, int64_t p,
-                           int64_t n, unsigned* perr, cudaStream_t s) {
+                           int64_t n, int nb, const PrepColumns* out, unsigned* perr, cudaStream_t s) {
   if (p <= 0) return cudaSuccess;
-  dim3 grid(64, (unsigned)(p < 65535 ? p : 65535));
-  if (prec == 0) k_check_csc<float><<<grid, kPrepThreads, 0, s>>>(col_ptr, row_idx, (const float*)values, p, n, perr);
-  else k_check_csc<double><<<grid, kPrepThreads, 0, s>>>(col_ptr, row_idx, (const double*)values, p, n, perr);
+  const dim3 grid((unsigned)nb, (unsigned)(p < 65535 ? p : 65535));
+  const PrepColumns o = out ? *out : PrepColumns{};
+  const uint32_t wpw = (uint32_t)std::max<int64_t>(1, o.rows_per_warp / 32);
+  if (prec == 0) {
+    auto k = out ? k_check_csc<float, true> : k_check_csc<float, false>;
+    k<<<grid, kColThreads, 0, s>>>(col_ptr, row_idx, (const float*)values, p, n, o.status, o.nwarps, wpw, (ff*)o.part,
+                                   o.woff, perr);
+  } else {
+    auto k = out ? k_check_csc<double, true> : k_check_csc<double, false>;
+    k<<<grid, kColThreads, 0, s>>>(col_ptr, row_idx, (const double*)values, p, n, o.status, o.nwarps, wpw,
+                                   (double*)o.part, o.woff, perr);
+  }
   return cudaGetLastError();
 }
 
-cudaError_t prep_check_dense(const void* X, int prec, int64_t ld, int64_t n, int64_t p, unsigned* perr,
-                             cudaStream_t s) {
+cudaError_t prep_check_dense(const void* X, int prec, int64_t ld, int64_t n, int64_t p, int nb,
+                             const PrepColumns* out, unsigned* perr, cudaStream_t s) {
   if (n <= 0 || p <= 0) return cudaSuccess;
-  const unsigned g = grid_for(n * p, kPrepThreads, 8192);
-  if (prec == 0) k_check_dense<float><<<g, kPrepThreads, 0, s>>>((const float*)X, ld, n, p, perr);
-  else k_check_dense<double><<<g, kPrepThreads, 0, s>>>((const double*)X, ld, n, p, perr);
+  const dim3 grid((unsigned)nb, (unsigned)(p < 65535 ? p : 65535));
+  const int8_t* status = out ? out->status : nullptr;
+  void* part = out ? out->part : nullptr;
+  if (prec == 0) k_check_dense<float><<<grid, kColThreads, 0, s>>>((const float*)X, ld, n, p, status, (ff*)part, perr);
+  else k_check_dense<double><<<grid, kColThreads, 0, s>>>((const double*)X, ld, n, p, status, (double*)part, perr);
+  return cudaGetLastError();
+}
+
+cudaError_t prep_coord_init(const void* part, int prec, int nb, int64_t p, double* dTx, double* width,
+                            cudaStream_t s) {
+  if (p <= 0) return cudaSuccess;
+  const unsigned g = (unsigned)((p * 32 + kColThreads - 1) / kColThreads);
+  if (prec == 0) k_coord_init<ff><<<g, kColThreads, 0, s>>>((const ff*)part, nb, p, dTx, width);
+  else k_coord_init<double><<<g, kColThreads, 0, s>>>((const double*)part, nb, p, dTx, width);
   return cudaGetLastError();
 }
 
@@ -598,39 +807,28 @@ cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t 
   return cudaGetLastError();
 }
 
-cudaError_t prep_km(const int32_t* gend, const int32_t* ck, int32_t K, double* Gk, float2* Gkff, cudaStream_t s) {
+cudaError_t prep_km(const int32_t* gend, const int32_t* ck, int32_t K, double* Gk, cudaStream_t s) {
   if (K <= 0) return cudaSuccess;
   k_km_factor<<<grid_for(K, kPrepThreads, 16384), kPrepThreads, 0, s>>>(gend, ck, K, Gk);
   cudaError_t st = cudaGetLastError();
   if (st != cudaSuccess) return st;
-  k_km_product<<<1, kKmThreads, 0, s>>>(K, Gk, Gkff);
+  k_km_product<<<1, kKmThreads, 0, s>>>(K, Gk);
   return cudaGetLastError();
 }
 
-cudaError_t prep_w2(const int32_t* gend, int32_t K, const int8_t* status, const double* Gk, void* w2, int prec,
-                    cudaStream_t s) {
-  if (K <= 0) return cudaSuccess;
-  const unsigned g = grid_for((int64_t)K * 32, kPrepThreads, 16384);
-  if (prec == 0) k_w2<float><<<g, kPrepThreads, 0, s>>>(gend, K, status, Gk, (float*)w2);
-  else k_w2<double><<<g, kPrepThreads, 0, s>>>(gend, K, status, Gk, (double*)w2);
-  return cudaGetLastError();
-}
-
-cudaError_t prep_dtx_csc(const int64_t* col_ptr, const int32_t* row_idx, const void* values, int prec,
-                         const int8_t* status, int64_t p, double* dTx, cudaStream_t s) {
-  if (p <= 0) return cudaSuccess;
-  if (prec == 0)
-    k_dtx_csc<float><<<(unsigned)p, 1024, 0, s>>>(col_ptr, row_idx, (const float*)values, status, dTx);
-  else
-    k_dtx_csc<double><<<(unsigned)p, 1024, 0, s>>>(col_ptr, row_idx, (const double*)values, status, dTx);
-  return cudaGetLastError();
-}
-
-cudaError_t prep_dtx_dense(const void* X, int prec, int64_t ld, int64_t n, const int8_t* status, int64_t p,
-                           double* dTx, cudaStream_t s) {
-  if (p <= 0) return cudaSuccess;
-  if (prec == 0) k_dtx_dense<float><<<(unsigned)p, 1024, 0, s>>>((const float*)X, ld, n, status, dTx);
-  else k_dtx_dense<double><<<(unsigned)p, 1024, 0, s>>>((const double*)X, ld, n, status, dTx);
+cudaError_t prep_weights(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
+                         const double* Gk, float2* Gkff, void* inv, void* w2, int prec, cudaStream_t s) {
+  if (K <= 0 || n <= 0) return cudaSuccess;
+  const int64_t nb = (n + kGrpRows - 1) / kGrpRows;
+  const unsigned g = grid_for(K, kPrepThreads, 16384);
+  const int32_t* c = static_cast<const int32_t*>(cnt);
+  if (prec == 0) {
+    k_km_finish<float><<<g, kPrepThreads, 0, s>>>(K, Gk, Gkff, (float*)inv);
+    k_w2<float><<<(unsigned)nb, kGrpThreads, 0, s>>>(time, status, n, nb, c, (const float*)inv, (float*)w2);
+  } else {
+    k_km_finish<double><<<g, kPrepThreads, 0, s>>>(K, Gk, Gkff, (double*)inv);
+    k_w2<double><<<(unsigned)nb, kGrpThreads, 0, s>>>(time, status, n, nb, c, (const double*)inv, (double*)w2);
+  }
   return cudaGetLastError();
 }
 
@@ -695,7 +893,7 @@ cudaError_t prep_fill_f64(double* v, double value, int64_t count, cudaStream_t s
 cudaError_t prep_convert_dense(const void* src, int src_dtype, int64_t n, int64_t p, void* dst, int prec, int64_t ld,
                                cudaStream_t s) {
   if (ld * p <= 0) return cudaSuccess;
-  const unsigned g = grid_for(ld * p, kPrepThreads, 16384);
+  const dim3 g(grid_for((ld + 3) / 4, kPrepThreads, 1024), (unsigned)std::min<int64_t>(p, 65535));
   if (src_dtype == 0 && prec == 0) k_convert_dense<float, float><<<g, kPrepThreads, 0, s>>>((const float*)src, n, p, (float*)dst, ld);
   else if (src_dtype == 0) k_convert_dense<float, double><<<g, kPrepThreads, 0, s>>>((const float*)src, n, p, (double*)dst, ld);
   else if (src_dtype == 2 && prec == 0)

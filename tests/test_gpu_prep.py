@@ -52,3 +52,54 @@ def test_sort_at_tile_edges_and_key_spans(lib, n, span):
     np.testing.assert_array_equal(binding.surv_sort_desc(t).cpu().numpy(), ref)
     binding.surv_sort_desc(t, perm=t)   # the order written over the times
     np.testing.assert_array_equal(t.cpu().numpy(), ref)
+
+
+def _against_oracle(model, d, X, values, where, j_list):
+    """l, l', l'' in the FP64 mode: 1e-10 of the sums of magnitudes, as the
+    parity tests hold it."""
+    import torch
+    put = (lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda())
+    if where == "csc":
+        import scipy.sparse
+        S = scipy.sparse.csc_matrix(X)
+        S.sort_indices()
+        sd = binding.SurvData(put(d["time"]), put(d["status"]), col_ptr=put(S.indptr.astype(np.int64)),
+                              row_idx=put(S.indices.astype(np.int32)), values=put(S.data) if values else None,
+                              n=X.shape[0], p=X.shape[1])
+    else:
+        sd = binding.SurvData(put(d["time"]), put(d["status"]), X=put(np.ascontiguousarray(X.T)))
+    beta = np.linspace(-0.2, 0.2, X.shape[1])
+    ev = d["status"] == 1
+    for j in j_list:
+        l, g, h = binding.loglik_grad_hess(sd, model, beta, j, precision="f64")
+        lo, go, ho = oracle.model_terms(model, d["time"], d["status"], X, beta, j)
+        m = np.max(np.abs(X[:, j]), initial=0.0)
+        scale = max(1.0, float(np.count_nonzero(ev)))
+        assert abs(l - lo) <= 1e-10 * max(1.0, abs(lo))
+        assert abs(g - go) <= 1e-10 * scale * max(m, 1e-300)
+        assert abs(h - ho) <= 1e-10 * scale * max(m * m, 1e-300)
+
+
+# the column pass takes 1024 entries a round and 4096 a block
+@pytest.mark.parametrize("values", [False, True])
+def test_columns_of_every_length(lib, values):
+    from paper_2204_08183_gb300 import synth
+    n = 9001
+    d = synth.cohort_small(n, 1, seed=5, n_times=700)
+    rng = np.random.default_rng(6)
+    lengths = [0, 1, 2, 31, 33, 1023, 1024, 1025, 4095, 4097, n]
+    X = np.zeros((n, len(lengths)))
+    for j, k in enumerate(lengths):
+        rows = np.sort(rng.choice(n, k, replace=False))
+        if k in (1, 2):
+            rows = np.array([0, n - 1])[:k] if k == 2 else np.array([n - 1])
+        X[rows, j] = rng.normal(size=k) if values else 1.0
+    _against_oracle("cox", d, X, values, "csc", range(len(lengths)))
+
+
+@pytest.mark.parametrize("n", [1, 5, 127, 4095, 4097, 8193, 20003])
+def test_dense_and_weights_at_block_edges(lib, n):
+    from paper_2204_08183_gb300 import synth
+    d = synth.cohort_small(n, 3, seed=n, n_times=max(1, n // 7), competing_frac=0.3)
+    d["status"][0] = 1
+    _against_oracle("fg", d, np.asarray(d["X"]), True, "dense", range(3))
