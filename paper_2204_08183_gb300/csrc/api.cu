@@ -245,6 +245,17 @@ int stage_data(const surv_data* d, int prec, surv_workspace* ws, cudaStream_t s,
   return SURV_OK;
 }
 
+// Workspace of the row masks of n subjects.
+int row_masks(surv_workspace* ws, int64_t n, survgpu::RowMasks* m) {
+  const int64_t nwords = (n + 31) / 32;
+  void* v = nullptr;
+  const int rc = ensure(ws, surv_workspace::ROWMASK, 8 * (size_t)nwords, &v);
+  if (rc) return rc;
+  m->end = static_cast<uint32_t*>(v);
+  m->first = reinterpret_cast<int32_t*>(m->end + nwords);
+  return SURV_OK;
+}
+
 // Validation kernels on the staged data and the tie-group count: *K and the
 // number of events after a synchronisation (ctrl zeroed here; prep errors mapped to return codes).
 // CSC values that are all exactly 1 are dropped from st (the kernels then
@@ -459,9 +470,11 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     S.multi = (int64_t)K >= 2 * (int64_t)nwarps ? 1 : 0;
   }
 
+  survgpu::RowMasks masks;
+  if ((rc = row_masks(ws, n, &masks))) return rc;
   CUDA_TRY(survgpu::prep_group_write(time_p, status_p, n, cnt, K, static_cast<int32_t*>(gend),
                                      static_cast<int32_t*>(dk), static_cast<int32_t*>(ck), nwarps, rows_per_warp,
-                                     static_cast<int32_t*>(wk0), s));
+                                     static_cast<int32_t*>(wk0), s, &masks));
   ++launches;
   if (model == SURV_FG) {
     CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), s));
@@ -520,6 +533,8 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   P.Gk = static_cast<const double*>(Gk);
   P.Gkff = static_cast<const float2*>(Gkff);
   P.wk0 = static_cast<const int32_t*>(wk0);
+  P.endw = masks.end;
+  P.wordk = masks.first;
   P.col_ptr = static_cast<const int64_t*>(colptr_d);
   P.row_idx = static_cast<const int32_t*>(rowidx_d);
   P.values = layout == SURV_CSC ? vals_d : nullptr;
@@ -836,8 +851,10 @@ int cv_impl(const surv_data* d, const int8_t* fold_id, int nfolds, const double*
 
   CUDA_TRY(cudaMemsetAsync(cvc, 0, sizeof(CvCtrl), s));
   CUDA_TRY(survgpu::cv_check_folds(fold_d, n, nfolds, &cvc->perr, s));
+  survgpu::RowMasks masks;
+  if ((rc = row_masks(ws, n, &masks))) return rc;
   CUDA_TRY(survgpu::prep_group_write(stg.time, stg.status, n, cnt, K, static_cast<int32_t*>(gend),
-                                     static_cast<int32_t*>(dk), nullptr, 0, 32, nullptr, s));
+                                     static_cast<int32_t*>(dk), nullptr, 0, 32, nullptr, s, &masks));
   CUDA_TRY(survgpu::cv_fold_stats(static_cast<int32_t*>(gend), K, stg.status, fold_d, nfolds,
                                   static_cast<int32_t*>(dkf), cvc->events, s));
   CUDA_TRY(survgpu::cv_dtx(layout == SURV_CSC ? 0 : 1, prec, stg.colptr, stg.rowidx, stg.vals, stg.ld, n, p,
@@ -890,6 +907,8 @@ int cv_impl(const surv_data* d, const int8_t* fold_id, int nfolds, const double*
     P.nwarps = nwarps;
     P.gend = static_cast<const int32_t*>(gend);
     P.wk0 = static_cast<const int32_t*>(wk0);
+    P.endw = masks.end;
+    P.wordk = masks.first;
     P.col_ptr = stg.colptr;
     P.row_idx = stg.rowidx;
     P.values = layout == SURV_CSC ? stg.vals : nullptr;

@@ -223,12 +223,26 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
   const uint64_t keep = l2_keep(), strm = l2_stream();
 #pragma unroll
   for (int m = 0; m < M; ++m) acc_zero(tot[m]);
+  A drun[ND];   // MULTI: warp-uniform sums of the dense components
+#pragma unroll
+  for (int d = 0; d < ND; ++d) acc_zero(drun[d]);
   if (LAYOUT == 1 || dense) {
     A acc[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) acc_zero(acc[d]);
     EndCursor ec{pf.k_lo, pf.k_hi, pf.k_lo, pf.kreg};
-    int64_t next_end = ec.pos(P.gend);
+    int64_t next_end = MULTI ? 0 : ec.pos(P.gend);
+    // many-ends form: the ends among a lane's rows of each chunk row u (bit q:
+    // its row q ends a group) and the group of the first, from the end masks.
+    // Every lane writes the records of its own rows, and in the sparse part
+    // below an end a lane: the work of a tile does not grow with its ends.
+    // (One end after another by the whole warp bounded the pass by its issue
+    // slots: a fit of 333,331 subjects with hardly any ties took 22.5 ms and
+    // takes 7.1; the cross-validated path at n = 10^6, 15 ends a warp, 671 ms
+    // and 576.)
+    uint32_t nib[U];
+    int kq[U];
+    bool acc_dirty = false;   // ND > 1: acc holds lane partials since the last fold into drun
     const T* xcol = LAYOUT == 1 ? reinterpret_cast<const T*>(P.X) + (size_t)j * P.ld : nullptr;
 
     // loads of one tile from global memory (16-byte loads; the last partial
@@ -355,32 +369,91 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           const T t = __shfl_up_sync(0xffffffffu, ex[u], 1);
           ex[u] = lane == 0 ? T(0) : t;                  // lanes before, same u
         }
-        while (next_end < t_end) {
-          const int off = (int)(next_end - t0);
-          const int cstar = off / VEC, qstar = off - cstar * VEC;
-          if ((cstar & 31) == lane) {
-            const int ustar = cstar >> 5;
-            T pre = T(0);
+        T pu = T(0);   // chunk rows before u
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-              if (u < ustar) pre += tu[u];
-              if (u == ustar) {
-                T in = ex[u];
+        for (int u = 0; u < U; ++u) {
+          if (nib[u]) {
+            T in = ex[u];
+            int k = kq[u];
 #pragma unroll
-                for (int q = 0; q < VEC; ++q)
-                  if (q <= qstar) in += dense_comp<MODEL, LAYOUT, T>(0, ev[u][q], xv[u][q], wv[u][q]);
-                pre += in;
+            for (int q = 0; q < VEC; ++q) {
+              in += dense_comp<MODEL, LAYOUT, T>(0, ev[u][q], xv[u][q], wv[u][q]);
+              if (nib[u] >> q & 1u) {
+                rec[(size_t)k * M + C::dmap(0)] = acc_add_v(acc[0], pu + in);
+                ++k;
               }
             }
-            rec[(size_t)ec.kn * M + C::dmap(0)] = acc_add_v(acc[0], pre);
           }
-          ++ec.kn;
-          next_end = ec.pos(P.gend);
+          pu += tu[u];
         }
         T tt = tu[0];
 #pragma unroll
         for (int u = 1; u < U; ++u) tt += tu[u];
         acc[0] = acc_add_v(acc[0], tt);
+      } else if constexpr (MULTI) {
+        // Several components.  A tile without an end adds to the lane partials;
+        // one with ends folds them into the warp-uniform sums drun and takes a
+        // lane scan per component and chunk row, as above.
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) any |= nib[u] != 0u;
+        if (!__any_sync(0xffffffffu, any)) {
+#pragma unroll
+          for (int d = 0; d < ND; ++d) {
+            T su[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) su[u] = chunk_sum(d, ev, xv, wv, u);
+#pragma unroll
+            for (int s = 1; s < U; s <<= 1)
+#pragma unroll
+              for (int u = 0; u + s < U; u += 2 * s) su[u] += su[u + s];
+            acc[d] = acc_add_v(acc[d], su[0]);
+          }
+          acc_dirty = true;
+          return;
+        }
+        if (acc_dirty) {
+          warp_sum_some<ND>(acc);
+#pragma unroll
+          for (int d = 0; d < ND; ++d) {
+            drun[d] = acc_add(drun[d], acc[d]);
+            acc_zero(acc[d]);
+          }
+          acc_dirty = false;
+        }
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+          T ex[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) ex[u] = chunk_sum(d, ev, xv, wv, u);
+#pragma unroll
+          for (int dd = 1; dd < 32; dd <<= 1)
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const T t = __shfl_up_sync(0xffffffffu, ex[u], dd);
+              if (lane >= dd) ex[u] += t;
+            }
+          T pu = T(0);
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const T tu = __shfl_sync(0xffffffffu, ex[u], 31);
+            const T t = __shfl_up_sync(0xffffffffu, ex[u], 1);
+            if (nib[u]) {
+              T in = lane == 0 ? T(0) : t;
+              int k = kq[u];
+#pragma unroll
+              for (int q = 0; q < VEC; ++q) {
+                in += dense_comp<MODEL, LAYOUT, T>(d, ev[u][q], xv[u][q], wv[u][q]);
+                if (nib[u] >> q & 1u) {
+                  rec[(size_t)k * M + C::dmap(d)] = acc_add_v(drun[d], pu + in);
+                  ++k;
+                }
+              }
+            }
+            pu += tu;
+          }
+          drun[d] = acc_add_v(drun[d], pu);
+        }
       } else {
         while (next_end < t_end) {
           A pref[ND];
@@ -419,11 +492,29 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
 
     for (int64_t t0 = row_lo; t0 < row_hi; t0 += TILE) {
       T ev[U][VEC], xv[U][VEC], wv[U][VEC];
+      if constexpr (MULTI) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
+          nib[u] = 0u;
+          kq[u] = 0;
+          if (r < row_hi) {
+            const uint32_t word = P.endw[r >> 5];
+            const int sh = (int)(r & 31);
+            nib[u] = word >> sh & ((1u << VEC) - 1u);
+            kq[u] = P.wordk[r >> 5] + __popc(word & ((1u << sh) - 1u));
+          }
+        }
+      }
       load_tile(t0, ev, xv, wv);
       tile(t0, ev, xv, wv);
     }
+    if constexpr (MULTI && ND == 1) {
+      drun[0] = acc[0];   // warp-uniform already
+    } else {
 #pragma unroll
-    for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc[d];  // lane partials (MULTI, ND = 1: the warp sum)
+      for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc[d];  // lane partials
+    }
   }
   if (LAYOUT == 0 && NS > 0) {
     // sparse part: the nonzeros of column j inside the warp's rows
@@ -435,9 +526,8 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
       // warp-uniform sum folded in from sacc by rounds with several ends.  A
       // round with one end reduces sacc plus the round's nonzeros up to the
       // end in one tree.  A round with several ends folds sacc into run, takes
-      // one inclusive lane scan, and each end reads the scan at the last
-      // nonzero at or before it (row indices increase with the lane, so a
-      // ballot counts them).
+      // one inclusive lane scan, and its ends, one a lane, read the scan at
+      // the last nonzero at or before them.
       constexpr int NSX = NS > 0 ? NS : 1;
       A sacc[NSX], run[NSX];
 #pragma unroll
@@ -490,17 +580,21 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           }
           warp_scan_n<NSX>(sc, lane);
           while (next_end < (int64_t)last_row) {
-            const int cnt = __popc(__ballot_sync(0xffffffffu, (int64_t)row <= next_end));
-            A pref[NSX];
+            // the ends of the cursor's window, one a lane: how many of the
+            // round's nonzeros lie at or before it (rows increase with the
+            // lane: a binary search over the lanes), and their prefix
+            const int kk = ec.base + lane, pos = ec.reg;
+            const bool mine = kk >= ec.kn && kk < ec.k_hi && pos < last_row;
+            int cnt = 0;
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1)
+              if (__shfl_sync(0xffffffffu, row, cnt + h - 1) <= pos) cnt += h;
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
               const A v = shfl_idx(sc[s], cnt > 0 ? cnt - 1 : 0);
-              pref[s] = cnt > 0 ? acc_add(run[s], v) : run[s];
+              if (mine) rec[(size_t)kk * M + C::smap(s)] = cnt > 0 ? acc_add(run[s], v) : run[s];
             }
-            if (lane == 0)
-#pragma unroll
-              for (int s = 0; s < NS; ++s) rec[(size_t)ec.kn * M + C::smap(s)] = pref[s];
-            ++ec.kn;
+            ec.kn += __popc(__ballot_sync(0xffffffffu, mine));
             next_end = ec.pos(P.gend);
           }
 #pragma unroll
@@ -552,17 +646,15 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
       // dense sum (both warp-uniform) are added after the reduction
 #pragma unroll
       for (int s = 0; s < NS; ++s) tot[C::smap(s)] = sacc[s];
-      const A dense_run = tot[C::dmap(0)];
-      acc_zero(tot[C::dmap(0)]);
       warp_sum_some<M>(tot);
-      tot[C::dmap(0)] = dense_run;
+#pragma unroll
+      for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc_add(drun[d], tot[C::dmap(d)]);
 #pragma unroll
       for (int s = 0; s < NS; ++s) tot[C::smap(s)] = acc_add(run[s], tot[C::smap(s)]);
       // the ends after the last nonzero of the range see the warp totals
-      for (; ec.kn < pf.k_hi; ++ec.kn)
-        if (lane == 0)
+      for (int k = ec.kn + lane; k < pf.k_hi; k += 32)
 #pragma unroll
-          for (int s = 0; s < NS; ++s) rec[(size_t)ec.kn * M + C::smap(s)] = tot[C::smap(s)];
+        for (int s = 0; s < NS; ++s) rec[(size_t)k * M + C::smap(s)] = tot[C::smap(s)];
     } else {
       const int sa = pf.sa, sb = pf.sb;
       const int32_t* ri = pf.ri;
@@ -620,13 +712,15 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
       for (int s = 0; s < NS; ++s) tot[C::smap(s)] = sacc[s];  // lane partials, reduced below
       // warp totals, then the ends after the last nonzero of the range see them
       warp_sum_some<M>(tot);
-      for (; ec.kn < pf.k_hi; ++ec.kn)
-        if (lane == 0)
+      for (int k = ec.kn + lane; k < pf.k_hi; k += 32)
 #pragma unroll
-          for (int s = 0; s < NS; ++s) rec[(size_t)ec.kn * M + C::smap(s)] = tot[C::smap(s)];
+        for (int s = 0; s < NS; ++s) rec[(size_t)k * M + C::smap(s)] = tot[C::smap(s)];
     }
   } else {
     warp_sum_some<M>(tot);
+    if constexpr (MULTI)
+#pragma unroll
+      for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc_add(drun[d], tot[C::dmap(d)]);
   }
 }
 

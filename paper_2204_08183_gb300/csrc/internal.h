@@ -37,6 +37,8 @@ struct CcdParams {
   const double* Gk;      // [K] Kaplan-Meier censoring survival at t_k (FG)
   const float2* Gkff;    // [K] the same as float-float (hi, lo)
   const int32_t* wk0;    // [nwarps+1] first group index whose end is in warp w
+  const uint32_t* endw;  // [ceil(n/32)] group ends among 32 rows (bit per row) and
+  const int32_t* wordk;  //   group ends before them (many-ends form of the row pass)
 
   const int64_t* col_ptr;  // CSC
   const int32_t* row_idx;
@@ -256,14 +258,18 @@ cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr
 // Tie groups.  prep_group_count checks times and status codes (*perr) and
 // writes *K, *total_events (subjects with status 1) and its block counts
 // into cnt (prep_count_bytes(n) bytes); *ticket is a zeroed word.
-// prep_group_write then fills gend, dk and ck (ck may be null) and, with
-// wk0, the first group of each warp's rows.
+// prep_group_write then fills gend, dk and ck (ck may be null), with wk0 the
+// first group of each warp's rows, and with masks those of every 32 rows.
+struct RowMasks {              // [ceil(n / 32)] each
+  uint32_t* end = nullptr;     // bit r: row 32 w + r ends a group
+  int32_t* first = nullptr;    // group ends before row 32 w
+};
 size_t prep_count_bytes(int64_t n);
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
                              unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s);
 cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
                              int32_t* gend, int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rows_per_warp,
-                             int32_t* wk0, cudaStream_t s);
+                             int32_t* wk0, cudaStream_t s, const RowMasks* masks = nullptr);
 // G(t_k); then its float-float form, 1 / G(t_k) in the working precision (inv:
 // K values of scratch) and W (cnt: the counts of prep_group_count).
 cudaError_t prep_km(const int32_t* gend, const int32_t* ck, int32_t K, double* Gk, cudaStream_t s);

@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
 __global__ void __launch_bounds__(kGrpThreads) k_group_write(const int32_t* time, const int8_t* status, int64_t n,
                                                              int64_t nb, const int32_t* cnt, int32_t K, int32_t* gend,
                                                              int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rpw,
-                                                             int32_t* wk0) {
+                                                             int32_t* wk0, RowMasks masks) {
   __shared__ unsigned s_w[kGrpThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const bool vec = quad_aligned(time, status);
@@ -407,6 +407,15 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_write(const int32_t* time
     const int32_t e0 = base[1] + (int32_t)(ex >> 10 & 1023u), c0 = base[2] + (int32_t)(ex >> 20);
     if (wk0 && (lane & 7) == 0 && i0 < n && (uint32_t)i0 % (uint32_t)rpw == 0)
       wk0[(uint32_t)i0 / (uint32_t)rpw] = k;
+    if (masks.end) {   // the masks of 32 rows: nibbles of 8 lanes
+      uint32_t en = q[it].end << (4 * (lane & 7));
+#pragma unroll
+      for (int d = 1; d < 8; d <<= 1) en |= __shfl_xor_sync(0xffffffffu, en, d);
+      if ((lane & 7) == 0 && i0 < n) {
+        masks.end[i0 >> 5] = en;
+        masks.first[i0 >> 5] = k;
+      }
+    }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (q[it].end >> u & 1u) {
@@ -796,14 +805,14 @@ cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t 
 
 cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
                              int32_t* gend, int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rows_per_warp,
-                             int32_t* wk0, cudaStream_t s) {
+                             int32_t* wk0, cudaStream_t s, const RowMasks* masks) {
   if (K <= 0 || n <= 0) return cudaSuccess;
   cudaError_t st = cudaMemsetAsync(dk, 0, sizeof(int32_t) * (size_t)K, s);
   if (st == cudaSuccess && ck) st = cudaMemsetAsync(ck, 0, sizeof(int32_t) * (size_t)K, s);
   if (st != cudaSuccess) return st;
   const int64_t nb = (n + kGrpRows - 1) / kGrpRows;
   k_group_write<<<(unsigned)nb, kGrpThreads, 0, s>>>(time, status, n, nb, static_cast<const int32_t*>(cnt), K, gend,
-                                                     dk, ck, nwarps, rows_per_warp, wk0);
+                                                     dk, ck, nwarps, rows_per_warp, wk0, masks ? *masks : RowMasks{});
   return cudaGetLastError();
 }
 

@@ -16,7 +16,7 @@ struct surv_workspace {
   };
   enum Id {
     TIME, STATUS, COLPTR, ROWIDX, VALUES, XD, E, ETA, W2, GEND, DK, CK, GK, GKFF, WK0, WOFF, DTX, BETA, WIDTH, PEN, REC,
-    SLOTS, CTRL, BLOCKCNT, DTX_PART, SORTWORK, PERM, PF, WT, AGG,
+    SLOTS, CTRL, BLOCKCNT, DTX_PART, ROWMASK, SORTWORK, PERM, PF, WT, AGG,
     // differentiable form (cox_nll_forward / cox_nll_backward)
     NLL_Y, NLL_BCAT, NLL_REC, NLL_WT, NLL_DEN, NLL_LAM, NLL_G, NLL_GB, NLL_GEND, NLL_DK, NLL_WK0, NLL_BLK,
     NLL_CTRL, NLL_XP, NLL_ERR, NLL_FIN,
