@@ -195,7 +195,9 @@ struct EndCursor {
 // the warp totals (every lane holds them).  The dense components stream e
 // (and X, W) in tiles of 32 * U * VEC rows; the CSC components walk the
 // column's nonzeros in the warp's rows (woff holds the per-warp offsets).
-template <int MODEL, int LAYOUT, typename T, int U_, int SR, bool MULTI = false>
+// WIDE: registers allow every reduction of several components to run
+// interleaved (one tree's latency instead of one per component).
+template <int MODEL, int LAYOUT, typename T, int U_, int SR, bool MULTI = false, bool WIDE = false>
 // dense = false (CSC only): e has not changed since the previous pass of the
 // fit, so the dense components (e, and for Fine-Gray W e), their records at
 // the group ends and their totals are the stored ones; they are neither
@@ -223,9 +225,6 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
   const uint64_t keep = l2_keep(), strm = l2_stream();
 #pragma unroll
   for (int m = 0; m < M; ++m) acc_zero(tot[m]);
-  A drun[ND];   // MULTI: warp-uniform sums of the dense components
-#pragma unroll
-  for (int d = 0; d < ND; ++d) acc_zero(drun[d]);
   if (LAYOUT == 1 || dense) {
     A acc[ND];
 #pragma unroll
@@ -233,7 +232,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
     EndCursor ec{pf.k_lo, pf.k_hi, pf.k_lo, pf.kreg};
     int64_t next_end = MULTI ? 0 : ec.pos(P.gend);
     // many-ends form: the ends among a lane's rows of each chunk row u (bit q:
-    // its row q ends a group) and the group of the first, from the end masks.
+    // its row q ends a group), from the end masks.
     // Every lane writes the records of its own rows, and in the sparse part
     // below an end a lane: the work of a tile does not grow with its ends.
     // (One end after another by the whole warp bounded the pass by its issue
@@ -241,8 +240,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
     // takes 7.1; the cross-validated path at n = 10^6, 15 ends a warp, 671 ms
     // and 576.)
     uint32_t nib[U];
-    int kq[U];
-    bool acc_dirty = false;   // ND > 1: acc holds lane partials since the last fold into drun
+    bool acc_dirty = false;   // acc holds partials of several lanes (else lane 0's alone)
     const T* xcol = LAYOUT == 1 ? reinterpret_cast<const T*>(P.X) + (size_t)j * P.ld : nullptr;
 
     // loads of one tile from global memory (16-byte loads; the last partial
@@ -253,12 +251,18 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           // fused update of the pending step (FP32 mode: eta float-float)
           float2* etap = reinterpret_cast<float2*>(P.eta);
           float* ep = reinterpret_cast<float*>(P.e);
+          auto moved = [&](float2& q, float x) {   // the new eta of a row, and its e
+            const ff v = ff_add({q.x, q.y}, ff_mul_f(delta, x));
+            q = make_float2(v.hi, v.lo);
+            const float ex = expf(v.hi);
+            return fmaf(ex, v.lo, ex);
+          };
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
-            float xx[VEC];
-            float2 qq[VEC];
             if (r + VEC <= row_hi) {
+              float xx[VEC];
+              float2 qq[VEC];
               ld4_hint(reinterpret_cast<const float*>(xq) + r, strm, xx);
               const float4 a = *reinterpret_cast<const float4*>(etap + r);
               const float4 b = *reinterpret_cast<const float4*>(etap + r + 2);
@@ -268,37 +272,32 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
               qq[3] = make_float2(b.z, b.w);
               ld4_hint(xcol + r, strm, xv[u]);
               if (MODEL == 1) ld4_hint(w2 + r, keep, wv[u]);
-            } else {
 #pragma unroll
-              for (int q = 0; q < VEC; ++q) {
-                const bool in = r + q < row_hi;
-                xx[q] = in ? reinterpret_cast<const float*>(xq)[r + q] : 0.f;
-                qq[q] = in ? etap[r + q] : make_float2(0.f, 0.f);
-                xv[u][q] = in ? xcol[r + q] : T(0);
-                wv[u][q] = (MODEL == 1 && in) ? w2[r + q] : T(0);
+              for (int q = 0; q < VEC; ++q) ev[u][q] = moved(qq[q], xx[q]);
+              if (P.fold_id) {
+#pragma unroll
+                for (int q = 0; q < VEC; ++q)
+                  if (P.fold_id[r + q] == P.fold) ev[u][q] = 0.f;
               }
-            }
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-              const ff v = ff_add({qq[q].x, qq[q].y}, ff_mul_f(delta, xx[q]));
-              qq[q] = make_float2(v.hi, v.lo);
-              const float ex = expf(v.hi);
-              // rows past the warp's range take no part (e = 0), as in the plain loads
-              const bool in = r + q < row_hi;
-              const bool held = in && P.fold_id && P.fold_id[r + q] == P.fold;
-              ev[u][q] = (!in || held) ? 0.f : fmaf(ex, v.lo, ex);
-            }
-            if (r + VEC <= row_hi) {
               *reinterpret_cast<float4*>(etap + r) = make_float4(qq[0].x, qq[0].y, qq[1].x, qq[1].y);
               *reinterpret_cast<float4*>(etap + r + 2) = make_float4(qq[2].x, qq[2].y, qq[3].x, qq[3].y);
               *reinterpret_cast<float4*>(ep + r) = make_float4(ev[u][0], ev[u][1], ev[u][2], ev[u][3]);
             } else {
+              // rows past the warp's range take no part (e = 0), as in the plain loads
 #pragma unroll
-              for (int q = 0; q < VEC; ++q)
-                if (r + q < row_hi) {
-                  etap[r + q] = qq[q];
+              for (int q = 0; q < VEC; ++q) {
+                const bool in = r + q < row_hi;
+                ev[u][q] = 0.f;
+                xv[u][q] = in ? xcol[r + q] : T(0);
+                wv[u][q] = (MODEL == 1 && in) ? w2[r + q] : T(0);
+                if (in) {
+                  float2 qv = etap[r + q];
+                  const float en = moved(qv, reinterpret_cast<const float*>(xq)[r + q]);
+                  ev[u][q] = P.fold_id && P.fold_id[r + q] == P.fold ? 0.f : en;
+                  etap[r + q] = qv;
                   ep[r + q] = ev[u][q];
                 }
+              }
             }
           }
           return;
@@ -346,54 +345,13 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
     };
     auto tile = [&](int64_t t0, const T (&ev)[U][VEC], const T (&xv)[U][VEC], const T (&wv)[U][VEC]) {
       const int64_t t_end = min(t0 + (int64_t)TILE, row_hi);
-      if constexpr (ND == 1 && MULTI) {
-        // acc[0] is the warp-uniform sum of the rows before the tile.  One
-        // FP32 lane scan per chunk row u gives every chunk's tile-relative
-        // exclusive prefix; the lane that owns an end's chunk adds the rows
-        // of the chunk up to the end and writes the record.
-        T su[U], ex[U], tu[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) su[u] = chunk_sum(0, ev, xv, wv, u);
-#pragma unroll
-        for (int u = 0; u < U; ++u) ex[u] = su[u];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1)
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const T t = __shfl_up_sync(0xffffffffu, ex[u], d);
-            if (lane >= d) ex[u] += t;
-          }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          tu[u] = __shfl_sync(0xffffffffu, ex[u], 31);  // chunk row total
-          const T t = __shfl_up_sync(0xffffffffu, ex[u], 1);
-          ex[u] = lane == 0 ? T(0) : t;                  // lanes before, same u
-        }
-        T pu = T(0);   // chunk rows before u
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          if (nib[u]) {
-            T in = ex[u];
-            int k = kq[u];
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-              in += dense_comp<MODEL, LAYOUT, T>(0, ev[u][q], xv[u][q], wv[u][q]);
-              if (nib[u] >> q & 1u) {
-                rec[(size_t)k * M + C::dmap(0)] = acc_add_v(acc[0], pu + in);
-                ++k;
-              }
-            }
-          }
-          pu += tu[u];
-        }
-        T tt = tu[0];
-#pragma unroll
-        for (int u = 1; u < U; ++u) tt += tu[u];
-        acc[0] = acc_add_v(acc[0], tt);
-      } else if constexpr (MULTI) {
-        // Several components.  A tile without an end adds to the lane partials;
-        // one with ends folds them into the warp-uniform sums drun and takes a
-        // lane scan per component and chunk row, as above.
+      if constexpr (MULTI) {
+        // A tile without an end adds to the lane partials.  One with ends takes
+        // their sum (from lane 0 alone where the previous tile left it there:
+        // acc_dirty is false) and one FP32 lane scan per chunk row u, which gives
+        // every chunk its tile-relative exclusive prefix; a lane adds the rows
+        // of its chunk up to an end and writes the record.  One component at a
+        // time: the scans of a tile need few registers.
         bool any = false;
 #pragma unroll
         for (int u = 0; u < U; ++u) any |= nib[u] != 0u;
@@ -412,17 +370,10 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           acc_dirty = true;
           return;
         }
-        if (acc_dirty) {
-          warp_sum_some<ND>(acc);
-#pragma unroll
-          for (int d = 0; d < ND; ++d) {
-            drun[d] = acc_add(drun[d], acc[d]);
-            acc_zero(acc[d]);
-          }
-          acc_dirty = false;
-        }
+        if (acc_dirty) warp_sum_set<ND, WIDE>(acc);
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
+          const A before = acc_dirty ? acc[d] : shfl_idx(acc[d], 0);   // the warp's rows before the tile
           T ex[U];
 #pragma unroll
           for (int u = 0; u < U; ++u) ex[u] = chunk_sum(d, ev, xv, wv, u);
@@ -440,20 +391,23 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
             const T t = __shfl_up_sync(0xffffffffu, ex[u], 1);
             if (nib[u]) {
               T in = lane == 0 ? T(0) : t;
-              int k = kq[u];
+              const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
+              int k = P.wordk[r >> 5] + __popc(P.endw[r >> 5] & ((1u << (r & 31)) - 1u));   // its first end
 #pragma unroll
               for (int q = 0; q < VEC; ++q) {
                 in += dense_comp<MODEL, LAYOUT, T>(d, ev[u][q], xv[u][q], wv[u][q]);
                 if (nib[u] >> q & 1u) {
-                  rec[(size_t)k * M + C::dmap(d)] = acc_add_v(drun[d], pu + in);
+                  rec[(size_t)k * M + C::dmap(d)] = acc_add_v(before, pu + in);
                   ++k;
                 }
               }
             }
             pu += tu;
           }
-          drun[d] = acc_add_v(drun[d], pu);
+          acc_zero(acc[d]);
+          if (lane == 0) acc[d] = acc_add_v(before, pu);
         }
+        acc_dirty = false;
       } else {
         while (next_end < t_end) {
           A pref[ND];
@@ -469,7 +423,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
               }
             pref[d] = acc_add_v(acc[d], part);
           }
-          warp_sum_some<ND>(pref);
+          warp_sum_set<ND, WIDE>(pref);
           if (lane == 0)
 #pragma unroll
             for (int d = 0; d < ND; ++d) rec[(size_t)ec.kn * M + C::dmap(d)] = pref[d];
@@ -496,25 +450,14 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
-          nib[u] = 0u;
-          kq[u] = 0;
-          if (r < row_hi) {
-            const uint32_t word = P.endw[r >> 5];
-            const int sh = (int)(r & 31);
-            nib[u] = word >> sh & ((1u << VEC) - 1u);
-            kq[u] = P.wordk[r >> 5] + __popc(word & ((1u << sh) - 1u));
-          }
+          nib[u] = r < row_hi ? P.endw[r >> 5] >> (int)(r & 31) & ((1u << VEC) - 1u) : 0u;
         }
       }
       load_tile(t0, ev, xv, wv);
       tile(t0, ev, xv, wv);
     }
-    if constexpr (MULTI && ND == 1) {
-      drun[0] = acc[0];   // warp-uniform already
-    } else {
 #pragma unroll
-      for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc[d];  // lane partials
-    }
+    for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc[d];  // lane partials
   }
   if (LAYOUT == 0 && NS > 0) {
     // sparse part: the nonzeros of column j inside the warp's rows
@@ -553,7 +496,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           A pref[NSX];
 #pragma unroll
           for (int s = 0; s < NS; ++s) pref[s] = acc_add_v(sacc[s], (int64_t)row <= next_end ? sv[s] : T(0));
-          warp_sum_some<NSX>(pref);
+          warp_sum_set<NSX, WIDE>(pref);
           if (lane == 0)
 #pragma unroll
             for (int s = 0; s < NS; ++s) rec[(size_t)ec.kn * M + C::smap(s)] = acc_add(run[s], pref[s]);
@@ -564,7 +507,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           sacc_dirty = true;
         } else if (next_end < (int64_t)last_row) {
           if (sacc_dirty) {
-            warp_sum_some<NSX>(sacc);
+            warp_sum_set<NSX, WIDE>(sacc);
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
               run[s] = acc_add(run[s], sacc[s]);
@@ -642,13 +585,10 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
         }
         round(row, x, ev, wv, min(32, sb - base));
       }
-      // lane partials of the rounds without ends are reduced; run and the
-      // dense sum (both warp-uniform) are added after the reduction
+      // lane partials are reduced; run (warp-uniform) is added after it
 #pragma unroll
       for (int s = 0; s < NS; ++s) tot[C::smap(s)] = sacc[s];
-      warp_sum_some<M>(tot);
-#pragma unroll
-      for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc_add(drun[d], tot[C::dmap(d)]);
+      warp_sum_set<M, WIDE>(tot);
 #pragma unroll
       for (int s = 0; s < NS; ++s) tot[C::smap(s)] = acc_add(run[s], tot[C::smap(s)]);
       // the ends after the last nonzero of the range see the warp totals
@@ -678,7 +618,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           A pref[NS > 0 ? NS : 1];
 #pragma unroll
           for (int s = 0; s < NS; ++s) pref[s] = acc_add_v(sacc[s], (int64_t)row <= next_end ? sv[s] : T(0));
-          warp_sum_some<(NS > 0 ? NS : 1)>(pref);
+          warp_sum_set<(NS > 0 ? NS : 1), WIDE>(pref);
           if (lane == 0)
 #pragma unroll
             for (int s = 0; s < NS; ++s) rec[(size_t)ec.kn * M + C::smap(s)] = pref[s];
@@ -711,16 +651,13 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
 #pragma unroll
       for (int s = 0; s < NS; ++s) tot[C::smap(s)] = sacc[s];  // lane partials, reduced below
       // warp totals, then the ends after the last nonzero of the range see them
-      warp_sum_some<M>(tot);
+      warp_sum_set<M, WIDE>(tot);
       for (int k = ec.kn + lane; k < pf.k_hi; k += 32)
 #pragma unroll
         for (int s = 0; s < NS; ++s) rec[(size_t)k * M + C::smap(s)] = tot[C::smap(s)];
     }
   } else {
-    warp_sum_some<M>(tot);
-    if constexpr (MULTI)
-#pragma unroll
-      for (int d = 0; d < ND; ++d) tot[C::dmap(d)] = acc_add(drun[d], tot[C::dmap(d)]);
+    warp_sum_set<M, WIDE>(tot);
   }
 }
 

@@ -48,7 +48,7 @@ template <int MODEL, int LAYOUT>
 struct GCfg {
   static constexpr int NT = 512;
   static constexpr int MINB = 2;
-  static constexpr int U = (MODEL == 1 && LAYOUT == 1) ? 1 : (MODEL == 1 ? 2 : 4);
+  static constexpr int U = (MODEL == 1 && LAYOUT == 1) ? 1 : (MODEL == 1 || LAYOUT == 1 ? 2 : 4);
   static constexpr int SR = 4;
 };
 constexpr int kTransThreads = 256;
@@ -657,12 +657,17 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   ct.blockDim = dim3(kTransThreads);
   // batched fits: Cox only (the censoring weights of Fine-Gray would have
   // to be re-estimated on each training set)
-  // Cox passes whose warps hold two group ends or more on average take the
-  // many-ends form of the row pass
+  // The many-ends form of the row pass where warps hold two group ends or
+  // more on average, and where they hold few rows: the ends are then few on
+  // average but crowd into the warps of the latest times, whose way through
+  // them one after another is the pass (us a coordinate, the plain and the
+  // many-ends form: 20.9 and 18.2 at 500,009 x 24 dense, 20.1 and 19.1 at
+  // 400,000 x 100 sparse; at 10^7 the latter costs more, 20.2 and 21.2).
+  const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps, few_rows = P.nfit == 0 && P.wpw <= 16;
   auto kp = k_pass<MODEL, LAYOUT, T, false, false>;
   auto kt = k_trans<MODEL, LAYOUT, T, false>;
   if constexpr (MODEL == 0) {
-    const bool multi = P.pass_form == 2 || (P.pass_form == 0 && (int64_t)P.K >= 2 * (int64_t)P.nwarps);
+    const bool multi = P.pass_form == 2 || (P.pass_form == 0 && (many || few_rows));
     if (P.nfit > 0) {
       kp = multi ? k_pass<MODEL, LAYOUT, T, true, true> : k_pass<MODEL, LAYOUT, T, true, false>;
       if constexpr (LAYOUT == 0 && sizeof(T) == 4) {
@@ -677,6 +682,7 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
       kp = k_pass<MODEL, LAYOUT, T, false, true>;
     }
   } else {
+    if (many || few_rows) kp = k_pass<MODEL, LAYOUT, T, false, true>;
     if (P.nfit > 0) {
       cudaGraph_t junk = nullptr;
       cudaStreamEndCapture(cs, &junk);

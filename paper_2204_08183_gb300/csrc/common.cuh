@@ -194,6 +194,13 @@ __device__ __forceinline__ void warp_sum_some(A (&v)[N]) {
   }
 }
 
+// warp_sum_n where registers are plentiful (WIDE), else warp_sum_some.
+template <int N, bool WIDE, typename A>
+__device__ __forceinline__ void warp_sum_set(A (&v)[N]) {
+  if constexpr (WIDE) warp_sum_n<N>(v);
+  else warp_sum_some<N>(v);
+}
+
 // Sums of N values over the 32 lanes (N a power of two, 2..32) by recursive
 // halving: at distance d = 16, 8, ... each lane keeps half of its values
 // and adds the partner's copy of that half, so N values cost N - 1 + 5 -

@@ -39,3 +39,24 @@ def test_many_ends(lib, n, kind, layout, density, precision):
     f64 = precision == "f64"
     np.testing.assert_allclose(b, ref["beta"], rtol=0, atol=1e-9 if f64 else 1e-5)
     assert i["loglik"] == pytest.approx(ref["loglik"], rel=1e-10 if f64 else 1e-6)
+
+
+# few rows a warp: the same form although the groups are fewer than the warps
+@pytest.mark.parametrize("precision", ["f32c", "f64"])
+@pytest.mark.parametrize("layout", ["csc", "dense"])
+@pytest.mark.parametrize("model", ["cox", "fg"])
+@pytest.mark.parametrize("n", [2, 31, 4099, 160_003])
+def test_few_rows_a_warp(lib, n, model, layout, precision):
+    competing = 0.25 if model == "fg" else 0.0
+    if layout == "csc":
+        d = small_csc(n, 2, seed=n + 1, density=0.3, n_times=200, competing=competing)
+    else:
+        d = synth.cohort_small(n, 2, n + 1, n_times=200, competing_frac=competing)
+    d["status"][-1] = 1
+    fit = binding.cox_fit if model == "cox" else binding.fg_fit
+    kw = dict(penalty="l2", lam=1.0, precision=precision, tol=0.0, max_sweeps=2, flags=PAIR)
+    b, i, _ = fit(survdata(d), **kw)
+    ref = oracle.ccd_fit(model, d["time"], d["status"], oracle_X(d), "l2", 1.0, tol=0.0, max_sweeps=2)
+    f64 = precision == "f64"
+    np.testing.assert_allclose(b, ref["beta"], rtol=0, atol=1e-9 if f64 else 1e-5)
+    assert i["loglik"] == pytest.approx(ref["loglik"], rel=1e-10 if f64 else 1e-6, abs=1e-12 if f64 else 1e-6)
