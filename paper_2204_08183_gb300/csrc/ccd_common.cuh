@@ -231,20 +231,26 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
     for (int d = 0; d < ND; ++d) acc_zero(acc[d]);
     EndCursor ec{pf.k_lo, pf.k_hi, pf.k_lo, pf.kreg};
     int64_t next_end = MULTI ? 0 : ec.pos(P.gend);
-    // many-ends form: the ends among a lane's rows of each chunk row u (bit q:
-    // its row q ends a group), from the end masks.
-    // Every lane writes the records of its own rows, and in the sparse part
-    // below an end a lane: the work of a tile does not grow with its ends.
-    // (One end after another by the whole warp bounded the pass by its issue
-    // slots: a fit of 333,331 subjects with hardly any ties took 22.5 ms and
-    // takes 7.1; the cross-validated path at n = 10^6, 15 ends a warp, 671 ms
-    // and 576.)
-    uint32_t nib[U];
+    // Many-ends form: a lane holds U VEC consecutive rows of a tile, so one
+    // scan over the lanes serves them all; nib: which of them end a group
+    // (bit i: its row i), from the end masks.  Every lane writes the records
+    // of its own rows, and in the sparse part below an end a lane: the work of
+    // a tile does not grow with its ends.  (One end after another by the whole
+    // warp bounded the pass by its issue slots: a fit of 333,331 subjects with
+    // hardly any ties took 22.5 ms and takes 7.1; the cross-validated path at
+    // n = 10^6, 15 ends a warp, 671 ms and 567.)
+    constexpr int LR = U * VEC;   // divides 32: a lane's rows lie in one mask word
+    static_assert(!MULTI || 32 % LR == 0, "rows of a lane");
+    uint32_t nib = 0u;
     bool acc_dirty = false;   // acc holds partials of several lanes (else lane 0's alone)
     const T* xcol = LAYOUT == 1 ? reinterpret_cast<const T*>(P.X) + (size_t)j * P.ld : nullptr;
 
     // loads of one tile from global memory (16-byte loads; the last partial
     // tile element by element)
+    // first row of chunk row u of the lane
+    auto row_of = [&](int64_t t0, int u) -> int64_t {
+      return MULTI ? t0 + (int64_t)lane * (U * VEC) + u * VEC : t0 + (int64_t)(lane + 32 * u) * VEC;
+    };
     auto load_tile = [&](int64_t t0, T (&ev)[U][VEC], T (&xv)[U][VEC], T (&wv)[U][VEC]) {
       if constexpr (LAYOUT == 1 && sizeof(T) == 4) {
         if (xq) {
@@ -259,7 +265,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
           };
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
+            const int64_t r = row_of(t0, u);
             if (r + VEC <= row_hi) {
               float xx[VEC];
               float2 qq[VEC];
@@ -305,7 +311,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
+        const int64_t r = row_of(t0, u);
         if (r + VEC <= row_hi) {
           ld4_hint(e + r, keep, ev[u]);
           if (LAYOUT == 1) ld4_hint(xcol + r, strm, xv[u]);
@@ -322,15 +328,10 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
       }
     };
     // One tile.  Lane l holds chunks c = 32 u + l of VEC consecutive rows
-    // (rows t0 + VEC c .. + VEC - 1); chunk sums are pairwise within the
-    // lane and feed the running sums.
-    //   One dense component (CSC layouts of Cox): the lane's share of the
-    //   rows up to an end in chunk c* is its chunks before c* plus chunk c*
-    //   up to the end.  A tile with one end reduces (running sum + share)
-    //   in one float-float tree; a tile with several reduces the running
-    //   sums once and each end's shares in an FP32 tree.
-    //   Several components (register pressure): every end reduces the
-    //   running sums plus the tile's rows up to the end in one tree.
+    // (rows t0 + VEC c .. + VEC - 1; in the many-ends form the U chunks after
+    // one another); chunk sums are pairwise within the lane and feed the
+    // running sums.  Outside the many-ends form every end reduces the running
+    // sums plus the tile's rows up to the end in one tree.
     auto chunk_sum = [&](int d, const T (&ev)[U][VEC], const T (&xv)[U][VEC], const T (&wv)[U][VEC], int u) {
       const T a0 = dense_comp<MODEL, LAYOUT, T>(d, ev[u][0], xv[u][0], wv[u][0]);
       const T a1 = dense_comp<MODEL, LAYOUT, T>(d, ev[u][1], xv[u][1], wv[u][1]);
@@ -348,66 +349,47 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
       if constexpr (MULTI) {
         // A tile without an end adds to the lane partials.  One with ends takes
         // their sum (from lane 0 alone where the previous tile left it there:
-        // acc_dirty is false) and one FP32 lane scan per chunk row u, which gives
-        // every chunk its tile-relative exclusive prefix; a lane adds the rows
-        // of its chunk up to an end and writes the record.  One component at a
-        // time: the scans of a tile need few registers.
-        bool any = false;
-#pragma unroll
-        for (int u = 0; u < U; ++u) any |= nib[u] != 0u;
-        if (!__any_sync(0xffffffffu, any)) {
-#pragma unroll
-          for (int d = 0; d < ND; ++d) {
-            T su[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) su[u] = chunk_sum(d, ev, xv, wv, u);
-#pragma unroll
-            for (int s = 1; s < U; s <<= 1)
-#pragma unroll
-              for (int u = 0; u + s < U; u += 2 * s) su[u] += su[u + s];
-            acc[d] = acc_add_v(acc[d], su[0]);
-          }
-          acc_dirty = true;
-          return;
-        }
-        if (acc_dirty) warp_sum_set<ND, WIDE>(acc);
+        // acc_dirty is false) and an exclusive lane scan of the lanes' totals in
+        // twice the working precision, and a lane walks its rows up to each end.
+        // One component at a time: the scans of a tile need few registers.
+        const bool any = __any_sync(0xffffffffu, nib != 0u);
+        if (any && acc_dirty) warp_sum_set<ND, WIDE>(acc);
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
-          const A before = acc_dirty ? acc[d] : shfl_idx(acc[d], 0);   // the warp's rows before the tile
-          T ex[U];
+          T su[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) ex[u] = chunk_sum(d, ev, xv, wv, u);
+          for (int u = 0; u < U; ++u) su[u] = chunk_sum(d, ev, xv, wv, u);
 #pragma unroll
-          for (int dd = 1; dd < 32; dd <<= 1)
+          for (int s = 1; s < U; s <<= 1)
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const T t = __shfl_up_sync(0xffffffffu, ex[u], dd);
-              if (lane >= dd) ex[u] += t;
-            }
-          T pu = T(0);
+            for (int u = 0; u + s < U; u += 2 * s) su[u] += su[u + s];
+          if (!any) {
+            acc[d] = acc_add_v(acc[d], su[0]);
+            continue;
+          }
+          A before = acc_dirty ? acc[d] : shfl_idx(acc[d], 0);   // the warp's rows before the tile
+          A all;
+          const A ex = lane_scan_exclusive(su[0], lane, all);
+          acc_zero(acc[d]);
+          if (lane == 0) acc[d] = acc_add(before, all);
+          if (nib) {
+            before = acc_add(before, ex);
+            const int64_t r = row_of(t0, 0);
+            int k = P.wordk[r >> 5] + __popc(P.endw[r >> 5] & ((1u << (r & 31)) - 1u));   // its first end
+            T in = T(0);
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const T tu = __shfl_sync(0xffffffffu, ex[u], 31);
-            const T t = __shfl_up_sync(0xffffffffu, ex[u], 1);
-            if (nib[u]) {
-              T in = lane == 0 ? T(0) : t;
-              const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
-              int k = P.wordk[r >> 5] + __popc(P.endw[r >> 5] & ((1u << (r & 31)) - 1u));   // its first end
+            for (int u = 0; u < U; ++u)
 #pragma unroll
               for (int q = 0; q < VEC; ++q) {
                 in += dense_comp<MODEL, LAYOUT, T>(d, ev[u][q], xv[u][q], wv[u][q]);
-                if (nib[u] >> q & 1u) {
-                  rec[(size_t)k * M + C::dmap(d)] = acc_add_v(before, pu + in);
+                if (nib >> (u * VEC + q) & 1u) {
+                  rec[(size_t)k * M + C::dmap(d)] = acc_add_v(before, in);
                   ++k;
                 }
               }
-            }
-            pu += tu;
           }
-          acc_zero(acc[d]);
-          if (lane == 0) acc[d] = acc_add_v(before, pu);
         }
-        acc_dirty = false;
+        acc_dirty = !any;
       } else {
         while (next_end < t_end) {
           A pref[ND];
@@ -418,7 +400,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
             for (int u = 0; u < U; ++u)
 #pragma unroll
               for (int q = 0; q < VEC; ++q) {
-                const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC + q;
+                const int64_t r = row_of(t0, u) + q;
                 if (r <= next_end) part += dense_comp<MODEL, LAYOUT, T>(d, ev[u][q], xv[u][q], wv[u][q]);
               }
             pref[d] = acc_add_v(acc[d], part);
@@ -447,11 +429,8 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
     for (int64_t t0 = row_lo; t0 < row_hi; t0 += TILE) {
       T ev[U][VEC], xv[U][VEC], wv[U][VEC];
       if constexpr (MULTI) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int64_t r = t0 + (int64_t)(lane + 32 * u) * VEC;
-          nib[u] = r < row_hi ? P.endw[r >> 5] >> (int)(r & 31) & ((1u << VEC) - 1u) : 0u;
-        }
+        const int64_t r = row_of(t0, 0);
+        nib = r < row_hi ? P.endw[r >> 5] >> (int)(r & 31) & (uint32_t)((1ull << LR) - 1ull) : 0u;
       }
       load_tile(t0, ev, xv, wv);
       tile(t0, ev, xv, wv);

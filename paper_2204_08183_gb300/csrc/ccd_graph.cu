@@ -658,12 +658,14 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   // batched fits: Cox only (the censoring weights of Fine-Gray would have
   // to be re-estimated on each training set)
   // The many-ends form of the row pass where warps hold two group ends or
-  // more on average, and where they hold few rows: the ends are then few on
-  // average but crowd into the warps of the latest times, whose way through
-  // them one after another is the pass (us a coordinate, the plain and the
-  // many-ends form: 20.9 and 18.2 at 500,009 x 24 dense, 20.1 and 19.1 at
-  // 400,000 x 100 sparse; at 10^7 the latter costs more, 20.2 and 21.2).
-  const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps, few_rows = P.nfit == 0 && P.wpw <= 16;
+  // more on average, and, with more than one dense component, where they hold
+  // few rows: the ends are then few on average but crowd into the warps of the
+  // latest times, whose way through them one after another is the pass (us a
+  // coordinate, the plain and the many-ends form: 20.9 and 18.2 at 500,009 x
+  // 24 dense Cox, 31.8 and 26.7 at 200,003 x 40 sparse Fine-Gray; at 5 x 10^6
+  // x 50 dense Fine-Gray the plain form, 49.0 against 52.4).
+  const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps;
+  const bool few_rows = P.nfit == 0 && P.wpw <= 16 && (Cfg<MODEL, LAYOUT, T>::ND > 1 || sizeof(T) == 8);
   auto kp = k_pass<MODEL, LAYOUT, T, false, false>;
   auto kt = k_trans<MODEL, LAYOUT, T, false>;
   if constexpr (MODEL == 0) {

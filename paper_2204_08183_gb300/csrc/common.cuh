@@ -273,6 +273,36 @@ __device__ __forceinline__ void warp_scan_n(double (&v)[N], int lane) {
   }
 }
 
+// Exclusive scan over the lanes of one FP32 value each, in float-float (the
+// rounding error of every addition is carried, renormalised once at the end),
+// or of one FP64 value each; `all` gets the total.
+__device__ __forceinline__ ff lane_scan_exclusive(float v, int lane, ff& all) {
+  ff s = {v, 0.f};
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const ff u = shfl_up(s, d);
+    if (lane >= d) {
+      const ff t = two_sum(u.hi, s.hi);
+      s.lo = __fadd_rn(__fadd_rn(u.lo, s.lo), t.lo);
+      s.hi = t.hi;
+    }
+  }
+  s = fast_two_sum(s.hi, s.lo);
+  all = shfl_idx(s, 31);
+  const ff ex = shfl_up(s, 1);
+  return lane == 0 ? ff_zero() : ex;
+}
+__device__ __forceinline__ double lane_scan_exclusive(double v, int lane, double& all) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const double u = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += u;
+  }
+  all = __shfl_sync(0xffffffffu, v, 31);
+  const double ex = __shfl_up_sync(0xffffffffu, v, 1);
+  return lane == 0 ? 0.0 : ex;
+}
+
 // Inclusive scan over lanes (Hillis-Steele, fixed shape).
 static __device__ __noinline__ ff warp_scan_ff(ff v, int lane) {
 #pragma unroll
