@@ -6,7 +6,7 @@
 //               each warp applies eta += x_q * step and e = exp(eta) to its
 //               own rows, then runs the row pass (step 2) of coordinate j
 //               over those rows and the CTA publishes its warp totals and its
-//               aggregate (the latter in kRep replicas).
+//               aggregate.
 //   k_trans(j)  every CTA sums the aggregates of the CTAs before it (its
 //               exclusive prefix) in a fixed order, transforms its group ends
 //               (steps 3-4) and publishes three partial sums.  The last CTA
@@ -172,10 +172,10 @@ __global__ void __launch_bounds__(GCfg<MODEL, LAYOUT>::NT, GCfg<MODEL, LAYOUT>::
       if (lane < WPC && !keep) P.wt[(size_t)m * P.nwarps + c * WPC + lane] = pack8(ex);
       v[m] = shfl_idx(v[m], WPC - 1);
     }
-    if (lane < kRep)
+    if (lane == 0)
 #pragma unroll
       for (int m = 0; m < M; ++m)
-        if (!(LAYOUT == 0 && !dense && (m == 0 || m == 3))) P.agg[((size_t)lane * M + m) * G + c] = pack8(v[m]);
+        if (!(LAYOUT == 0 && !dense && (m == 0 || m == 3))) P.agg[(size_t)m * G + c] = pack8(v[m]);
   }
 }
 
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kTransThreads) k_trans(const __grid_constant__
     lv = load_line(ctl, c);
     s_stopped = lv.stop;
   }
-  const uint64_t* agg = P.agg + (size_t)(c % kRep) * M * G;
+  const uint64_t* agg = P.agg;
   // warp of this thread's group end (relative to the CTA); the pass kernel
   // stored each warp's offset inside the CTA in wt
   const int wl = (one_end && tid < nends) ? (int)((kge >> 5) / P.wpw) - c * WPC : (tid < WPC ? tid : 0);
@@ -426,16 +426,26 @@ __global__ void __launch_bounds__(kTransThreads) k_trans(const __grid_constant__
 // first end's group table entries before the wait: the line was written by
 // the previous coordinate's transform, which finished before this
 // coordinate's pass kernel passed its own wait.
-constexpr int kBtNT = 512;
-constexpr int kBtWarps = kBtNT / 32;
+//
+// Threads: it is a chain of float-float scans and reductions, and several
+// warps on a scheduler lengthen every one of them, so the block has one warp
+// per scheduler and the ends more CTAs, as long as a thread then gets one end
+// (us a coordinate, 512 and 128 threads: 27.1 and 24.8 for 1000 ends of
+// Fine-Gray, 20.5 and 18.5 for 3650 of Cox; 28.6 and 39.0 for 310,400, where
+// 128 threads on every SM walk 16 ends each).
+constexpr int kBtSmall = 128, kBtLarge = 512;
+constexpr int kBtMaxG = 384;   // pass CTAs
+constexpr int kBtMaxCtas = 152;
+inline int btrans_threads(int K) { return K <= kBtSmall * kBtMaxCtas ? kBtSmall : kBtLarge; }
 
-template <int MODEL, int LAYOUT, typename T>
+template <int MODEL, int LAYOUT, typename T, int kBtNT>
 __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ CcdParams P, int j) {
   using A = typename AccOf<T>::type;
   constexpr int M = MODEL == 0 ? 3 : 6;
-  __shared__ A s_T[kBtNT][M];
+  constexpr int kBtWarps = kBtNT / 32, kAgg = kBtNT == kBtSmall ? 3 : 1;
+  __shared__ A s_T[kBtNT * kAgg][M];
   __shared__ A s_w[kBtWarps][M];
-  __shared__ A s_tot3[3];
+  __shared__ A s_all[M];   // grand totals (Fine-Gray: the suffix components)
   __shared__ A s_red[kBtWarps][3];
   __shared__ int s_last, s_stop;
   __shared__ double s_lin[2];
@@ -448,6 +458,17 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
   if (tid == 0) {
     lv = load_line(ctl, c2);
     s_stop = lv.stop;
+  }
+  // the next coordinate's scalars for the control line (warp 3; last written a
+  // sweep ago, or, for two coordinates, two transforms ago)
+  static_assert(kBtWarps >= 4 && kBtNT * kAgg >= kBtMaxG, "three warps sum the partials, the fourth does the rest");
+  double nx[4] = {0.0, 0.0, 0.0, 0.0};
+  if (w == 3 && lane == 0) {
+    const int jn = j + 1 < P.p ? j + 1 : 0;
+    nx[0] = __ldcg(P.beta + jn);
+    nx[1] = __ldcg(P.width + jn);
+    nx[2] = P.pen[jn];
+    nx[3] = P.dTx[jn];
   }
   const int stride = G2 * kBtNT;
   const int k0 = c2 * kBtNT + tid;
@@ -469,51 +490,8 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
   }
   pdl_wait();
 
-  // exclusive prefix over the pass CTAs of their aggregates, fixed order
-  {
-    const uint64_t* agg = P.agg + (size_t)(c2 % kRep) * M * G;
-    A v[M], incl[M];
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      acc_zero(v[m]);
-      if (tid < G) v[m] = unpack8<A>(__ldcg(agg + (size_t)m * G + tid));
-      incl[m] = v[m];
-    }
-    warp_scan_n<M>(incl, lane);
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const A ex = shfl_up(incl[m], 1);
-      if (lane == 0) acc_zero(v[m]);
-      else v[m] = ex;
-    }
-    if (lane == 31)
-#pragma unroll
-      for (int m = 0; m < M; ++m) s_w[w][m] = incl[m];
-    __syncthreads();
-    if (w == 0) {
-      A t[M];
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        acc_zero(t[m]);
-        if (lane < kBtWarps) t[m] = s_w[lane][m];
-      }
-      warp_scan_n<M>(t, lane);
-      __syncwarp();
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const A ex = shfl_up(t[m], 1);
-        const A all = shfl_idx(t[m], kBtWarps - 1);
-        if (lane < kBtWarps) {
-          if (lane == 0) acc_zero(s_w[lane][m]);
-          else s_w[lane][m] = ex;
-        }
-        if (MODEL == 1 && m >= 3 && lane == 0) s_tot3[m % 3] = all;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < M; ++m) s_T[tid][m] = acc_add(s_w[w][m], v[m]);
-  }
+  // prefixes of the pass CTAs' aggregates
+  scan_aggregates<kBtNT, kAgg, M, A>(P.agg, G, s_T, s_w, MODEL == 1 ? s_all : nullptr);
   __syncthreads();
 
   // steps 3-4 at the group ends
@@ -525,7 +503,7 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     acc_zero(tot3[i]);
-    if (MODEL == 1) tot3[i] = s_tot3[i];
+    if (MODEL == 1) tot3[i] = s_all[(3 + i) % M];
   }
   const A* rec = reinterpret_cast<const A*>(P.rec);
   for (int k = k0; k < P.K; k += stride) {
@@ -599,19 +577,18 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
     A r[1] = {acc};
     warp_sum_n<1>(r);
     if (lane == 0) s_red[0][w] = r[0];
-  } else if (w == 3 && eval) {
-    double lin, pen;
-    warp_lin_pen(P, -1, 0.0, lin, pen);
-    if (lane == 0) {
-      s_lin[0] = lin;
-      s_lin[1] = pen;
+  } else if (w == 3) {
+    if (eval) {
+      double lin, pen;
+      warp_lin_pen(P, -1, 0.0, lin, pen);
+      if (lane == 0) {
+        s_lin[0] = lin;
+        s_lin[1] = pen;
+      }
     }
-  } else if (w == 4 && lane == 0) {
-    const int jn = j + 1 < P.p ? j + 1 : 0;
-    s_next[0] = __ldcg(P.beta + jn);
-    s_next[1] = __ldcg(P.width + jn);
-    s_next[2] = P.pen[jn];
-    s_next[3] = P.dTx[jn];
+    if (lane == 0)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s_next[i] = nx[i];
   }
   __syncthreads();
   if (w == 0)
@@ -619,8 +596,11 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
                  acc_to_d(s_red[0][2]), s_next);
 }
 
-// CTAs of the balanced transform: about one group end a thread, 4 to 152.
-inline int btrans_ctas(int K) { return std::max(4, std::min(152, (K + kBtNT - 1) / kBtNT)); }
+// CTAs of the balanced transform: about one group end a thread.
+inline int btrans_ctas(int K) {
+  const int nt = btrans_threads(K);
+  return std::max(4, std::min(kBtMaxCtas, (K + nt - 1) / nt));
+}
 
 // Grid of the pass kernel: as many CTAs per SM (up to MINB) as fit.
 template <int MODEL, int LAYOUT, typename T>
@@ -692,12 +672,11 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
       return cudaErrorInvalidValue;
     }
   }
-  // single fits: the balanced transform (one pass-CTA aggregate per thread
-  // in its scan, so up to kBtNT pass CTAs)
-  if (P.nfit == 0 && P.G <= kBtNT) {
-    kt = k_btrans<MODEL, LAYOUT, T>;
+  // single fits: the balanced transform (up to kBtMaxG pass CTAs)
+  if (P.nfit == 0 && P.G <= kBtMaxG) {
+    kt = btrans_threads(P.K) == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;
     ct.gridDim = dim3(btrans_ctas(P.K));
-    ct.blockDim = dim3(kBtNT);
+    ct.blockDim = dim3(btrans_threads(P.K));
   }
   cudaError_t lst = cudaSuccess;
   for (int j = 0; j < P.p && lst == cudaSuccess; ++j) {

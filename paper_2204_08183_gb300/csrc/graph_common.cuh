@@ -38,6 +38,72 @@ __device__ __forceinline__ LineView load_line(const GraphCtl* ctl, int c) {
   return v;
 }
 
+// Exclusive prefixes of the pass CTAs' aggregates agg [NV][G] into s_T (and
+// their totals into s_all, if given), in a fixed order, by a block of NT
+// threads that takes AGG consecutive aggregates a thread (G <= NT AGG).  The
+// caller synchronises the block before reading them; s_w is scratch.
+template <int NT, int AGG, int NV, typename A>
+__device__ __forceinline__ void scan_aggregates(const uint64_t* agg, int G, A (*s_T)[NV], A (*s_w)[NV], A* s_all) {
+  constexpr int W = NT / 32;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  A v[AGG][NV], t[NV];
+#pragma unroll
+  for (int a = 0; a < AGG; ++a) {
+    const int q = tid * AGG + a;
+#pragma unroll
+    for (int m = 0; m < NV; ++m) {
+      acc_zero(v[a][m]);
+      if (q < G) v[a][m] = unpack8<A>(__ldcg(agg + (size_t)m * G + q));
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < NV; ++m) {
+    t[m] = v[0][m];
+#pragma unroll
+    for (int a = 1; a < AGG; ++a) t[m] = acc_add(t[m], v[a][m]);
+  }
+  warp_scan_n<NV>(t, lane);
+  if (lane == 31)
+#pragma unroll
+    for (int m = 0; m < NV; ++m) s_w[w][m] = t[m];
+  __syncthreads();
+  if constexpr (W > 4) {   // many warps: their totals by one more scan
+    if (w == 0) {
+      A u[NV];
+#pragma unroll
+      for (int m = 0; m < NV; ++m) {
+        acc_zero(u[m]);
+        if (lane < W) u[m] = s_w[lane][m];
+      }
+      warp_scan_n<NV>(u, lane);
+      __syncwarp();
+#pragma unroll
+      for (int m = 0; m < NV; ++m) {
+        A ex = shfl_up(u[m], 1);
+        if (lane == 0) acc_zero(ex);
+        if (lane < W) s_w[lane][m] = ex;
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int m = 0; m < NV; ++m) {
+    A run = shfl_up(t[m], 1);
+    if (lane == 0) acc_zero(run);
+    if constexpr (W > 4) {
+      run = acc_add(s_w[w][m], run);
+    } else {
+      for (int q = w - 1; q >= 0; --q) run = acc_add(s_w[q][m], run);
+    }
+#pragma unroll
+    for (int a = 0; a < AGG; ++a) {
+      s_T[tid * AGG + a][m] = run;
+      if (s_all || a + 1 < AGG) run = acc_add(run, v[a][m]);
+    }
+    if (s_all && tid == NT - 1) s_all[m] = run;
+  }
+}
+
 // Per-fit parameters of a batched launch, read once per CTA into shared
 // memory (the table is written before the fit starts: it may be read before
 // the wait on the previous kernel).

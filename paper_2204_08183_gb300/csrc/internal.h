@@ -76,7 +76,7 @@ struct CcdParams {
 
   // per-coordinate kernel pair only (null for the persistent kernel)
   uint64_t* wt;          // [M][nwarps] warp totals of the last pass (8-byte payload words)
-  uint64_t* agg;         // [kRep][M][G] CTA aggregates of the last pass, replicated
+  uint64_t* agg;         // [M][G] CTA aggregates of the last pass
   struct GraphCtl* gctl; // fit state carried between kernels
   unsigned* done_count;  // fits that have stopped (the host polls it)
 

@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kSnPassThreads, 2) k_sn_den_a(const __grid_con
     if (lane == 0) acc_zero(ex);
     if (lane < WPC) P.wt[c * WPC + lane] = pack8(ex);
     const A t = shfl_idx(v[0], WPC - 1);
-    if (lane < kRep) P.agg[(size_t)lane * G + c] = pack8(t);
+    if (lane == 0) P.agg[c] = pack8(t);
   }
 }
 
@@ -205,8 +205,8 @@ __global__ void __launch_bounds__(kSnThreads) k_sn_den_b(const __grid_constant__
   const int kc_lo = P.wk0[c * WPC], kc_hi = P.wk0[(c + 1) * WPC];
   pdl_wait();
   if (!sn_rebuilt(P, c, &s_flag)) return;
-  // aggregate of the CTAs before c (replica c mod kRep), fixed order
-  const uint64_t* agg = P.agg + (size_t)(c % kRep) * G;
+  // aggregate of the CTAs before c, fixed order
+  const uint64_t* agg = P.agg;
   ff pre = ff_zero();
   for (int qc = tid; qc < c; qc += kSnThreads) pre = ff_add(pre, unpack8<ff>(__ldcg(agg + qc)));
   const ff T_c = block_sum_ff(pre, s_wf);

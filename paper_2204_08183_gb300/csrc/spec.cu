@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kSpNT, 2) k_spass(const __grid_constant__ CcdP
     if (lane == 0) ex = ff_zero();
     if (lane < WPC) P.wt[(size_t)m * P.nwarps + c * WPC + lane] = pack8(ex);
     const ff t = shfl_idx(incl, WPC - 1);
-    if (lane < kRep) P.agg[((size_t)lane * R + m) * G + c] = pack8(t);
+    if (lane == 0) P.agg[(size_t)m * G + c] = pack8(t);
   }
 }
 
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kStNT) k_strans(const __grid_constant__ CcdPar
 
   // prefix of the aggregates of the CTAs before c, fixed order
   {
-    const uint64_t* agg = P.agg + (size_t)(c % kRep) * R * G;
+    const uint64_t* agg = P.agg;
     ff t[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) t[r] = ff_zero();
@@ -527,8 +527,12 @@ struct IpCfg {
   // 64-register cap of two CTAs per SM and measured 2 % slower)
   static constexpr int SR = 1;
 };
-constexpr int kItNT = 512;   // transform kernel threads
+// Transform kernel threads: the K B items of a batch want more threads than
+// the ends of one coordinate (us a row pass at n = 10^7, p = 100 with 128
+// threads on more CTAs: 15 % more than with 512).
+constexpr int kItNT = 512;
 constexpr int kItWarps = kItNT / 32;
+constexpr int kItAgg = 1;
 
 // Position of the warp's group end k (k warp-uniform): lane registers for
 // the first 32, a broadcast load beyond.
@@ -722,8 +726,8 @@ __global__ void __launch_bounds__(kSpNT, 2) k_ipass(const __grid_constant__ CcdP
 template <int B>
 __global__ void __launch_bounds__(kItNT, 1) k_itrans(const __grid_constant__ CcdParams P, int slot) {
   constexpr int R = IpCfg<B>::R, NP = IpCfg<B>::NP, NPP = IpCfg<B>::NPP;
-  __shared__ ff s_T[kItNT][R];           // exclusive prefix of the pass CTAs' aggregates (G <= kItNT)
-  __shared__ ff s_w[kItWarps][R];        // warp totals of that scan, then their exclusive prefix
+  __shared__ ff s_T[kItNT * kItAgg][R];       // exclusive prefix of the pass CTAs' aggregates
+  __shared__ ff s_w[kItWarps][R];
   __shared__ ff s_red[kItWarps][NP];
   __shared__ ff s_tot[NP];
   __shared__ int s_stop, s_j0, s_last;
@@ -765,40 +769,8 @@ __global__ void __launch_bounds__(kItNT, 1) k_itrans(const __grid_constant__ Ccd
   if (w == 0) ci = load_coord(P, j0, nb);
   pdl_wait();
 
-  // exclusive prefix over the pass CTAs of their aggregates, fixed order
-  {
-    ff v[R];
-#pragma unroll
-    for (int m = 0; m < R; ++m) v[m] = tid < G ? unpack8<ff>(__ldcg(P.agg + (size_t)m * G + tid)) : ff_zero();
-    ff incl[R];
-#pragma unroll
-    for (int m = 0; m < R; ++m) incl[m] = v[m];
-    warp_scan_n<R>(incl, lane);
-#pragma unroll
-    for (int m = 0; m < R; ++m) {
-      ff ex = shfl_up(incl[m], 1);
-      v[m] = lane == 0 ? ff_zero() : ex;   // exclusive within the warp
-    }
-    if (lane == 31)
-#pragma unroll
-      for (int m = 0; m < R; ++m) s_w[w][m] = incl[m];
-    __syncthreads();
-    if (w == 0) {
-      ff t[R];
-#pragma unroll
-      for (int m = 0; m < R; ++m) t[m] = lane < kItWarps ? s_w[lane][m] : ff_zero();
-      warp_scan_n<R>(t, lane);
-      __syncwarp();
-#pragma unroll
-      for (int m = 0; m < R; ++m) {
-        const ff ex = shfl_up(t[m], 1);
-        if (lane < kItWarps) s_w[lane][m] = lane == 0 ? ff_zero() : ex;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < R; ++m) s_T[tid][m] = ff_add(s_w[w][m], v[m]);
-  }
+  // prefixes of the pass CTAs' aggregates
+  scan_aggregates<kItNT, kItAgg, R, ff>(P.agg, G, s_T, s_w, nullptr);
   __syncthreads();
 
   // G_k of the batch's columns at the group ends (steps 3-4); column 0's
@@ -912,7 +884,7 @@ cudaError_t capture_spec(const CcdParams& P, int S, bool pdl, cudaStream_t cs, c
   // indicator columns: the lockstep walks and the ranged transform
   const bool ind = P.values == nullptr;
   if (ind) {
-    if (P.G > kItNT) return cudaErrorInvalidValue;   // the transform scans one aggregate per thread
+    if (P.G > kItNT * kItAgg) return cudaErrorInvalidValue;   // the transform scans kItAgg aggregates a thread
     ct.gridDim = dim3(itrans_ctas(P.K, B));
     ct.blockDim = dim3(kItNT);
   }
