@@ -125,8 +125,9 @@ typedef struct surv_opts {
  * device memory, bounded waits) instead of the default schedule of two
  * kernels per coordinate replayed as a CUDA graph, one replay per sweep.
  * Both schedules compute the same quantities in the same order of
- * coordinates; this flag exists to compare them.  loglik_grad_hess always
- * uses the persistent kernel. */
+ * coordinates; this flag exists to compare them.  (Without flags, cohorts
+ * that one thread-block cluster holds run in one launch on that cluster;
+ * loglik_grad_hess uses it too, and the persistent kernel for larger ones.) */
 #define SURV_FLAG_PERSISTENT 2
 /* cox_cv_path only, with ctas_per_fit = 0: time one sweep of the batched
  * schedule for each of a few CTA-per-fit counts around the default and, for

@@ -346,21 +346,32 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   const int M = model == SURV_COX ? 3 : 6;
   using W = surv_workspace;
 
-  // fits run as per-coordinate kernels replayed in a CUDA graph; the single
-  // evaluation of loglik_grad_hess, the stall test and SURV_FLAG_PERSISTENT
-  // use the persistent kernel
-  const bool graph = single_j < 0 && (o.flags & (SURV_FLAG_TEST_STALL | SURV_FLAG_PERSISTENT)) == 0;
+  // A cohort that one cluster holds runs there (ccd_cluster.cu; a flag asks
+  // for one of the other schedules).  Else fits run as per-coordinate kernels
+  // replayed in a CUDA graph; the single evaluation of loglik_grad_hess, the
+  // stall test and SURV_FLAG_PERSISTENT use the persistent kernel.
+  bool cluster = false, graph = false;
   int G = 0, wpc = 0;
-  if (graph) CUDA_TRY(survgpu::graph_grid_size(model, layout, prec, &G, &wpc));
-  else CUDA_TRY(survgpu::ccd_grid_size(model, layout, prec, &G, &wpc));
-  if (G < 1) { set_error("CCD kernel cannot be made co-resident"); return SURV_E_CUDA; }
-  const int32_t nwarps = G * wpc;
-  const int64_t nwords = (n + 31) / 32;
-  const int32_t wpw = (int32_t)((nwords + nwarps - 1) / nwarps);
-  const int64_t rows_per_warp = (int64_t)wpw * 32;
+  int32_t nwarps = 0, wpw = 0;
+  int64_t rows_per_warp = 0;
+  auto partition = [&](bool may_cluster) -> int {
+    G = 0;
+    if (may_cluster) CUDA_TRY(survgpu::cluster_grid_size(model, layout, prec, n, p, &G, &wpc));
+    cluster = G > 0;
+    graph = !cluster && single_j < 0 && (o.flags & (SURV_FLAG_TEST_STALL | SURV_FLAG_PERSISTENT)) == 0;
+    if (graph) CUDA_TRY(survgpu::graph_grid_size(model, layout, prec, &G, &wpc));
+    else if (!cluster) CUDA_TRY(survgpu::ccd_grid_size(model, layout, prec, &G, &wpc));
+    if (G < 1) { set_error("CCD kernel cannot be made co-resident"); return SURV_E_CUDA; }
+    nwarps = G * wpc;
+    const int64_t nwords = (n + 31) / 32;
+    wpw = (int32_t)((nwords + nwarps - 1) / nwarps);
+    rows_per_warp = (int64_t)wpw * 32;
+    return SURV_OK;
+  };
+  int rc;
+  if ((rc = partition(o.flags == 0))) return rc;
 
   // ---------------------------------------------------------- staging
-  int rc;
   Staged stg;
   if ((rc = stage_data(d, prec, ws, s, &stg, &launches))) return rc;
   const void *colptr_d = stg.colptr, *rowidx_d = stg.rowidx;
@@ -401,6 +412,15 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
                                &cols_nb)))
     return rc;
   if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
+  if (cluster && K > survgpu::kClusterMaxEnds) {   // too many group ends for a few SMs: the warps' rows change
+    if ((rc = partition(false))) return rc;
+    if (layout == SURV_CSC) {
+      if ((rc = ensure(ws, W::WOFF, 4 * (size_t)p * (nwarps + 1), &woff))) return rc;
+      CUDA_TRY(survgpu::prep_warp_offsets(stg.colptr, stg.rowidx, p, n, nwarps, rows_per_warp,
+                                          static_cast<int32_t*>(woff), s));
+      ++launches;
+    }
+  }
   const void* vals_d = stg.vals;  // null for indicator CSC data (all values 1)
   DevCtrl hc;
 
@@ -561,10 +581,10 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   P.withhold_cta = (o.flags & SURV_FLAG_TEST_STALL) ? 0 : -1;
   P.no_pdl = (o.flags & SURV_FLAG_NO_PDL) ? 1 : 0;
   P.timeout_ns = (uint64_t)((o.wait_limit_s > 0.0 ? o.wait_limit_s : 2.0) * 1e9);
+  P.gctl = &ctrl->gctl;
   if (graph) {
     P.wt = static_cast<uint64_t*>(wt);
     P.agg = static_cast<uint64_t*>(aggr);
-    P.gctl = &ctrl->gctl;
   }
   struct Events {
     cudaEvent_t a = nullptr, b = nullptr;
@@ -576,6 +596,8 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   CUDA_TRY(cudaEventCreate(&ev.a));
   CUDA_TRY(cudaEventCreate(&ev.b));
   int replays = 0;
+  // sweeps a cluster launch may run (8192 coordinates: some tens of ms)
+  const int cluster_sweeps = (int)std::max<int64_t>(1, 8192 / p);
   if (graph) {
     int glaunches = 0;
     CUDA_TRY(survgpu::graph_init(P, s));
@@ -593,6 +615,10 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
                                       ev.a, &replays, &glaunches));
     }
     launches += glaunches;
+  } else if (cluster) {
+    CUDA_TRY(cudaEventRecord(ev.a, s));
+    CUDA_TRY(survgpu::run_cluster(model, layout, prec, P, cluster_sweeps, s));
+    ++launches;
   } else {
     CUDA_TRY(cudaEventRecord(ev.a, s));
     CUDA_TRY(survgpu::launch_ccd(model, layout, prec, P, s));
@@ -603,6 +629,15 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   std::vector<double> beta_out(p);
   CUDA_TRY(cudaMemcpyAsync(beta_out.data(), beta, 8 * (size_t)p, cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
+  // every launch but the last runs cluster_sweeps sweeps
+  for (int64_t done = cluster_sweeps; cluster && hc.gctl.done != 1 && done <= o.max_sweeps; done += cluster_sweeps) {
+    CUDA_TRY(survgpu::run_cluster(model, layout, prec, P, cluster_sweeps, s));
+    ++launches;
+    CUDA_TRY(cudaEventRecord(ev.b, s));
+    CUDA_TRY(cudaMemcpyAsync(&hc, ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaMemcpyAsync(beta_out.data(), beta, 8 * (size_t)p, cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+  }
   float kernel_ms = 0.f;
   CUDA_TRY(cudaEventElapsedTime(&kernel_ms, ev.a, ev.b));
 
@@ -630,7 +665,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     info->phase_ms[survgpu::PH_PASS_SUM] /= (double)G;  // mean over CTAs
     info->row_passes = (int64_t)hc.out[spec_b ? survgpu::OUT_BATCHES : survgpu::OUT_PASSES];
   }
-  if (graph && hc.gctl.done != 1) {
+  if ((graph || cluster) && hc.gctl.done != 1) {
     set_error("CCD stopped after %d sweep replays without a stop decision", replays);
     return SURV_E_CUDA;
   }

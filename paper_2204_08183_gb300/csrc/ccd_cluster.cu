@@ -1,0 +1,435 @@
+// CCD for cohorts that a few SMs hold (Sections 2.4 and 2.7): one kernel on
+// one thread-block cluster runs whole sweeps.
+//
+// At these sizes the kernel pair of ccd_graph.cu is bound by its dependent
+// steps, not by bytes: two launches a coordinate, an aggregate and a partial
+// exchange through L2, a ticket, and replays that run empty after the stop
+// (17 to 30 us a coordinate whatever the size).  Here the CTAs of one cluster
+// exchange through distributed shared memory and the hardware's cluster
+// barrier, and every CTA takes the Newton step itself from the same numbers in
+// the same order, so a coordinate needs two cluster barriers and nothing else
+// (11 to 23 us; its row pass, on 16 SMs instead of 152, is the longest part,
+// the two barriers take 1 us):
+//
+//   rows     each warp updates and passes over its own rows (warp_pass, the
+//            same code as the kernel pair); warp totals -> the CTA's aggregate,
+//            stored into every CTA of the cluster; barrier
+//   ends     prefix of the CTAs before, steps 3-4 at the CTA's group ends,
+//            the CTA's three partial sums stored into every CTA; barrier
+//   step     the partials summed in rank order, trust-region Newton step
+//
+// The barrier is hardware and the CTAs of a cluster run together, so there
+// is no wait that could fail to end.  A launch runs a bounded number of
+// sweeps; the state goes back to the control line, and the host launches
+// again until the fit reports its stop.
+#include <algorithm>
+
+#include "graph_common.cuh"
+
+namespace survgpu {
+namespace {
+
+using namespace ccdk;
+
+constexpr int kClThreads = 512;
+constexpr int kClWarps = kClThreads / 32;
+constexpr int kClMax = 16;    // CTAs of the cluster (8 where 16 cannot be placed)
+constexpr int kClMaxP = 1024; // coordinate scalars in shared memory: 32 bytes each
+
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// (.aligned: the lanes of a warp arrive and wait together)
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// store an 8-byte accumulator at the address that `local` has in CTA `rank`
+__device__ __forceinline__ void store_remote(const void* local, unsigned rank, uint64_t v) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(local);
+  uint32_t ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(ra), "l"(v) : "memory");
+}
+
+// 16-byte loads per lane a tile: a warp holds few rows, and rows that a tile
+// has beyond them are worked on all the same, which costs most in FP64
+// (sparse Cox, ms a fit with 1, 2 and 4 loads: 4.83, 4.91, 5.16 at 20,000 x
+// 100; 5.42, 4.94, 4.75 at 200,000)
+template <typename T>
+struct ClCfg {
+  static constexpr int U = sizeof(T) == 8 ? 1 : 2;
+  static constexpr int SR = 4;
+};
+
+template <int MODEL, int LAYOUT, typename T, bool MULTI>
+__global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant__ CcdParams P, int sweeps) {
+  using A = typename AccOf<T>::type;
+  using C = Cfg<MODEL, LAYOUT, T>;
+  constexpr int M = C::M;
+  constexpr int U = ClCfg<T>::U, SR = ClCfg<T>::SR;
+  extern __shared__ double s_coord[];   // beta, width, lambda * penalty factor, delta^T X of each coordinate
+  __shared__ A s_wtot[kClWarps][M];     // warp totals (components of an unchanged e stay)
+  __shared__ A s_base[kClWarps][M];     // sums of the rows before each warp
+  __shared__ A s_tot[3];                // Fine-Gray: grand totals of the weighted components
+  __shared__ A s_agg[kClMax][M];        // every CTA's totals (written by the CTAs)
+  __shared__ A s_part[kClMax][3];       // every CTA's partial sums (written by the CTAs)
+  __shared__ A s_red[kClWarps][3];
+  __shared__ double s_lin[2], s_applied;
+  __shared__ float s_delta[2];
+  __shared__ int s_stop;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int rank = (int)cluster_rank(), CL = P.G, WPC = P.wpc, p = P.p;
+  const int64_t n = P.n, nwords = (n + 31) >> 5;
+  const bool rows = w < WPC;            // warps that hold rows
+  const int gw = rank * WPC + (rows ? w : 0);
+  const int64_t word_lo = min((int64_t)gw * P.wpw, nwords), word_hi = min(word_lo + P.wpw, nwords);
+  const int64_t row_lo = word_lo * 32, row_hi = min(word_hi * 32, n);
+  const int kc_lo = P.wk0[rank * WPC], kc_hi = P.wk0[(rank + 1) * WPC];
+  double *s_beta = s_coord, *s_width = s_coord + p, *s_pen = s_coord + 2 * p, *s_dtx = s_coord + 3 * p;
+  for (int i = tid; i < p; i += kClThreads) {
+    s_beta[i] = P.beta[i];
+    s_width[i] = P.width[i];
+    s_pen[i] = P.pen[i];
+    s_dtx[i] = P.dTx[i];
+  }
+  const CtlLine* L = &P.gctl->line[0];
+  double applied = L->applied;
+  ff delta = {L->delta_hi, L->delta_lo};
+  int nevals = L->nevals, stop = L->stop;
+  double f_prev = L->f_prev;
+  long long passes = L->passes, eta_updates = L->eta_updates;
+  bool dirty = passes == 0;   // the first pass of a fit
+  if (stop) return;   // the same in every CTA
+  // the group end that thread tid takes first
+  int d1 = 0, wl1 = 0;
+  double g1 = 0.0;
+  float2 gf1 = make_float2(0.f, 0.f);
+  if (kc_lo + tid < kc_hi) {
+    const int k = kc_lo + tid;
+    d1 = P.dk[k];
+    wl1 = (int)((P.gend[k] >> 5) / P.wpw) - rank * WPC;
+    if (MODEL == 1) {
+      g1 = P.Gk[k];
+      gf1 = P.Gkff[k];
+    }
+  }
+  constexpr bool kFuse = LAYOUT == 1 && sizeof(T) == 4;
+  A* rec = reinterpret_cast<A*>(P.rec);
+  const bool single = P.single_j >= 0;
+  int j = single ? P.single_j : 0;
+  PassPrefetch<T, SR> pf;
+  if (rows) pass_prefetch<LAYOUT, T, SR>(P, j, gw, pf);
+  __syncthreads();
+  cluster_arrive();   // every CTA of the cluster has started: its shared memory may be written
+  cluster_wait();
+
+  for (int sw = 0; sw < sweeps && !stop;) {
+    const int q = j == 0 ? p - 1 : j - 1;
+    const bool eval = j == 0 || single;
+    const bool dense = LAYOUT == 1 || applied != 0.0 || dirty;
+    // ------------------------------------------------ steps 1-2, own rows
+    if (rows) {
+      if (applied != 0.0 && !kFuse) warp_update<LAYOUT, T>(P, q, gw, row_lo, row_hi, applied, delta);
+      const T* xq = (kFuse && applied != 0.0) ? reinterpret_cast<const T*>(P.X) + (size_t)q * P.ld : nullptr;
+      A tot[M];
+      warp_pass<MODEL, LAYOUT, T, U, SR, MULTI, true>(P, j, row_lo, row_hi, rec, tot, pf, dense, xq, delta);
+      if (lane == 0)
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+          if (dense || !(m == 0 || m == 3)) s_wtot[w][m] = tot[m];
+    }
+    __syncthreads();
+    A wex[M];
+    if (w == 0) {
+      A v[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        acc_zero(v[m]);
+        if (lane < WPC) v[m] = s_wtot[lane][m];
+      }
+      warp_scan_n<M>(v, lane);
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        wex[m] = shfl_up(v[m], 1);
+        if (lane == 0) acc_zero(wex[m]);
+        const A t = shfl_idx(v[m], WPC - 1);
+        if (lane < CL) store_remote(&s_agg[rank][m], lane, pack8(t));
+      }
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (w == 0) {
+      A v[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        acc_zero(v[m]);
+        if (lane < CL) v[m] = s_agg[lane][m];
+      }
+      warp_scan_n<M>(v, lane);
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        A before = shfl_idx(v[m], rank > 0 ? rank - 1 : 0);
+        if (rank == 0) acc_zero(before);
+        const A all = shfl_idx(v[m], CL - 1);
+        if (lane < WPC) s_base[lane][m] = acc_add(before, wex[m]);
+        if (MODEL == 1 && m >= 3 && lane == 0) s_tot[m % 3] = all;
+      }
+    }
+    __syncthreads();
+    // ------------------------------------------------ steps 3-4, own ends
+    A fg1, fg2;
+    acc_zero(fg1);
+    acc_zero(fg2);
+    double pl = 0.0;
+    for (int k = kc_lo + tid; k < kc_hi; k += kClThreads) {
+      int d = d1, wl = wl1;
+      double g = g1;
+      float2 gf = gf1;
+      if (k != kc_lo + tid) {
+        d = P.dk[k];
+        wl = (int)((P.gend[k] >> 5) / P.wpw) - rank * WPC;
+        if (MODEL == 1) {
+          g = P.Gk[k];
+          gf = P.Gkff[k];
+        }
+      }
+      if (d == 0) continue;
+      A Pm[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) Pm[m] = acc_add(s_base[wl][m], rec[(size_t)k * M + m]);
+      A den = Pm[0], num1 = Pm[1], num2 = Pm[2];
+      if (MODEL == 1) {
+        const A gg = acc_base<A>(g, ff{gf.x, gf.y});
+        den = acc_add(den, acc_mul(gg, acc_add(s_tot[0], acc_neg(Pm[3 % M]))));
+        num1 = acc_add(num1, acc_mul(gg, acc_add(s_tot[1], acc_neg(Pm[4 % M]))));
+        num2 = acc_add(num2, acc_mul(gg, acc_add(s_tot[2], acc_neg(Pm[5 % M]))));
+      }
+      const A inv = acc_recip(den);
+      const A Gr = acc_mul(num1, inv);
+      const A H = acc_mul(num2, inv);
+      fg1 = acc_add(fg1, acc_scale(Gr, d));
+      fg2 = acc_add(fg2, acc_scale(acc_add(H, acc_neg(acc_mul(Gr, Gr))), d));
+      if (eval) pl += (double)d * log(acc_to_d(den));
+    }
+    const int nred = min((kc_hi - kc_lo + 31) >> 5, kClWarps);   // warps that had ends
+    if (w < nred) {
+      A r[3] = {fg1, fg2, eval ? acc_from_d(pl, (A*)nullptr) : A{}};
+      warp_sum_n<3>(r);
+      if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) s_red[w][i] = r[i];
+    }
+    __syncthreads();
+    if (w == 0) {
+      A r[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc_zero(r[i]);
+        if (lane < nred) r[i] = s_red[lane][i];
+      }
+      warp_sum_n<3>(r);
+      if (lane < CL)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) store_remote(&s_part[rank][i], lane, pack8(r[i]));
+    } else if (w == 1 && eval) {
+      // pieces of the objective at the current beta, in the order of warp_lin_pen
+      double lin = 0.0, pen = 0.0;
+      for (int i = lane; i < p; i += 32) {
+        const double b = s_beta[i];
+        lin += b * s_dtx[i];
+        if (P.penalty == 1) pen -= s_pen[i] * fabs(b);
+        else if (P.penalty == 2) pen -= s_pen[i] * b * b * 0.5;
+      }
+      lin = warp_sum(lin);
+      pen = warp_sum(pen);
+      if (lane == 0) {
+        s_lin[0] = lin;
+        s_lin[1] = pen;
+      }
+    }
+    cluster_arrive();
+    // the next coordinate's column entries do not depend on this step
+    const int jn = j + 1 < p ? j + 1 : 0;
+    if (rows && !single) pass_prefetch<LAYOUT, T, SR>(P, jn, gw, pf);
+    cluster_wait();
+    // ------------------------------------------------ the step (every CTA)
+    if (w == 0) {
+      A r[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc_zero(r[i]);
+        if (lane < CL) r[i] = s_part[lane][i];
+      }
+      warp_sum_n<3>(r);
+      if (lane == 0) {
+        const double grad = s_dtx[j] - acc_to_d(r[0]), hess = -acc_to_d(r[1]);
+        int st = 0;
+        double ap = 0.0;
+        if (eval) {
+          const double ll = s_lin[0] - acc_to_d(r[2]);
+          const double f = ll + s_lin[1];
+          const double fp = nevals >= 1 ? f_prev : 0.0;
+          const bool conv = nevals >= 1 && fabs(f - fp) / fabs(f) < P.tol;
+          st = (single || conv || nevals >= P.max_sweeps) ? 1 : 0;
+          if (st && rank == 0) {
+            P.out[OUT_LOGLIK] = ll;
+            P.out[OUT_OBJECTIVE] = f;
+            P.out[OUT_OBJECTIVE_PREV] = fp;
+            P.out[OUT_SWEEPS] = (double)nevals;
+            P.out[OUT_CONVERGED] = conv ? 1.0 : 0.0;
+            P.out[OUT_ETA_UPDATES] = (double)eta_updates;
+            P.out[OUT_PASSES] = (double)(passes + 1);
+            P.out[OUT_GRAD] = grad;
+            P.out[OUT_HESS] = hess;
+            P.gctl->done = 1;
+          }
+          ++nevals;
+          f_prev = f;
+        }
+        ++passes;
+        if (!st) {
+          const double b = s_beta[j], wd = s_width[j];
+          const double step = newton_step(b, grad, hess, P.penalty, s_pen[j]);
+          if (step != 0.0) ap = copysign(fmin(fabs(step), wd), step);
+          s_beta[j] = b + ap;
+          s_width[j] = fmax(2.0 * fabs(ap), wd / 2.0);
+          if (ap != 0.0) ++eta_updates;
+        }
+        const ff df = d_to_ff(ap);
+        s_applied = ap;
+        s_delta[0] = df.hi;
+        s_delta[1] = df.lo;
+        s_stop = st;
+      }
+    }
+    __syncthreads();
+    applied = s_applied;
+    delta = {s_delta[0], s_delta[1]};
+    stop = s_stop;
+    dirty = false;
+    if (!stop && jn == 0) ++sw;
+    if (!stop) j = jn;
+  }
+  // the state for the next launch
+  if (rank == 0) {
+    for (int i = tid; i < p; i += kClThreads) {
+      P.beta[i] = s_beta[i];
+      P.width[i] = s_width[i];
+    }
+    if (tid == 0) {
+      CtlLine* W = &P.gctl->line[0];
+      W->stop = stop;
+      W->nevals = nevals;
+      W->applied = applied;
+      W->delta_hi = delta.hi;
+      W->delta_lo = delta.lo;
+      W->f_prev = f_prev;
+      W->passes = passes;
+      W->eta_updates = eta_updates;
+      W->dirty = 0;
+    }
+  }
+}
+
+template <int MODEL, int LAYOUT, typename T>
+cudaError_t cluster_size_of(int* G) {
+  static_assert(kClWarps <= 32 && kClMax <= 32, "one lane per warp and per CTA");
+  auto k = k_cluster<MODEL, LAYOUT, T, false>;
+  *G = 0;
+  cudaError_t st = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (st != cudaSuccess) return st;
+  for (int cl : {kClMax, 8}) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)cl, 1, 1};
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(cl);
+    c.blockDim = dim3(kClThreads);
+    c.dynamicSmemBytes = 4 * sizeof(double) * kClMaxP;
+    c.attrs = at;
+    c.numAttrs = 1;
+    int num = 0;
+    if (cudaOccupancyMaxActiveClusters(&num, k, &c) == cudaSuccess && num >= 1) {
+      *G = cl;
+      return cudaSuccess;
+    }
+    cudaGetLastError();
+  }
+  return cudaSuccess;
+}
+
+template <int MODEL, int LAYOUT, typename T>
+cudaError_t launch_cluster(const CcdParams& P, int sweeps, cudaStream_t s) {
+  const bool multi = (int64_t)P.K >= 2 * (int64_t)P.nwarps;
+  auto k = multi ? k_cluster<MODEL, LAYOUT, T, true> : k_cluster<MODEL, LAYOUT, T, false>;
+  cudaError_t st = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (st != cudaSuccess) return st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)P.G, 1, 1};
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(P.G);
+  c.blockDim = dim3(kClThreads);
+  c.dynamicSmemBytes = 4 * sizeof(double) * (size_t)P.p;
+  c.stream = s;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, P, sweeps);
+}
+
+#define SURV_DISPATCH_CL(FN, ...)                                                          \
+  do {                                                                                     \
+    if (model == 0 && layout == 0 && prec == 0) return FN<0, 0, float>(__VA_ARGS__);       \
+    if (model == 0 && layout == 0 && prec == 1) return FN<0, 0, double>(__VA_ARGS__);      \
+    if (model == 0 && layout == 1 && prec == 0) return FN<0, 1, float>(__VA_ARGS__);       \
+    if (model == 0 && layout == 1 && prec == 1) return FN<0, 1, double>(__VA_ARGS__);      \
+    if (model == 1 && layout == 0 && prec == 0) return FN<1, 0, float>(__VA_ARGS__);       \
+    if (model == 1 && layout == 0 && prec == 1) return FN<1, 0, double>(__VA_ARGS__);      \
+    if (model == 1 && layout == 1 && prec == 0) return FN<1, 1, float>(__VA_ARGS__);       \
+    if (model == 1 && layout == 1 && prec == 1) return FN<1, 1, double>(__VA_ARGS__);      \
+    return cudaErrorInvalidValue;                                                          \
+  } while (0)
+
+// Largest cohorts for which a fit in one cluster was the faster (whole calls,
+// ms, cluster and kernel pair).  FP64 is bound by the FP64 pipes of the 16
+// SMs beyond two words a warp: 0.83 and 1.37 at 10,000 x 10 dense, 2.06 and
+// 1.37 at 20,000.  FP32: sparse Cox (against batches) 4.65 and 5.89 at 200,000
+// x 100, 5.79 and 5.16 at 400,000; dense Cox 1.73 and 1.98 at 100,000 x 24,
+// 2.27 and 2.0 at 200,000; sparse Fine-Gray 3.92 and 4.27 at 200,003 x 40, 5.35
+// and 4.3 at 400,000; dense Fine-Gray 4.69 and 4.85 at 100,000 x 50, 6.74 and
+// 5.0 at 200,000.  By group ends (kClusterMaxEnds): sparse Cox with hardly any
+// ties 4.93 and 5.64 at 20,000 x 80, 7.3 and 6.5 at 50,000.
+int64_t cluster_rows(int model, int layout, int prec) {
+  if (prec == 1) return 2 * 32 * kClMax * kClWarps;   // 16,384
+  if (layout == 0) return model == 0 ? 300000 : 262144;
+  return model == 0 ? 131072 : 100000;
+}
+
+}  // namespace
+
+cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc) {
+  *G = 0;
+  *wpc = 0;
+  if (n > cluster_rows(model, layout, prec) || p > kClMaxP) return cudaSuccess;
+  cudaError_t st = [&] { SURV_DISPATCH_CL(cluster_size_of, G); }();
+  if (st != cudaSuccess || *G == 0) return st;
+  // no more row warps than the words need, so that the rows are spread evenly
+  // over the CTAs
+  const int64_t nwords = (n + 31) / 32, most = (int64_t)*G * kClWarps;
+  const int64_t wpw = (nwords + most - 1) / most, used = (nwords + wpw - 1) / wpw;
+  *wpc = (int)((used + *G - 1) / *G);
+  return cudaSuccess;
+}
+
+cudaError_t run_cluster(int model, int layout, int prec, const CcdParams& P, int sweeps, cudaStream_t s) {
+  SURV_DISPATCH_CL(launch_cluster, P, sweeps, s);
+}
+
+}  // namespace survgpu

@@ -198,6 +198,15 @@ cudaError_t graph_cache_prepare(GraphCache* gc);
 cudaError_t replay_until_stop(const CcdParams& P, cudaStream_t s, GraphCache* gc, cudaEvent_t t0,
                               int launches_per_replay, int* replays, int* launches, int max_replays = 0);
 
+// ---- one cluster for small cohorts (ccd_cluster.cu) ----------------------
+// CTAs (0: not for this problem) and row warps per CTA of the cluster kernel,
+// which is for cohorts of at most kClusterMaxEnds tie groups (known later).
+constexpr int32_t kClusterMaxEnds = 32768;
+cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc);
+// Up to `sweeps` sweeps of a fit (or the evaluation of P.single_j) in one
+// launch; *P.gctl zeroed before the first.  P.gctl->done tells the stop.
+cudaError_t run_cluster(int model, int layout, int prec, const CcdParams& P, int sweeps, cudaStream_t s);
+
 // ---- speculative coordinate batches (spec.cu) ----------------------------
 // Cox, CSC, FP32 mode: each row pass evaluates the derivatives of B
 // consecutive coordinates at the same e; the steps are taken in order up to
