@@ -272,6 +272,7 @@ cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr
 struct RowMasks {              // [ceil(n / 32)] each
   uint32_t* end = nullptr;     // bit r: row 32 w + r ends a group
   int32_t* first = nullptr;    // group ends before row 32 w
+  uint32_t* event = nullptr;   // bit r: its status is 1 (optional)
 };
 size_t prep_count_bytes(int64_t n);
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,

@@ -565,17 +565,27 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   const int K = hc.K;
   NLL_TRY(ws_ensure(ws, W::NLL_GEND, 4 * (size_t)K, &gend));
   NLL_TRY(ws_ensure(ws, W::NLL_DK, 4 * (size_t)K, &dk));
-  // row partition of the scan kernels: two CTAs of 16 warps per SM
+  // units of consecutive rows in the scan: four per CTA of the fused kernel,
+  // else the warps of two CTAs of 16 warps per SM
   int dev = 0, sms = 0;
   NLL_TRY(cuda_err(cudaGetDevice(&dev), "device"));
   NLL_TRY(cuda_err(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count"));
-  const int G = 2 * sms, wpc = kNllThreads / 32, nwarps = G * wpc;
+  const bool fused = nll_fused_fits(n, (int)p, C);
+  const int G = fused ? sms : 2 * sms, wpc = fused ? 4 : kNllThreads / 32, nwarps = G * wpc;
   const int64_t nwords = (n + 31) / 32;
-  const int64_t wpw = (nwords + nwarps - 1) / nwarps;
-  const int64_t rpw = wpw * 32;
+  const int64_t rpw = fused ? nll_fused_unit_rows(n, nwarps) : (nwords + nwarps - 1) / nwarps * 32;
+  RowMasks masks;
+  if (fused) {
+    void* mk = nullptr;
+    NLL_TRY(ws_ensure(ws, W::NLL_MASK, 12 * (size_t)nwords, &mk));
+    masks.end = static_cast<uint32_t*>(mk);
+    masks.event = masks.end + nwords;
+    masks.first = reinterpret_cast<int32_t*>(masks.event + nwords);
+  }
   NLL_TRY(ws_ensure(ws, W::NLL_WK0, 4 * (size_t)(nwarps + 1), &wk0));
   NLL_TRY(cuda_err(prep_group_write(time, status, n, blk, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
-                                    nullptr, nwarps, rpw, static_cast<int32_t*>(wk0), s),
+                                    nullptr, nwarps, rpw, fused ? nullptr : static_cast<int32_t*>(wk0), s,
+                                    fused ? &masks : nullptr),
                    "write groups"));
   // eta = X B_hi + X B_lo on the tensor cores (nll_tc.cu).  Bcat^T holds the
   // split in 2 Cp rows, Cp = C rounded up to 16 (at least 32); X and Bcat^T
@@ -592,29 +602,36 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
     NLL_TRY(cuda_err(cudaGetLastError(), "pad X"));
     Xt = xp;
   }
-  NLL_TRY(ws_ensure(ws, W::NLL_Y, sizeof(float) * (size_t)n * C, &Y));
-  NLL_TRY(ws_ensure(ws, W::NLL_BCAT, sizeof(__nv_bfloat16) * (size_t)2 * Cp * ld, &Bcat));
+  NLL_TRY(ws_ensure(ws, W::NLL_BCAT, sizeof(__nv_bfloat16) * (size_t)std::max(128, 2 * Cp) * ld, &Bcat));
   void* errw = nullptr;
   NLL_TRY(ws_ensure(ws, W::NLL_ERR, sizeof(unsigned), &errw));
   if (!ws->nll_err_init) {
     NLL_TRY(cuda_err(cudaMemsetAsync(errw, 0, sizeof(unsigned), s), "memset"));
     ws->nll_err_init = true;
   }
-  const int64_t nbt = (int64_t)2 * Cp * ld;
-  k_split_bt<<<(unsigned)((nbt + 255) / 256), 256, 0, s>>>(B, p, C, Cp, ld, static_cast<__nv_bfloat16*>(Bcat));
-  NLL_TRY(cuda_err(cudaGetLastError(), "split B"));
-  NLL_TRY(cuda_err(nll_xb_tc(Xt, n, (int)p, ld, Bcat, C, Cp, static_cast<float*>(Y), static_cast<unsigned*>(errw), s),
-                   "tensor-core X B"));
   NLL_TRY(ws_ensure(ws, W::NLL_REC, sizeof(float2) * (size_t)K * C, &rec));
   NLL_TRY(ws_ensure(ws, W::NLL_WT, 2 * sizeof(float2) * (size_t)nwarps * C, &wt));
   NLL_TRY(ws_ensure(ws, W::NLL_DEN, sizeof(double) * (size_t)K * C, &den));
   float2* wt2 = static_cast<float2*>(wt);
-  const size_t ssm = stage_smem(C);
-  NLL_TRY(cuda_err(cudaFuncSetAttribute(k_nll_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm), "smem"));
-  k_nll_scan<<<G, kNllThreads, ssm, s>>>(static_cast<const float*>(Y), n, C, status, static_cast<int32_t*>(gend),
-                                         static_cast<int32_t*>(wk0), rpw, static_cast<float2*>(rec), wt2,
-                                         wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw));
-  NLL_TRY(cuda_err(cudaGetLastError(), "scan"));
+  if (fused) {
+    NLL_TRY(cuda_err(nll_fused_split(B, p, C, ld, Bcat, s), "split B"));
+    NLL_TRY(cuda_err(nll_fused_forward(Xt, n, (int)p, ld, Bcat, C, G, rpw, masks, static_cast<float2*>(rec), wt2,
+                                       wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw), s),
+                     "fused forward"));
+  } else {
+    NLL_TRY(ws_ensure(ws, W::NLL_Y, sizeof(float) * (size_t)n * C, &Y));
+    const int64_t nbt = (int64_t)2 * Cp * ld;
+    k_split_bt<<<(unsigned)((nbt + 255) / 256), 256, 0, s>>>(B, p, C, Cp, ld, static_cast<__nv_bfloat16*>(Bcat));
+    NLL_TRY(cuda_err(cudaGetLastError(), "split B"));
+    NLL_TRY(cuda_err(nll_xb_tc(Xt, n, (int)p, ld, Bcat, C, Cp, static_cast<float*>(Y), static_cast<unsigned*>(errw), s),
+                     "tensor-core X B"));
+    const size_t ssm = stage_smem(C);
+    NLL_TRY(cuda_err(cudaFuncSetAttribute(k_nll_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm), "smem"));
+    k_nll_scan<<<G, kNllThreads, ssm, s>>>(static_cast<const float*>(Y), n, C, status, static_cast<int32_t*>(gend),
+                                           static_cast<int32_t*>(wk0), rpw, static_cast<float2*>(rec), wt2,
+                                           wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw));
+    NLL_TRY(cuda_err(cudaGetLastError(), "scan"));
+  }
   const size_t smem = sizeof(float2) * (size_t)nwarps;
   if (smem > 48 * 1024)
     NLL_TRY(cuda_err(cudaFuncSetAttribute(k_nll_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
@@ -637,7 +654,8 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   ws->nll_K = K;
   ws->nll_G = G;
   ws->nll_wpc = wpc;
-  ws->nll_wpw = (int32_t)wpw;
+  ws->nll_wpw = (int32_t)(rpw / 32);
+  ws->nll_fused = fused;
   ws->nll_x = d->X;
   ws->nll_xt = Xt;
   ws->nll_ld = ld;
@@ -668,7 +686,6 @@ int cox_nll_backward(const surv_nll_data* d, const double* grad_nll, float* grad
   int nx = 0;
   const size_t part_floats = nll_xtg_part_floats(n, (int)p, NB, &nx);
   NLL_TRY(ws_ensure(ws, W::NLL_LAM, sizeof(float) * (size_t)K * C, &lam));
-  NLL_TRY(ws_ensure(ws, W::NLL_G, sizeof(__nv_bfloat16) * (size_t)n * NB, &G2));
   NLL_TRY(ws_ensure(ws, W::NLL_GB, sizeof(float) * part_floats, &part));
   const double* den = static_cast<const double*>(ws->bufs[W::NLL_DEN].p);
   const int32_t* dk = static_cast<const int32_t*>(ws->bufs[W::NLL_DK].p);
@@ -676,6 +693,18 @@ int cox_nll_backward(const surv_nll_data* d, const double* grad_nll, float* grad
   const int32_t* wk0 = static_cast<const int32_t*>(ws->bufs[W::NLL_WK0].p);
   k_nll_lambda<<<C, 256, 0, s>>>(den, dk, K, C, static_cast<float*>(lam));
   NLL_TRY(cuda_err(cudaGetLastError(), "lambda"));
+  if (ws->nll_fused) {
+    const int64_t nwords = (n + 31) / 32;
+    RowMasks masks;
+    masks.end = static_cast<uint32_t*>(ws->bufs[W::NLL_MASK].p);
+    masks.event = masks.end + nwords;
+    masks.first = reinterpret_cast<int32_t*>(masks.event + nwords);
+    return cuda_err(nll_fused_backward(ws->nll_xt, n, (int)p, ws->nll_ld, ws->bufs[W::NLL_BCAT].p, C, Cp, K, masks,
+                                       static_cast<float*>(lam), grad_nll, static_cast<float*>(part), nx, grad_B,
+                                       static_cast<unsigned*>(ws->bufs[W::NLL_ERR].p), s),
+                    "fused backward");
+  }
+  NLL_TRY(ws_ensure(ws, W::NLL_G, sizeof(__nv_bfloat16) * (size_t)n * NB, &G2));
   const size_t ssm = stage_smem(C);
   NLL_TRY(cuda_err(cudaFuncSetAttribute(k_nll_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm), "smem"));
   k_nll_grad<<<G, kNllThreads, ssm, s>>>(static_cast<const float*>(ws->bufs[W::NLL_Y].p), n, C, Cp,

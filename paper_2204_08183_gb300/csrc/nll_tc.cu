@@ -29,6 +29,7 @@
 
 #include "internal.h"
 #include "tc.cuh"
+#include "workspace.h"
 
 namespace survgpu {
 namespace {
@@ -375,7 +376,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 // bfloat16 row-major rows x cols (row pitch ld elements, ld * 2 a multiple of
 // 16 bytes), boxes of 64 columns x box_rows rows, 128-byte swizzle, zero fill
 // outside the matrix.
-cudaError_t make_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+cudaError_t encode_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
   if (((uintptr_t)ptr & 15) != 0 || (ld * 2) % 16 != 0) return cudaErrorInvalidValue;
@@ -428,8 +429,8 @@ cudaError_t nll_xb_tc(const void* X, int64_t n, int p, int64_t ldx, const void* 
   const int NB = 2 * Cp;
   const int nkb = (p + kBoxK - 1) / kBoxK;
   CUtensorMap mx, mb;
-  cudaError_t st = make_map(&mx, X, n, p, ldx, kFwdRows);
-  if (st == cudaSuccess) st = make_map(&mb, BcatT, NB, p, ldx, NB);
+  cudaError_t st = encode_map(&mx, X, n, p, ldx, kFwdRows);
+  if (st == cudaSuccess) st = encode_map(&mb, BcatT, NB, p, ldx, NB);
   if (st != cudaSuccess) return st;
   const int ns = nll_xb_stages(p, Cp);
   if (ns < 3) return cudaErrorInvalidValue;
@@ -453,12 +454,22 @@ size_t nll_xtg_part_floats(int64_t n, int p, int NB, int* nx) {
   return (size_t)gx * p * NB;
 }
 
+cudaError_t nll_make_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+  return encode_map(m, ptr, rows, cols, ld, box_rows);
+}
+
+cudaError_t nll_xtg_reduce(const float* part, int nx, int p, int NB, int C, int Cp, float* grad_B, cudaStream_t s) {
+  const int64_t pc = (int64_t)p * C;
+  k_xtg_reduce<<<(unsigned)((pc + kRedX - 1) / kRedX), dim3(kRedX, kRedY), 0, s>>>(part, nx, p, NB, C, Cp, grad_B);
+  return cudaGetLastError();
+}
+
 cudaError_t nll_xtg_tc(const void* X, int64_t n, int p, int64_t ldx, const void* Gcat, int C, int Cp, float* part,
                        int nx, float* grad_B, unsigned* err, cudaStream_t s) {
   const int NB = 2 * Cp;
   CUtensorMap mx, mg;
-  cudaError_t st = make_map(&mx, X, n, p, ldx, kBwdRows);
-  if (st == cudaSuccess) st = make_map(&mg, Gcat, n, NB, NB, kBwdRows);
+  cudaError_t st = encode_map(&mx, X, n, p, ldx, kBwdRows);
+  if (st == cudaSuccess) st = encode_map(&mg, Gcat, n, NB, NB, kBwdRows);
   if (st != cudaSuccess) return st;
   const size_t smem = 1024 + (size_t)kBwdStages * 6 * 8192 + sizeof(TcBars);
   st = cudaFuncSetAttribute(k_xtg_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -468,10 +479,7 @@ cudaError_t nll_xtg_tc(const void* X, int64_t n, int p, int64_t ldx, const void*
   const int64_t rows_per_cta = (per + kBwdRows - 1) / kBwdRows * kBwdRows;
   k_xtg_tc<<<dim3(nx, gy), kTcThreads, smem, s>>>(mx, mg, n, p, NB, rows_per_cta, part, err);
   st = cudaGetLastError();
-  if (st != cudaSuccess) return st;
-  const int64_t pc = (int64_t)p * C;
-  k_xtg_reduce<<<(unsigned)((pc + kRedX - 1) / kRedX), dim3(kRedX, kRedY), 0, s>>>(part, nx, p, NB, C, Cp, grad_B);
-  return cudaGetLastError();
+  return st == cudaSuccess ? nll_xtg_reduce(part, nx, p, NB, C, Cp, grad_B, s) : st;
 }
 
 }  // namespace survgpu

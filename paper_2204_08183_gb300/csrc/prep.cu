@@ -408,12 +408,16 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_write(const int32_t* time
     if (wk0 && (lane & 7) == 0 && i0 < n && (uint32_t)i0 % (uint32_t)rpw == 0)
       wk0[(uint32_t)i0 / (uint32_t)rpw] = k;
     if (masks.end) {   // the masks of 32 rows: nibbles of 8 lanes
-      uint32_t en = q[it].end << (4 * (lane & 7));
+      uint32_t en = q[it].end << (4 * (lane & 7)), ev = q[it].ev << (4 * (lane & 7));
 #pragma unroll
-      for (int d = 1; d < 8; d <<= 1) en |= __shfl_xor_sync(0xffffffffu, en, d);
+      for (int d = 1; d < 8; d <<= 1) {
+        en |= __shfl_xor_sync(0xffffffffu, en, d);
+        ev |= __shfl_xor_sync(0xffffffffu, ev, d);
+      }
       if ((lane & 7) == 0 && i0 < n) {
         masks.end[i0 >> 5] = en;
         masks.first[i0 >> 5] = k;
+        if (masks.event) masks.event[i0 >> 5] = ev;
       }
     }
 #pragma unroll

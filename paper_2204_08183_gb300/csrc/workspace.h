@@ -4,6 +4,8 @@
 // calls.  Internal to the library.
 #pragma once
 
+#include <cuda.h>
+
 #include <cstddef>
 #include <cstdint>
 
@@ -19,7 +21,7 @@ struct surv_workspace {
     SLOTS, CTRL, BLOCKCNT, DTX_PART, ROWMASK, SORTWORK, PERM, PF, WT, AGG,
     // differentiable form (cox_nll_forward / cox_nll_backward)
     NLL_Y, NLL_BCAT, NLL_REC, NLL_WT, NLL_DEN, NLL_LAM, NLL_G, NLL_GB, NLL_GEND, NLL_DK, NLL_WK0, NLL_BLK,
-    NLL_CTRL, NLL_XP, NLL_ERR, NLL_FIN,
+    NLL_CTRL, NLL_XP, NLL_ERR, NLL_FIN, NLL_MASK,
     // cross-validated path (cox_cv_path) and lambda_max
     CV_FOLD, CV_DK, CV_DTX, CV_E, CV_ETA, CV_REC, CV_WT, CV_AGG, CV_PART, CV_GCTL, CV_BETA, CV_WIDTH, CV_PEN,
     CV_OUT, CV_FITS, CV_CTRL, CV_DEN, CV_HELD, CV_MEAN, LM_LAM, LM_R, LM_G,
@@ -36,6 +38,7 @@ struct surv_workspace {
   const void* nll_x = nullptr;
   const void* nll_xt = nullptr;   // X as the tensor-core kernels read it (padded copy if needed)
   int64_t nll_ld = 0;              // its row pitch in elements
+  bool nll_fused = false;          // the forward ran in nll_fused.cu (no eta was kept)
   bool nll_err_init = false;       // the tensor-core kernels' error word has been zeroed
   // CTAs per fit chosen by the cross-validation tuner, and the shape it was
   // tuned for (n, p, fits, layout * 2 + precision, dtype, layout tag)
@@ -60,4 +63,20 @@ size_t nll_xtg_part_floats(int64_t n, int p, int NB, int* nx);
 bool nll_tc_fits(int p, int C);
 cudaError_t nll_xtg_tc(const void* X, int64_t n, int p, int64_t ldx, const void* Gcat, int C, int Cp, float* part,
                        int nx, float* grad_B, unsigned* err, cudaStream_t s);
+cudaError_t nll_make_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows);
+// grad_B from the CTAs' partial sums part [nx][p][NB], halves added in FP64.
+cudaError_t nll_xtg_reduce(const float* part, int nx, int p, int NB, int C, int Cp, float* grad_B, cudaStream_t s);
+
+// The same form with eta kept on the chip (nll_fused.cu): sizes it takes, the
+// rows of one of `units` scan units, the split B (128 rows of ldx bf16), and
+// the two passes.  rec, wt, wd as k_nll_scan leaves them (one entry a unit).
+bool nll_fused_fits(int64_t n, int p, int C);
+int64_t nll_fused_unit_rows(int64_t n, int units);
+cudaError_t nll_fused_split(const float* B, int64_t p, int C, int64_t ldx, void* BcatT, cudaStream_t s);
+cudaError_t nll_fused_forward(const void* X, int64_t n, int p, int64_t ldx, const void* BcatT, int C, int ctas,
+                              int64_t unit_rows, const RowMasks& m, float2* rec, float2* wt, float2* wd, unsigned* err,
+                              cudaStream_t s);
+cudaError_t nll_fused_backward(const void* X, int64_t n, int p, int64_t ldx, const void* BcatT, int C, int Cp, int K,
+                               const RowMasks& m, const float* lam, const double* gout, float* part, int nx,
+                               float* grad_B, unsigned* err, cudaStream_t s);
 }  // namespace survgpu
