@@ -268,8 +268,14 @@ int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, St
   CUDA_TRY(cudaMemsetAsync(ctrl, 0, sizeof(DevCtrl), s));
   int rc;
   if ((rc = ensure(ws, surv_workspace::BLOCKCNT, survgpu::prep_count_bytes(n), cnt))) return rc;
+  uint32_t* event = nullptr;
+  if (cols && layout == SURV_CSC) {
+    void* ev = nullptr;
+    if ((rc = ensure(ws, surv_workspace::EVENTW, 4 * (size_t)((n + 31) / 32), &ev))) return rc;
+    cols->event = event = static_cast<uint32_t*>(ev);
+  }
   CUDA_TRY(survgpu::prep_group_count(st.time, st.status, n, model, *cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events,
-                                     &ctrl->ticket, s));
+                                     &ctrl->ticket, s, event));
   ++*launches;
   int64_t longest = n;
   if (layout == SURV_CSC) {

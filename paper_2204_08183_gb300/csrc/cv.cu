@@ -255,27 +255,36 @@ __global__ void k_cv_select(const double* heldout, int nlambda, int nfolds, doub
 
 // ---------------------------------------------------------------- lambda_max
 // Lambda_k = sum_{k' >= k} d_k' / (e_k' + 1): at beta = 0 every e_r = 1, so
-// the risk set of group k' (subjects 0..e_k') has e_k' + 1 members.  One CTA,
-// groups taken from the last one down in chunks of the block size (FP64).
-__global__ void __launch_bounds__(kScanThreads) k_lmax_lambda(const int32_t* gend, const int32_t* dk, int32_t K,
-                                                               double* lam) {
-  __shared__ double s_w[32];
+// the risk set of group k' (subjects 0..e_k') has e_k' + 1 members.  The
+// quotients by the whole device (FP64 divisions: on one SM they were a fifth
+// of the 96 us that 3,650 groups took), their suffix sums by one CTA, groups
+// taken from the last one down in chunks of the block size; one warp scans the
+// warp totals (every thread adding all 32 of them was most of the rest).
+__global__ void k_lmax_terms(const int32_t* gend, const int32_t* dk, int32_t K, double* lam) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x)
+    lam[k] = (double)dk[k] / ((double)gend[k] + 1.0);
+}
+__global__ void __launch_bounds__(kScanThreads) k_lmax_lambda(int32_t K, double* lam) {
+  __shared__ double s_w[33];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   double carry = 0.0;
   for (int64_t base = 0; base < K; base += kScanThreads) {
     const int64_t k = (int64_t)K - 1 - (base + tid);
-    const double v = k >= 0 ? (double)dk[k] / ((double)gend[k] + 1.0) : 0.0;
+    const double v = k >= 0 ? lam[k] : 0.0;
     const double incl = warp_inclusive_scan(v, lane);
-    __syncthreads();
+    __syncthreads();   // the previous chunk's totals have been read
     if (lane == 31) s_w[w] = incl;
     __syncthreads();
-    double woff = 0.0, tot = 0.0;
-    for (int q = 0; q < kScanThreads / 32; ++q) {
-      if (q < w) woff += s_w[q];
-      tot += s_w[q];
+    if (w == 0) {
+      const double t = warp_inclusive_scan(s_w[lane], lane);
+      __syncwarp();
+      const double ex = __shfl_up_sync(0xffffffffu, t, 1);
+      s_w[lane] = lane == 0 ? 0.0 : ex;
+      if (lane == 31) s_w[32] = t;
     }
-    if (k >= 0) lam[k] = carry + woff + incl;
-    carry += tot;
+    __syncthreads();
+    if (k >= 0) lam[k] = carry + s_w[w] + incl;
+    carry += s_w[32];
   }
 }
 
@@ -402,7 +411,8 @@ cudaError_t lambda_max_device(int layout, int prec, const int64_t* col_ptr, cons
                               const void* values, int64_t ld, int64_t n, int64_t p, const int8_t* status,
                               const int32_t* gend, const int32_t* dk, int32_t K, const double* pf, double* lam,
                               double* r, double* g, double* out, cudaStream_t s) {
-  k_lmax_lambda<<<1, kScanThreads, 0, s>>>(gend, dk, K, lam);
+  k_lmax_terms<<<grid_for(K, kCvThreads, 1024), kCvThreads, 0, s>>>(gend, dk, K, lam);
+  k_lmax_lambda<<<1, kScanThreads, 0, s>>>(K, lam);
   k_lmax_resid<<<grid_for(n, kCvThreads, 8192), kCvThreads, 0, s>>>(gend, K, status, lam, n, r);
   if (layout == 0) {
     if (prec == 0) k_lmax_grad_csc<float><<<(unsigned)p, kCvThreads, 0, s>>>(col_ptr, row_idx, (const float*)values, r, g);

@@ -249,7 +249,8 @@ cudaError_t time_one_sweep(int model, int layout, int prec, const CcdParams& P, 
 // delta^T X_j (part: p x nb accumulators of 8 bytes, nb = prep_col_blocks of
 // the longest column) and, for CSC, the offsets of each warp's first row.
 struct PrepColumns {
-  const int8_t* status = nullptr;
+  const int8_t* status = nullptr;    // dense
+  const uint32_t* event = nullptr;   // CSC: the event words of prep_group_count
   void* part = nullptr;
   int32_t nwarps = 0;
   int64_t rows_per_warp = 0;   // a multiple of 32
@@ -265,18 +266,19 @@ cudaError_t prep_coord_init(const void* part, int prec, int nb, int64_t p, doubl
                             cudaStream_t s);
 cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr, cudaStream_t s);
 // Tie groups.  prep_group_count checks times and status codes (*perr) and
-// writes *K, *total_events (subjects with status 1) and its block counts
-// into cnt (prep_count_bytes(n) bytes); *ticket is a zeroed word.
+// writes *K, *total_events (subjects with status 1), its block counts into cnt
+// (prep_count_bytes(n) bytes) and, with event [ceil(n / 32)], the events (bit r
+// of word w: row 32 w + r has status 1); *ticket is a zeroed word.
 // prep_group_write then fills gend, dk and ck (ck may be null), with wk0 the
 // first group of each warp's rows, and with masks those of every 32 rows.
 struct RowMasks {              // [ceil(n / 32)] each
   uint32_t* end = nullptr;     // bit r: row 32 w + r ends a group
   int32_t* first = nullptr;    // group ends before row 32 w
-  uint32_t* event = nullptr;   // bit r: its status is 1 (optional)
 };
 size_t prep_count_bytes(int64_t n);
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
-                             unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s);
+                             unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s,
+                             uint32_t* event = nullptr);
 cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
                              int32_t* gend, int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rows_per_warp,
                              int32_t* wk0, cudaStream_t s, const RowMasks* masks = nullptr);

@@ -502,6 +502,17 @@ struct NllCtrl {
   unsigned ticket;
 };
 
+// Row masks and event words of the fused form in the workspace.
+int nll_masks(surv_workspace* ws, int64_t nwords, RowMasks* m, uint32_t** event) {
+  void* v = nullptr;
+  const int rc = ws_ensure(ws, surv_workspace::NLL_MASK, 12 * (size_t)nwords, &v);
+  if (rc) return rc;
+  m->end = static_cast<uint32_t*>(v);
+  m->first = reinterpret_cast<int32_t*>(m->end + nwords);
+  *event = m->end + 2 * nwords;
+  return SURV_OK;
+}
+
 #define NLL_TRY(expr)        \
   do {                       \
     const int rc_ = (expr);  \
@@ -543,8 +554,13 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   const int32_t* time = static_cast<const int32_t*>(d->time);
   const int8_t* status = static_cast<const int8_t*>(d->status);
   NLL_TRY(ws_ensure(ws, W::NLL_BLK, prep_count_bytes(n), &blk));
+  const bool fused = nll_fused_fits(n, (int)p, C);
+  const int64_t nwords = (n + 31) / 32;
+  RowMasks masks;
+  uint32_t* event = nullptr;
+  if (fused) NLL_TRY(nll_masks(ws, nwords, &masks, &event));
   NLL_TRY(cuda_err(prep_group_count(time, status, n, 0, blk, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket,
-                                    s),
+                                    s, event),
                    "count groups"));
   NllCtrl hc;
   unsigned prev_err = 0;
@@ -570,18 +586,8 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   int dev = 0, sms = 0;
   NLL_TRY(cuda_err(cudaGetDevice(&dev), "device"));
   NLL_TRY(cuda_err(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count"));
-  const bool fused = nll_fused_fits(n, (int)p, C);
   const int G = fused ? sms : 2 * sms, wpc = fused ? 4 : kNllThreads / 32, nwarps = G * wpc;
-  const int64_t nwords = (n + 31) / 32;
   const int64_t rpw = fused ? nll_fused_unit_rows(n, nwarps) : (nwords + nwarps - 1) / nwarps * 32;
-  RowMasks masks;
-  if (fused) {
-    void* mk = nullptr;
-    NLL_TRY(ws_ensure(ws, W::NLL_MASK, 12 * (size_t)nwords, &mk));
-    masks.end = static_cast<uint32_t*>(mk);
-    masks.event = masks.end + nwords;
-    masks.first = reinterpret_cast<int32_t*>(masks.event + nwords);
-  }
   NLL_TRY(ws_ensure(ws, W::NLL_WK0, 4 * (size_t)(nwarps + 1), &wk0));
   NLL_TRY(cuda_err(prep_group_write(time, status, n, blk, K, static_cast<int32_t*>(gend), static_cast<int32_t*>(dk),
                                     nullptr, nwarps, rpw, fused ? nullptr : static_cast<int32_t*>(wk0), s,
@@ -615,8 +621,8 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   float2* wt2 = static_cast<float2*>(wt);
   if (fused) {
     NLL_TRY(cuda_err(nll_fused_split(B, p, C, ld, Bcat, s), "split B"));
-    NLL_TRY(cuda_err(nll_fused_forward(Xt, n, (int)p, ld, Bcat, C, G, rpw, masks, static_cast<float2*>(rec), wt2,
-                                       wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw), s),
+    NLL_TRY(cuda_err(nll_fused_forward(Xt, n, (int)p, ld, Bcat, C, G, rpw, masks, event, static_cast<float2*>(rec),
+                                       wt2, wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw), s),
                      "fused forward"));
   } else {
     NLL_TRY(ws_ensure(ws, W::NLL_Y, sizeof(float) * (size_t)n * C, &Y));
@@ -694,12 +700,10 @@ int cox_nll_backward(const surv_nll_data* d, const double* grad_nll, float* grad
   k_nll_lambda<<<C, 256, 0, s>>>(den, dk, K, C, static_cast<float*>(lam));
   NLL_TRY(cuda_err(cudaGetLastError(), "lambda"));
   if (ws->nll_fused) {
-    const int64_t nwords = (n + 31) / 32;
     RowMasks masks;
-    masks.end = static_cast<uint32_t*>(ws->bufs[W::NLL_MASK].p);
-    masks.event = masks.end + nwords;
-    masks.first = reinterpret_cast<int32_t*>(masks.event + nwords);
-    return cuda_err(nll_fused_backward(ws->nll_xt, n, (int)p, ws->nll_ld, ws->bufs[W::NLL_BCAT].p, C, Cp, K, masks,
+    uint32_t* event = nullptr;
+    NLL_TRY(nll_masks(ws, (n + 31) / 32, &masks, &event));
+    return cuda_err(nll_fused_backward(ws->nll_xt, n, (int)p, ws->nll_ld, ws->bufs[W::NLL_BCAT].p, C, Cp, K, masks, event,
                                        static_cast<float*>(lam), grad_nll, static_cast<float*>(part), nx, grad_B,
                                        static_cast<unsigned*>(ws->bufs[W::NLL_ERR].p), s),
                     "fused backward");

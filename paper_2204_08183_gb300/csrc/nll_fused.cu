@@ -621,7 +621,7 @@ cudaError_t nll_fused_split(const float* B, int64_t p, int C, int64_t ld, void* 
 }
 
 cudaError_t nll_fused_forward(const void* X, int64_t n, int p, int64_t ldx, const void* BcatT, int C, int ctas,
-                              int64_t ru, const RowMasks& m, float2* rec, float2* wt, float2* wd, unsigned* err,
+                              int64_t ru, const RowMasks& m, const uint32_t* event, float2* rec, float2* wt, float2* wd, unsigned* err,
                               cudaStream_t s) {
   const int nkb = (p + kFuBoxK - 1) / kFuBoxK;
   CUtensorMap mx, mb;
@@ -633,12 +633,13 @@ cudaError_t nll_fused_forward(const void* X, int64_t n, int p, int64_t ldx, cons
   const size_t smem = fwd_smem(nkb, ns);
   st = cudaFuncSetAttribute(k_nll_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (st != cudaSuccess) return st;
-  k_nll_fwd<<<ctas, kFuThreads, smem, s>>>(mx, mb, n, nkb, C, ns, ru, m.end, m.event, m.first, rec, wt, wd, err);
+  k_nll_fwd<<<ctas, kFuThreads, smem, s>>>(mx, mb, n, nkb, C, ns, ru, m.end, event, m.first, rec, wt, wd, err);
   return cudaGetLastError();
 }
 
 cudaError_t nll_fused_backward(const void* X, int64_t n, int p, int64_t ldx, const void* BcatT, int C, int Cp, int K,
-                               const RowMasks& m, const float* lam, const double* gout, float* part, int nx,
+                               const RowMasks& m, const uint32_t* event, const float* lam,
+                               const double* gout, float* part, int nx,
                                float* grad_B, unsigned* err, cudaStream_t s) {
   const int nkb = (p + kFuBoxK - 1) / kFuBoxK;
   CUtensorMap mx;
@@ -651,7 +652,7 @@ cudaError_t nll_fused_backward(const void* X, int64_t n, int p, int64_t ldx, con
   if (st != cudaSuccess) return st;
   const int64_t per = (n + nx - 1) / nx;
   const int64_t rows_per_cta = (per + 63) / 64 * 64;
-  k_nll_bwd<<<nx, kFuBwdThreads, smem, s>>>(mx, static_cast<const uint32_t*>(BcatT), (int)(ldx / 2), n, p, nkb, C, Cp, K, ns, rows_per_cta, m.end, m.event, m.first, lam,
+  k_nll_bwd<<<nx, kFuBwdThreads, smem, s>>>(mx, static_cast<const uint32_t*>(BcatT), (int)(ldx / 2), n, p, nkb, C, Cp, K, ns, rows_per_cta, m.end, event, m.first, lam,
                                          gout, part, err);
   st = cudaGetLastError();
   return st == cudaSuccess ? nll_xtg_reduce(part, nx, p, 2 * Cp, C, Cp, grad_B, s) : st;

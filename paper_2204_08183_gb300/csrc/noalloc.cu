@@ -215,11 +215,14 @@ int run(const surv_data* d, int model, const double* beta, int32_t j, double* ou
   TRY(cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), s));
   const int32_t* tp = static_cast<const int32_t*>(static_cast<const void*>(d->time));
   const int8_t* sp = d->status;
-  TRY(survgpu::prep_group_count(tp, sp, n, model, cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket, s));
+  // (the event words in eta, which is written later)
+  TRY(survgpu::prep_group_count(tp, sp, n, model, cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events, &ctrl->ticket, s,
+                                csc ? static_cast<uint32_t*>(eta) : nullptr));
   // partial sums of delta^T X_j: in the exchange slots, which are zeroed
   // after they have been summed
   survgpu::PrepColumns cols;
   cols.status = sp;
+  cols.event = static_cast<uint32_t*>(eta);
   cols.part = slots;
   cols.nwarps = nwarps;
   cols.rows_per_warp = rows_per_warp;

@@ -55,25 +55,31 @@ __device__ __forceinline__ void block_partial(A v, A* dst) {
 // leaves the block's share of delta^T X_j in part[j][blockIdx.x] and the
 // column's offsets at the warps' first rows in woff[j][.]: entry i is the
 // first at or after the first row of every warp after its predecessor's
-// warp, up to its own.  Three kernels did this before, two of them reading
-// the row indices again, one with a block per column and one with a binary
-// search per (column, warp): 248 us at 5 x 10^7 entries of 100 columns,
-// against 118 us for the one pass over 400 MB.
+// warp, up to its own.  A thread takes 4 consecutive entries (16-byte loads of
+// the indices and values), so neighbours are compared in registers, and looks
+// for a warp boundary once per 4: rows increase, so without one between the
+// entry before and the last there is none inside.  Values of 1 are counted
+// instead of added.  Whether a row is an event comes from a bit per subject: a
+// column at 5 % touches most sectors of the status bytes, 0.8 GB through L2
+// for 100 columns of 10^7 subjects (197 us with them; one entry at a time
+// 222; three separate passes before that 248).
 template <typename T, bool FULL>
 __global__ void __launch_bounds__(kColThreads) k_check_csc(const int64_t* col_ptr, const int32_t* row_idx,
                                                            const T* values, int64_t p, int64_t n,
-                                                           const int8_t* status, int32_t nwarps, uint32_t wpw,
+                                                           const uint32_t* event, int32_t nwarps, uint32_t wpw,
                                                            typename AccOf<T>::type* part, int32_t* woff,
                                                            unsigned* perr) {
   using A = typename AccOf<T>::type;
-  constexpr int U = 4;
+  constexpr int U = 2;
   const int lane = threadIdx.x & 31;
   const float inv_wpw = 1.f / (float)wpw;
+  const bool vec = (((uintptr_t)row_idx | (uintptr_t)values) & 15) == 0;
   unsigned bits = 0;
   for (int64_t j = blockIdx.y; j < p; j += gridDim.y) {
     const int64_t a = col_ptr[j], b = col_ptr[j + 1];
     A acc;
     acc_zero(acc);
+    int ones = 0;
     // the warp that holds row r: r / 32 / wpw by a float quotient, corrected
     auto warp_of = [&](int32_t r) {
       const uint32_t x = (uint32_t)r >> 5;
@@ -86,48 +92,89 @@ __global__ void __launch_bounds__(kColThreads) k_check_csc(const int64_t* col_pt
     int32_t* wo = FULL ? woff + j * (nwarps + 1) : nullptr;
     if (FULL && blockIdx.x == 0 && a == b)
       for (int g = threadIdx.x; g <= nwarps; g += kColThreads) wo[g] = 0;
-    // whole rounds of U x kColThreads entries per block (every lane takes part)
-    for (int64_t i0 = a + (int64_t)blockIdx.x * (U * kColThreads); i0 < b; i0 += (int64_t)gridDim.x * (U * kColThreads)) {
-      int32_t r[U], rp[U];
-      T v[U];
+    // entries 4 q .. 4 q + 3 of the array per thread, those inside [a, b)
+    const int64_t qa = a >> 2, qb = a < b ? (b + 3) >> 2 : qa;
+    // whole rounds of U x kColThreads quads per block (every lane takes part)
+    for (int64_t q0 = qa + (int64_t)blockIdx.x * (U * kColThreads); q0 < qb; q0 += (int64_t)gridDim.x * (U * kColThreads)) {
+      int32_t r[U][4], rp[U];
+      T v[U][4];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int64_t i = i0 + u * kColThreads + threadIdx.x;
-        r[u] = i < b ? row_idx[i] : -1;
-        rp[u] = (lane == 0 && i < b && i > a) ? row_idx[i - 1] : -1;
-        v[u] = (values && i < b) ? values[i] : T(1);
-      }
-      int8_t st[U];
+        const int64_t i = (q0 + u * kColThreads + threadIdx.x) * 4;
+        if (vec && i >= a && i + 4 <= b) {
+          const int4 t = __ldcs(reinterpret_cast<const int4*>(row_idx + i));
+          r[u][0] = t.x, r[u][1] = t.y, r[u][2] = t.z, r[u][3] = t.w;
+          if (values) {
+            if constexpr (sizeof(T) == 4) {
+              const float4 f = __ldcs(reinterpret_cast<const float4*>(values + i));
+              v[u][0] = f.x, v[u][1] = f.y, v[u][2] = f.z, v[u][3] = f.w;
+            } else {
+              const double2 f = __ldcs(reinterpret_cast<const double2*>(values + i));
+              const double2 g = __ldcs(reinterpret_cast<const double2*>(values + i + 2));
+              v[u][0] = f.x, v[u][1] = f.y, v[u][2] = g.x, v[u][3] = g.y;
+            }
+          } else {
 #pragma unroll
-      for (int u = 0; u < U; ++u) st[u] = (FULL && r[u] >= 0 && r[u] < n) ? status[r[u]] : (int8_t)0;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t i = i0 + u * kColThreads + threadIdx.x;
-        const int32_t up = __shfl_up_sync(0xffffffffu, r[u], 1);
-        const int32_t prev = lane == 0 ? rp[u] : up;
-        if (i >= b) continue;
-        bool good = r[u] >= 0 && r[u] < n;
-        if (i > a && prev >= r[u]) good = false;
-        if (!good) bits |= PREP_INDEX;
-        if (values) {
-          if (!isfinite(v[u])) bits |= PREP_NONFINITE;
-          if (v[u] != T(1)) bits |= PREP_VALUES_NOT_ONE;
-        }
-        if (FULL) {
-          if (st[u] == 1) acc = acc_add_v(acc, v[u]);
-          if (good && (i == a || prev >= 0)) {
-            const int32_t g1 = warp_of(r[u]);
-            const int32_t g0 = i > a ? warp_of(prev) + 1 : 0;
-            for (int32_t g = g0; g <= g1; ++g) wo[g] = (int32_t)(i - a);
-            if (i == b - 1)
-              for (int32_t g = g1 + 1; g <= nwarps; ++g) wo[g] = (int32_t)(b - a);
+            for (int e = 0; e < 4; ++e) v[u][e] = T(1);
           }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const bool in = i + e >= a && i + e < b;
+            r[u][e] = in ? row_idx[i + e] : -1;
+            v[u][e] = (values && in) ? values[i + e] : T(1);
+          }
+        }
+        rp[u] = (lane == 0 && i > a && i < b) ? row_idx[i - 1] : -1;
+      }
+      uint32_t st[U][4];
+      if (FULL) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) st[u][e] = (r[u][e] >= 0 && r[u][e] < n) ? event[r[u][e] >> 5] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = (q0 + u * kColThreads + threadIdx.x) * 4;
+        const int32_t up = __shfl_up_sync(0xffffffffu, r[u][3], 1);
+        const int32_t before = lane == 0 ? rp[u] : up;   // entry i - 1 (if it is one of the column's)
+        bool good = true;
+        int32_t prev = before, last = -1;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (i + e < a || i + e >= b) continue;
+          if (r[u][e] < 0 || r[u][e] >= n || (i + e > a && prev >= r[u][e])) good = false;
+          prev = last = r[u][e];
+          if (values) {
+            if (!isfinite(v[u][e])) bits |= PREP_NONFINITE;
+            if (v[u][e] != T(1)) bits |= PREP_VALUES_NOT_ONE;
+          }
+          if (FULL && (st[u][e] >> (r[u][e] & 31) & 1u)) {
+            if (v[u][e] == T(1)) ++ones;
+            else acc = acc_add_v(acc, v[u][e]);
+          }
+        }
+        if (!good) bits |= PREP_INDEX;
+        if (FULL && good && last >= 0 && (i <= a || before >= 0)) {
+          int32_t g0 = i > a ? warp_of(before) + 1 : 0;   // the first warp without its offset
+          const int32_t g1 = warp_of(last);
+          if (g0 <= g1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              if (i + e < a || i + e >= b) continue;
+              const int32_t ge = warp_of(r[u][e]);
+              for (; g0 <= ge; ++g0) wo[g0] = (int32_t)(i + e - a);
+            }
+          }
+          if (i + 4 >= b)   // the column's last entry
+            for (int32_t g = g1 + 1; g <= nwarps; ++g) wo[g] = (int32_t)(b - a);
         }
       }
     }
     if (FULL) {
       __syncthreads();   // the previous column's partial has been read
-      block_partial<A>(acc, part + j * gridDim.x + blockIdx.x);
+      block_partial<A>(acc_add_v(acc, (T)ones), part + j * gridDim.x + blockIdx.x);
     }
   }
   if (bits) atomicOr(perr, bits);
@@ -246,26 +293,36 @@ struct RowQuad {
   unsigned end, ev, ce, bad;   // 4-bit masks of the quad's rows; prep error bits
 };
 
-// Rows i .. i + 3 (those below n).  Every lane of the warp takes part.
-__device__ __forceinline__ RowQuad load_quad(const int32_t* time, const int8_t* status, int64_t n, int64_t i,
-                                             bool vec, int max_status) {
-  const int lane = threadIdx.x & 31;
-  int32_t t[5] = {0, 0, 0, 0, 0};
-  uint32_t st = 0;
+// Times and status codes of rows i .. i + 3 (those below n), and for lane 31
+// the time after them.
+struct RawQuad {
+  int32_t t[5];
+  uint32_t st;
+};
+__device__ __forceinline__ RawQuad load_raw(const int32_t* time, const int8_t* status, int64_t n, int64_t i, bool vec) {
+  RawQuad q = {{0, 0, 0, 0, 0}, 0u};
   if (vec && i + 4 <= n) {
-    const int4 q = *reinterpret_cast<const int4*>(time + i);
-    t[0] = q.x, t[1] = q.y, t[2] = q.z, t[3] = q.w;
-    st = *reinterpret_cast<const uint32_t*>(status + i);
+    const int4 v = *reinterpret_cast<const int4*>(time + i);
+    q.t[0] = v.x, q.t[1] = v.y, q.t[2] = v.z, q.t[3] = v.w;
+    q.st = *reinterpret_cast<const uint32_t*>(status + i);
   } else {
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (i + u < n) {
-        t[u] = time[i + u];
-        st |= (uint32_t)(uint8_t)status[i + u] << (8 * u);
+        q.t[u] = time[i + u];
+        q.st |= (uint32_t)(uint8_t)status[i + u] << (8 * u);
       }
   }
+  if ((threadIdx.x & 31) == 31 && i + 4 < n) q.t[4] = time[i + 4];
+  return q;
+}
+// Their flags.  Every lane of the warp takes part.
+__device__ __forceinline__ RowQuad quad_flags(const RawQuad& q, int64_t n, int64_t i, int max_status) {
+  const int lane = threadIdx.x & 31;
+  int32_t t[5] = {q.t[0], q.t[1], q.t[2], q.t[3], 0};
+  const uint32_t st = q.st;
   t[4] = __shfl_down_sync(0xffffffffu, t[0], 1);
-  if (lane == 31 && i + 4 < n) t[4] = time[i + 4];
+  if (lane == 31) t[4] = q.t[4];
   RowQuad r = {0u, 0u, 0u, 0u};
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -283,6 +340,13 @@ __device__ __forceinline__ RowQuad load_quad(const int32_t* time, const int8_t* 
 __device__ __forceinline__ unsigned quad_counts(const RowQuad& r) {
   return (unsigned)__popc(r.end) | (unsigned)__popc(r.ev) << 10 | (unsigned)__popc(r.ce) << 20;
 }
+// The masks of 8 lanes as one word of 32 rows (in each of them).
+__device__ __forceinline__ uint32_t word_of(unsigned nibble) {
+  uint32_t w = nibble << (4 * (threadIdx.x & 7));
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, d);
+  return w;
+}
 // 16-byte loads of the times and 4-byte loads of the status codes
 __device__ __forceinline__ bool quad_aligned(const int32_t* time, const int8_t* status) {
   return (((uintptr_t)time & 15) | ((uintptr_t)status & 3)) == 0;
@@ -292,7 +356,8 @@ __device__ __forceinline__ bool quad_aligned(const int32_t* time, const int8_t* 
 // censored on exit.  *ticket is zero on entry and on exit.
 __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time, const int8_t* status, int64_t n,
                                                              int model, int64_t nb, int32_t* cnt, unsigned* perr,
-                                                             int32_t* K, int32_t* total_events, unsigned* ticket) {
+                                                             int32_t* K, int32_t* total_events, unsigned* ticket,
+                                                             uint32_t* event) {
   __shared__ unsigned s_w[kGrpThreads / 32];
   __shared__ int32_t s_p[3][kGrpThreads / 32];
   __shared__ int s_last;
@@ -300,11 +365,18 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
   const bool vec = quad_aligned(time, status);
   const int64_t r0 = (int64_t)blockIdx.x * kGrpRows + w * (128 * kGrpRounds) + lane * 4;
   unsigned c = 0, bad = 0;
+  RawQuad raw[kGrpRounds];
+#pragma unroll
+  for (int it = 0; it < kGrpRounds; ++it) raw[it] = load_raw(time, status, n, r0 + 128 * it, vec);
 #pragma unroll
   for (int it = 0; it < kGrpRounds; ++it) {
-    const RowQuad q = load_quad(time, status, n, r0 + 128 * it, vec, model == 1 ? 2 : 1);
+    const RowQuad q = quad_flags(raw[it], n, r0 + 128 * it, model == 1 ? 2 : 1);
     c += quad_counts(q);
     bad |= q.bad;
+    if (event) {
+      const uint32_t ev = word_of(q.ev);
+      if ((lane & 7) == 0 && r0 + 128 * it < n) event[(r0 + 128 * it) >> 5] = ev;
+    }
   }
   if (bad) atomicOr(perr, bad);
   c = __reduce_add_sync(0xffffffffu, c);
@@ -327,8 +399,17 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
   // scanned over the block, the chunks walked again
   const int64_t per = (nb + kGrpThreads - 1) / kGrpThreads;
   const int64_t lo = min((int64_t)tid * per, nb), hi = min(lo + per, nb);
-  int32_t sum[3] = {0, 0, 0};
-  for (int64_t b = lo; b < hi; ++b)
+  constexpr int kKeep = 12;   // counts kept in registers (12.6 million subjects)
+  int32_t keep[3][kKeep], sum[3] = {0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < kKeep; ++q)
+#pragma unroll
+    for (int m = 0; m < 3; ++m) keep[m][q] = lo + q < hi ? __ldcg(cnt + m * nb + lo + q) : 0;
+#pragma unroll
+  for (int q = 0; q < kKeep; ++q)
+#pragma unroll
+    for (int m = 0; m < 3; ++m) sum[m] += keep[m][q];
+  for (int64_t b = lo + kKeep; b < hi; ++b)
 #pragma unroll
     for (int m = 0; m < 3; ++m) sum[m] += __ldcg(cnt + m * nb + b);
   int32_t inc[3] = {sum[0], sum[1], sum[2]};
@@ -349,7 +430,15 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
     run[m] = inc[m] - sum[m];
     for (int q = 0; q < w; ++q) run[m] += s_p[m][q];
   }
-  for (int64_t b = lo; b < hi; ++b)
+#pragma unroll
+  for (int q = 0; q < kKeep; ++q)
+    if (lo + q < hi)
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        cnt[m * nb + lo + q] = run[m];
+        run[m] += keep[m][q];
+      }
+  for (int64_t b = lo + kKeep; b < hi; ++b)
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       const int32_t v = __ldcg(cnt + m * nb + b);
@@ -374,11 +463,14 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_write(const int32_t* time
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const bool vec = quad_aligned(time, status);
   const int64_t r0 = (int64_t)blockIdx.x * kGrpRows + w * (128 * kGrpRounds) + lane * 4;
+  RawQuad raw[kGrpRounds];
   RowQuad q[kGrpRounds];
   unsigned c = 0;
 #pragma unroll
+  for (int it = 0; it < kGrpRounds; ++it) raw[it] = load_raw(time, status, n, r0 + 128 * it, vec);
+#pragma unroll
   for (int it = 0; it < kGrpRounds; ++it) {
-    q[it] = load_quad(time, status, n, r0 + 128 * it, vec, 2);
+    q[it] = quad_flags(raw[it], n, r0 + 128 * it, 2);
     c += quad_counts(q[it]);
   }
   c = __reduce_add_sync(0xffffffffu, c);
@@ -407,17 +499,11 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_write(const int32_t* time
     const int32_t e0 = base[1] + (int32_t)(ex >> 10 & 1023u), c0 = base[2] + (int32_t)(ex >> 20);
     if (wk0 && (lane & 7) == 0 && i0 < n && (uint32_t)i0 % (uint32_t)rpw == 0)
       wk0[(uint32_t)i0 / (uint32_t)rpw] = k;
-    if (masks.end) {   // the masks of 32 rows: nibbles of 8 lanes
-      uint32_t en = q[it].end << (4 * (lane & 7)), ev = q[it].ev << (4 * (lane & 7));
-#pragma unroll
-      for (int d = 1; d < 8; d <<= 1) {
-        en |= __shfl_xor_sync(0xffffffffu, en, d);
-        ev |= __shfl_xor_sync(0xffffffffu, ev, d);
-      }
+    if (masks.end) {
+      const uint32_t en = word_of(q[it].end);
       if ((lane & 7) == 0 && i0 < n) {
         masks.end[i0 >> 5] = en;
         masks.first[i0 >> 5] = k;
-        if (masks.event) masks.event[i0 >> 5] = ev;
       }
     }
 #pragma unroll
@@ -556,11 +642,14 @@ __global__ void __launch_bounds__(kGrpThreads) k_w2(const int32_t* time, const i
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const bool vec = quad_aligned(time, status);
   const int64_t r0 = (int64_t)blockIdx.x * kGrpRows + w * (128 * kGrpRounds) + lane * 4;
+  RawQuad raw[kGrpRounds];
   RowQuad q[kGrpRounds];
   unsigned c = 0;
 #pragma unroll
+  for (int it = 0; it < kGrpRounds; ++it) raw[it] = load_raw(time, status, n, r0 + 128 * it, vec);
+#pragma unroll
   for (int it = 0; it < kGrpRounds; ++it) {
-    q[it] = load_quad(time, status, n, r0 + 128 * it, vec, 2);
+    q[it] = quad_flags(raw[it], n, r0 + 128 * it, 2);
     c += (unsigned)__popc(q[it].end);
   }
   c = __reduce_add_sync(0xffffffffu, c);
@@ -760,11 +849,11 @@ cudaError_t prep_check_csc(const int64_t* col_ptr, const int32_t* row_idx, const
   const uint32_t wpw = (uint32_t)std::max<int64_t>(1, o.rows_per_warp / 32);
   if (prec == 0) {
     auto k = out ? k_check_csc<float, true> : k_check_csc<float, false>;
-    k<<<grid, kColThreads, 0, s>>>(col_ptr, row_idx, (const float*)values, p, n, o.status, o.nwarps, wpw, (ff*)o.part,
+    k<<<grid, kColThreads, 0, s>>>(col_ptr, row_idx, (const float*)values, p, n, o.event, o.nwarps, wpw, (ff*)o.part,
                                    o.woff, perr);
   } else {
     auto k = out ? k_check_csc<double, true> : k_check_csc<double, false>;
-    k<<<grid, kColThreads, 0, s>>>(col_ptr, row_idx, (const double*)values, p, n, o.status, o.nwarps, wpw,
+    k<<<grid, kColThreads, 0, s>>>(col_ptr, row_idx, (const double*)values, p, n, o.event, o.nwarps, wpw,
                                    (double*)o.part, o.woff, perr);
   }
   return cudaGetLastError();
@@ -799,11 +888,12 @@ cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr
 size_t prep_count_bytes(int64_t n) { return 3 * sizeof(int32_t) * (size_t)((n + kGrpRows - 1) / kGrpRows); }
 
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
-                             unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s) {
+                             unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s,
+                             uint32_t* event) {
   if (n <= 0) return cudaSuccess;
   const int64_t nb = (n + kGrpRows - 1) / kGrpRows;
   k_group_count<<<(unsigned)nb, kGrpThreads, 0, s>>>(time, status, n, model, nb, static_cast<int32_t*>(cnt), perr, K,
-                                                     total_events, ticket);
+                                                     total_events, ticket, event);
   return cudaGetLastError();
 }
 

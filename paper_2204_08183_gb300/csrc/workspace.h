@@ -18,7 +18,7 @@ struct surv_workspace {
   };
   enum Id {
     TIME, STATUS, COLPTR, ROWIDX, VALUES, XD, E, ETA, W2, GEND, DK, CK, GK, GKFF, WK0, WOFF, DTX, BETA, WIDTH, PEN, REC,
-    SLOTS, CTRL, BLOCKCNT, DTX_PART, ROWMASK, SORTWORK, PERM, PF, WT, AGG,
+    SLOTS, CTRL, BLOCKCNT, DTX_PART, ROWMASK, EVENTW, SORTWORK, PERM, PF, WT, AGG,
     // differentiable form (cox_nll_forward / cox_nll_backward)
     NLL_Y, NLL_BCAT, NLL_REC, NLL_WT, NLL_DEN, NLL_LAM, NLL_G, NLL_GB, NLL_GEND, NLL_DK, NLL_WK0, NLL_BLK,
     NLL_CTRL, NLL_XP, NLL_ERR, NLL_FIN, NLL_MASK,
@@ -74,9 +74,10 @@ bool nll_fused_fits(int64_t n, int p, int C);
 int64_t nll_fused_unit_rows(int64_t n, int units);
 cudaError_t nll_fused_split(const float* B, int64_t p, int C, int64_t ldx, void* BcatT, cudaStream_t s);
 cudaError_t nll_fused_forward(const void* X, int64_t n, int p, int64_t ldx, const void* BcatT, int C, int ctas,
-                              int64_t unit_rows, const RowMasks& m, float2* rec, float2* wt, float2* wd, unsigned* err,
+                              int64_t unit_rows, const RowMasks& m, const uint32_t* event, float2* rec, float2* wt, float2* wd, unsigned* err,
                               cudaStream_t s);
 cudaError_t nll_fused_backward(const void* X, int64_t n, int p, int64_t ldx, const void* BcatT, int C, int Cp, int K,
-                               const RowMasks& m, const float* lam, const double* gout, float* part, int nx,
+                               const RowMasks& m, const uint32_t* event, const float* lam,
+                               const double* gout, float* part, int nx,
                                float* grad_B, unsigned* err, cudaStream_t s);
 }  // namespace survgpu
