@@ -516,7 +516,9 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   CUDA_TRY(cudaMemcpyAsync(pen, pen_h.data(), 8 * (size_t)p, cudaMemcpyHostToDevice, s));
   bool any_beta = false;
   for (double b : beta_h) any_beta |= (b != 0.0);
-  if (!any_beta) {
+  if (cluster) {
+    // the cluster kernel starts from beta itself
+  } else if (!any_beta) {
     CUDA_TRY(survgpu::prep_eta_zero(prec, n, eta, e, s));
     ++launches;
   } else if (layout == SURV_DENSE) {
@@ -537,8 +539,8 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     CUDA_TRY(survgpu::prep_eta_exp(prec, n, eta, e, s));
     ++launches;
   }
-  CUDA_TRY(cudaMemsetAsync(slots, 0, 2 * slot_bytes, s));
-  {
+  if (!cluster) {
+    CUDA_TRY(cudaMemsetAsync(slots, 0, 2 * slot_bytes, s));
     const unsigned long long big = ~0ull;
     CUDA_TRY(cudaMemcpyAsync(&ctrl->timing[survgpu::PH_PASS_MIN], &big, sizeof(big), cudaMemcpyHostToDevice, s));
   }

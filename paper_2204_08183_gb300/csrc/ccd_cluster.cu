@@ -129,6 +129,20 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
   __syncthreads();
   cluster_arrive();   // every CTA of the cluster has started: its shared memory may be written
   cluster_wait();
+  if (dirty && rows) {
+    // eta = X beta and e on the warp's own rows, a column at a time (a launch
+    // per nonzero coefficient outside cost more than the evaluation it prepared)
+    using E = typename std::conditional<sizeof(T) == 4, float2, double>::type;
+    for (int64_t r = row_lo + lane; r < row_hi; r += 32) {
+      reinterpret_cast<E*>(P.eta)[r] = E{};
+      reinterpret_cast<T*>(P.e)[r] = T(1);
+    }
+    __syncwarp();
+    for (int i = 0; i < p; ++i) {
+      const double b = s_beta[i];
+      if (b != 0.0) warp_update<LAYOUT, T>(P, i, gw, row_lo, row_hi, b, d_to_ff(b));
+    }
+  }
 
   for (int sw = 0; sw < sweeps && !stop;) {
     const int q = j == 0 ? p - 1 : j - 1;

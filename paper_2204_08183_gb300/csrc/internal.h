@@ -204,7 +204,8 @@ cudaError_t replay_until_stop(const CcdParams& P, cudaStream_t s, GraphCache* gc
 constexpr int32_t kClusterMaxEnds = 32768;
 cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc);
 // Up to `sweeps` sweeps of a fit (or the evaluation of P.single_j) in one
-// launch; *P.gctl zeroed before the first.  P.gctl->done tells the stop.
+// launch; *P.gctl zeroed before the first, which also sets eta = X beta and e.
+// P.gctl->done tells the stop.
 cudaError_t run_cluster(int model, int layout, int prec, const CcdParams& P, int sweeps, cudaStream_t s);
 
 // ---- speculative coordinate batches (spec.cu) ----------------------------
