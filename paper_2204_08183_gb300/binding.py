@@ -363,18 +363,15 @@ def surv_groups(time, status, stream=None):
     """Tie-group table of sorted data: (gend int32[K], dk int32[K], Gk float64[K]) as numpy arrays."""
     n = int(time.shape[0])
     K = C.c_int64()
-    lib = load()
-    st = _stream(stream)
-    _check(lib.surv_groups(C.c_void_p(_ptr(time)), C.c_void_p(_ptr(status)), n, 0, C.byref(K), None, None, None, st))
+    # at most n groups: one call, which writes the first K entries only
+    gend = np.empty(n, np.int32)
+    dk = np.empty(n, np.int32)
+    Gk = np.empty(n, np.float64)
+    _check(load().surv_groups(C.c_void_p(_ptr(time)), C.c_void_p(_ptr(status)), n, n, C.byref(K),
+                              C.c_void_p(gend.ctypes.data), C.c_void_p(dk.ctypes.data), C.c_void_p(Gk.ctypes.data),
+                              _stream(stream)))
     k = K.value
-    gend = np.empty(k, np.int32)
-    dk = np.empty(k, np.int32)
-    Gk = np.empty(k, np.float64)
-    if k:
-        _check(lib.surv_groups(C.c_void_p(_ptr(time)), C.c_void_p(_ptr(status)), n, k, C.byref(K),
-                               C.c_void_p(gend.ctypes.data), C.c_void_p(dk.ctypes.data),
-                               C.c_void_p(Gk.ctypes.data), st))
-    return gend, dk, Gk
+    return gend[:k].copy(), dk[:k].copy(), Gk[:k].copy()
 
 
 def strerror(code: int) -> str:

@@ -21,6 +21,7 @@
 #include <cfloat>
 #include <climits>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 
@@ -316,27 +317,32 @@ __global__ void __launch_bounds__(kFinThreads) k_nll_finish(const float2* rec, c
     s_red[w][1] = sd;
   }
   __syncthreads();
-  if (tid == 0) {
-    double a = 0.0, b = 0.0;
-    for (int q = 0; q < kFinThreads / 32; ++q) {
-      a += s_red[q][0];
-      b += s_red[q][1];
-    }
-    part[((size_t)c * S + sc) * 2] = a;
-    part[((size_t)c * S + sc) * 2 + 1] = b;
+  // the two sums over the warps, each in order by a thread of its own
+  if (lane == 0 && w < 2) {
+    double a = 0.0;
+    for (int q = 0; q < kFinThreads / 32; ++q) a += s_red[q][w];
+    part[((size_t)c * S + sc) * 2 + w] = a;
     __threadfence();
-    s_last = atomicAdd(cnt + c, 1u) == (unsigned)(S - 1);
   }
   __syncthreads();
-  if (tid == 0 && s_last) {
+  if (tid == 0) {
+    s_last = atomicAdd(cnt + c, 1u) == (unsigned)(S - 1);
     __threadfence();
+  }
+  __syncthreads();
+  if (w == 0 && s_last) {
+    // lane q loads the sums of CTA q (S <= 8); added in the order q = 0 .. S - 1
+    const double av = lane < S ? __ldcg(part + ((size_t)c * S + lane) * 2) : 0.0;
+    const double bv = lane < S ? __ldcg(part + ((size_t)c * S + lane) * 2 + 1) : 0.0;
     double a = 0.0, b = 0.0;
     for (int q = 0; q < S; ++q) {
-      a += __ldcg(part + ((size_t)c * S + q) * 2);
-      b += __ldcg(part + ((size_t)c * S + q) * 2 + 1);
+      a += __shfl_sync(0xffffffffu, av, q);
+      b += __shfl_sync(0xffffffffu, bv, q);
     }
-    nll[c] = a - b;
-    cnt[c] = 0u;  // ready for the next forward
+    if (lane == 0) {
+      nll[c] = a - b;
+      cnt[c] = 0u;  // ready for the next forward
+    }
   }
 }
 
@@ -500,6 +506,7 @@ struct NllCtrl {
   int32_t K;
   int32_t total_events;
   unsigned ticket;
+  unsigned err;   // kept between calls: a bounded wait of the tensor-core kernels expired
 };
 
 // Row masks and event words of the fused form in the workspace.
@@ -550,7 +557,8 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   void *ctrl_v, *blk, *gend, *dk, *wk0, *Y, *Bcat, *rec, *wt, *den;
   NLL_TRY(ws_ensure(ws, W::NLL_CTRL, sizeof(NllCtrl), &ctrl_v));
   NllCtrl* ctrl = static_cast<NllCtrl*>(ctrl_v);
-  NLL_TRY(cuda_err(cudaMemsetAsync(ctrl, 0, sizeof(NllCtrl), s), "memset"));
+  NLL_TRY(cuda_err(cudaMemsetAsync(ctrl, 0, ws->nll_err_init ? offsetof(NllCtrl, err) : sizeof(NllCtrl), s), "memset"));
+  ws->nll_err_init = true;
   const int32_t* time = static_cast<const int32_t*>(d->time);
   const int8_t* status = static_cast<const int8_t*>(d->status);
   NLL_TRY(ws_ensure(ws, W::NLL_BLK, prep_count_bytes(n), &blk));
@@ -563,16 +571,12 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
                                     s, event),
                    "count groups"));
   NllCtrl hc;
-  unsigned prev_err = 0;
   NLL_TRY(cuda_err(cudaMemcpyAsync(&hc, ctrl, sizeof(hc), cudaMemcpyDeviceToHost, s), "copy"));
-  if (ws->nll_err_init)
-    NLL_TRY(cuda_err(cudaMemcpyAsync(&prev_err, ws->bufs[W::NLL_ERR].p, sizeof(unsigned), cudaMemcpyDeviceToHost, s),
-                     "copy"));
   NLL_TRY(cuda_err(cudaStreamSynchronize(s), "sync"));
-  if (prev_err) {
+  if (hc.err) {
     // a bounded wait of an earlier forward or backward on this workspace
     // expired: its results were not valid
-    NLL_TRY(cuda_err(cudaMemsetAsync(ws->bufs[W::NLL_ERR].p, 0, sizeof(unsigned), s), "memset"));
+    NLL_TRY(cuda_err(cudaMemsetAsync(&ctrl->err, 0, sizeof(unsigned), s), "memset"));
     set_last_error_text("a device-side wait of an earlier cox_nll call on this workspace expired");
     return SURV_E_DEVICE_TIMEOUT;
   }
@@ -609,12 +613,7 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
     Xt = xp;
   }
   NLL_TRY(ws_ensure(ws, W::NLL_BCAT, sizeof(__nv_bfloat16) * (size_t)std::max(128, 2 * Cp) * ld, &Bcat));
-  void* errw = nullptr;
-  NLL_TRY(ws_ensure(ws, W::NLL_ERR, sizeof(unsigned), &errw));
-  if (!ws->nll_err_init) {
-    NLL_TRY(cuda_err(cudaMemsetAsync(errw, 0, sizeof(unsigned), s), "memset"));
-    ws->nll_err_init = true;
-  }
+  unsigned* errw = &ctrl->err;
   NLL_TRY(ws_ensure(ws, W::NLL_REC, sizeof(float2) * (size_t)K * C, &rec));
   NLL_TRY(ws_ensure(ws, W::NLL_WT, 2 * sizeof(float2) * (size_t)nwarps * C, &wt));
   NLL_TRY(ws_ensure(ws, W::NLL_DEN, sizeof(double) * (size_t)K * C, &den));
@@ -622,20 +621,20 @@ int cox_nll_forward(const surv_nll_data* d, const float* B, double* nll, void* s
   if (fused) {
     NLL_TRY(cuda_err(nll_fused_split(B, p, C, ld, Bcat, s), "split B"));
     NLL_TRY(cuda_err(nll_fused_forward(Xt, n, (int)p, ld, Bcat, C, G, rpw, masks, event, static_cast<float2*>(rec),
-                                       wt2, wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw), s),
+                                       wt2, wt2 + (size_t)nwarps * C, errw, s),
                      "fused forward"));
   } else {
     NLL_TRY(ws_ensure(ws, W::NLL_Y, sizeof(float) * (size_t)n * C, &Y));
     const int64_t nbt = (int64_t)2 * Cp * ld;
     k_split_bt<<<(unsigned)((nbt + 255) / 256), 256, 0, s>>>(B, p, C, Cp, ld, static_cast<__nv_bfloat16*>(Bcat));
     NLL_TRY(cuda_err(cudaGetLastError(), "split B"));
-    NLL_TRY(cuda_err(nll_xb_tc(Xt, n, (int)p, ld, Bcat, C, Cp, static_cast<float*>(Y), static_cast<unsigned*>(errw), s),
+    NLL_TRY(cuda_err(nll_xb_tc(Xt, n, (int)p, ld, Bcat, C, Cp, static_cast<float*>(Y), errw, s),
                      "tensor-core X B"));
     const size_t ssm = stage_smem(C);
     NLL_TRY(cuda_err(cudaFuncSetAttribute(k_nll_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm), "smem"));
     k_nll_scan<<<G, kNllThreads, ssm, s>>>(static_cast<const float*>(Y), n, C, status, static_cast<int32_t*>(gend),
                                            static_cast<int32_t*>(wk0), rpw, static_cast<float2*>(rec), wt2,
-                                           wt2 + (size_t)nwarps * C, static_cast<unsigned*>(errw));
+                                           wt2 + (size_t)nwarps * C, errw);
     NLL_TRY(cuda_err(cudaGetLastError(), "scan"));
   }
   const size_t smem = sizeof(float2) * (size_t)nwarps;
@@ -705,7 +704,7 @@ int cox_nll_backward(const surv_nll_data* d, const double* grad_nll, float* grad
     NLL_TRY(nll_masks(ws, (n + 31) / 32, &masks, &event));
     return cuda_err(nll_fused_backward(ws->nll_xt, n, (int)p, ws->nll_ld, ws->bufs[W::NLL_BCAT].p, C, Cp, K, masks, event,
                                        static_cast<float*>(lam), grad_nll, static_cast<float*>(part), nx, grad_B,
-                                       static_cast<unsigned*>(ws->bufs[W::NLL_ERR].p), s),
+                                       &static_cast<NllCtrl*>(ws->bufs[W::NLL_CTRL].p)->err, s),
                     "fused backward");
   }
   NLL_TRY(ws_ensure(ws, W::NLL_G, sizeof(__nv_bfloat16) * (size_t)n * NB, &G2));
@@ -714,13 +713,13 @@ int cox_nll_backward(const surv_nll_data* d, const double* grad_nll, float* grad
   k_nll_grad<<<G, kNllThreads, ssm, s>>>(static_cast<const float*>(ws->bufs[W::NLL_Y].p), n, C, Cp,
                                          static_cast<const int8_t*>(d->status), gend, wk0, rpw,
                                          static_cast<float*>(lam), grad_nll, static_cast<__nv_bfloat16*>(G2),
-                                         static_cast<unsigned*>(ws->bufs[W::NLL_ERR].p));
+                                         &static_cast<NllCtrl*>(ws->bufs[W::NLL_CTRL].p)->err);
   NLL_TRY(cuda_err(cudaGetLastError(), "grad"));
   (void)nwarps;
   // grad_B = X^T [G_hi | G_lo] on the tensor cores, halves and CTA partials
   // summed in FP64 (nll_tc.cu)
   return cuda_err(nll_xtg_tc(ws->nll_xt, n, (int)p, ws->nll_ld, G2, C, Cp, static_cast<float*>(part), nx, grad_B,
-                             static_cast<unsigned*>(ws->bufs[W::NLL_ERR].p), s),
+                             &static_cast<NllCtrl*>(ws->bufs[W::NLL_CTRL].p)->err, s),
                   "tensor-core X^T G");
 }
 

@@ -21,7 +21,7 @@ struct surv_workspace {
     SLOTS, CTRL, BLOCKCNT, DTX_PART, ROWMASK, EVENTW, SORTWORK, PERM, PF, WT, AGG,
     // differentiable form (cox_nll_forward / cox_nll_backward)
     NLL_Y, NLL_BCAT, NLL_REC, NLL_WT, NLL_DEN, NLL_LAM, NLL_G, NLL_GB, NLL_GEND, NLL_DK, NLL_WK0, NLL_BLK,
-    NLL_CTRL, NLL_XP, NLL_ERR, NLL_FIN, NLL_MASK,
+    NLL_CTRL, NLL_XP, NLL_FIN, NLL_MASK,
     // cross-validated path (cox_cv_path) and lambda_max
     CV_FOLD, CV_DK, CV_DTX, CV_E, CV_ETA, CV_REC, CV_WT, CV_AGG, CV_PART, CV_GCTL, CV_BETA, CV_WIDTH, CV_PEN,
     CV_OUT, CV_FITS, CV_CTRL, CV_DEN, CV_HELD, CV_MEAN, LM_LAM, LM_R, LM_G,
@@ -30,6 +30,10 @@ struct surv_workspace {
     NBUF
   };
   int device = -1;
+  // Workspaces that live for one call take their buffers from the device's
+  // scratch pool, ordered on that call's stream (see ws_use_pool); null: cudaMalloc.
+  cudaMemPool_t pool = nullptr;
+  cudaStream_t pool_stream = nullptr;
   Buf bufs[NBUF];
   survgpu::GraphCache graph;  // instantiated sweep graph of the last fit
   // shape of the last cox_nll_forward (what cox_nll_backward continues from)
@@ -39,7 +43,7 @@ struct surv_workspace {
   const void* nll_xt = nullptr;   // X as the tensor-core kernels read it (padded copy if needed)
   int64_t nll_ld = 0;              // its row pitch in elements
   bool nll_fused = false;          // the forward ran in nll_fused.cu (no eta was kept)
-  bool nll_err_init = false;       // the tensor-core kernels' error word has been zeroed
+  bool nll_err_init = false;       // the tensor-core kernels' error word (in NLL_CTRL) has been zeroed
   // CTAs per fit chosen by the cross-validation tuner, and the shape it was
   // tuned for (n, p, fits, layout * 2 + precision, dtype, layout tag)
   int32_t cv_tuned_ctas = 0;
@@ -49,6 +53,8 @@ struct surv_workspace {
 };
 
 namespace survgpu {
+// Buffers of a one-call workspace come from the device's scratch pool.
+void ws_use_pool(surv_workspace* ws, cudaStream_t s);
 // Grow buffer `id` to at least `bytes` (api.cu); SURV_* error code.
 int ws_ensure(surv_workspace* ws, int id, size_t bytes, void** out);
 // Tensor-core products of the differentiable form (nll_tc.cu).  X: n rows of

@@ -103,3 +103,33 @@ def test_dense_and_weights_at_block_edges(lib, n):
     d = synth.cohort_small(n, 3, seed=n, n_times=max(1, n // 7), competing_frac=0.3)
     d["status"][0] = 1
     _against_oracle("fg", d, np.asarray(d["X"]), True, "dense", range(3))
+
+
+def test_one_call_scratch_from_threads_and_streams(lib):
+    """Calls without a workspace share the device's scratch pool: several
+    threads on streams of their own, sizes that grow and shrink."""
+    import threading
+
+    import torch
+    sizes = [1000, 300_000, 5000, 1_200_000]
+    times = [torch.randint(1, 3650, (n,), dtype=torch.int32, device="cuda") for n in sizes]
+    refs = [oracle.sort_desc(t.cpu().numpy()).astype(np.int32) for t in times]
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(k):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            for r in range(12):
+                i = (k + r) % len(sizes)
+                perm = binding.surv_sort_desc(times[i])
+                st.synchronize()
+                if not np.array_equal(perm.cpu().numpy(), refs[i]):
+                    bad.append((k, r))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
