@@ -959,7 +959,7 @@ int cv_impl(const surv_data* d, const int8_t* fold_id, int nfolds, const double*
   void *gend, *dk, *wk0, *woff = nullptr, *dkf, *dtxf, *cvc_v;
   void *e, *eta, *rec, *wt, *agg, *part, *gctl, *beta, *width, *pen, *out, *fits, *den, *held, *mean;
   const size_t rec_f = pad((size_t)K * RC, 8), wt_f = pad((size_t)RC * nwarps_alloc, 8);
-  const size_t agg_f = pad((size_t)RC * Galloc, 8), part_f = pad((size_t)NPART * Galloc, 8);
+  const size_t agg_f = pad((size_t)RC * Galloc, 8), part_f = pad((size_t)NPART * survgpu::kMaxTransCtas, 8);
   if ((rc = ensure(ws, W::GEND, 4 * (size_t)K, &gend))) return rc;
   if ((rc = ensure(ws, W::DK, 4 * (size_t)K, &dk))) return rc;
   if ((rc = ensure(ws, W::WK0, 4 * (size_t)(nwarps_alloc + 1), &wk0))) return rc;

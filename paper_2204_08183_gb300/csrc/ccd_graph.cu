@@ -7,14 +7,13 @@
 //               own rows, then runs the row pass (step 2) of coordinate j
 //               over those rows and the CTA publishes its warp totals and its
 //               aggregate.
-//   k_trans(j)  every CTA sums the aggregates of the CTAs before it (its
-//               exclusive prefix) in a fixed order, transforms its group ends
-//               (steps 3-4) and publishes three partial sums.  The last CTA
-//               to finish (atomic ticket; nobody waits for it) sums the
-//               partials in a fixed order, takes the FP64 Newton step of
-//               Section 2.4, stores beta_j and its trust-region width, on
-//               j = 0 evaluates the objective and the stopping rule, and
-//               publishes the step for k_pass(j + 1).
+//   k_btrans(j) every CTA scans the aggregates in a fixed order, transforms its
+//               share of the group ends (steps 3-4) and publishes three
+//               partial sums.  The last CTA to finish (atomic ticket; nobody
+//               waits for it) sums the partials in a fixed order, takes the
+//               FP64 Newton step of Section 2.4, stores beta_j and its
+//               trust-region width, on j = 0 evaluates the objective and the
+//               stopping rule, and publishes the step for k_pass(j + 1).
 //
 // Kernel boundaries order every producer before its consumers: no kernel
 // waits on another CTA.  A warp only reads and writes eta / e on its own
@@ -51,8 +50,6 @@ struct GCfg {
   static constexpr int U = (MODEL == 1 && LAYOUT == 1) ? 1 : (MODEL == 1 || LAYOUT == 1 ? 2 : 4);
   static constexpr int SR = 4;
 };
-constexpr int kTransThreads = 256;
-constexpr int kTransWarps = kTransThreads / 32;
 
 // Fill every control line for the first coordinate of a fit (of fit
 // blockIdx.y in a batched launch).
@@ -179,250 +176,14 @@ __global__ void __launch_bounds__(GCfg<MODEL, LAYOUT>::NT, GCfg<MODEL, LAYOUT>::
   }
 }
 
-// Latency-bound: every load that does not depend on another value of this
-// kernel is issued first (CTA aggregates, this CTA's warp totals, its group
-// ends), the several sums of each stage share one reduction tree, and the
-// common path (at most one group end per thread) has one block barrier
-// before the partials.
-template <int MODEL, int LAYOUT, typename T, bool BATCH>
-__global__ void __launch_bounds__(kTransThreads) k_trans(const __grid_constant__ CcdParams P0, int j) {
-  using A = typename AccOf<T>::type;
-  constexpr int M = MODEL == 0 ? 3 : 6;
-  // prefix sums of the M components (+ for Fine-Gray the grand totals of
-  // the three suffix components 3..5, which the transform subtracts from)
-  constexpr int NA = MODEL == 0 ? M : M + 3;
-  constexpr int NT = kTransThreads;
-  __shared__ A s_wp[kTransWarps][NA];
-  __shared__ A s_tc[NA];
-  __shared__ A s_base[kMaxWarpsPerCta][M];
-  __shared__ A s_red[kTransWarps][3];
-  __shared__ int s_last;
-  __shared__ int s_stopped;
-  __shared__ double s_lin[2];
-  __shared__ double s_next[4];
-  __shared__ CcdParams s_fit;
-  if (BATCH) load_fit(s_fit, P0);
-  const CcdParams& P = BATCH ? s_fit : P0;
-
-  GraphCtl* ctl = P.gctl;
-  const int tid = threadIdx.x;
-  const int lane = tid & 31;
-  const int w = tid >> 5;
-  const int WPC = P.wpc;
-  const int c = blockIdx.x;
-  const int G = P.G;
-  const bool eval = j == 0;
-  const int kc_lo = P.wk0[c * WPC], kc_hi = P.wk0[(c + 1) * WPC];
-  const int nends = kc_hi - kc_lo;
-  const bool one_end = nends <= NT;
-
-  // ---------------------------------------------- static loads
-  int kd = 0, kge = 0;
-  double kg = 0.0;
-  float2 kgf = make_float2(0.f, 0.f);
-  if (one_end && tid < nends) {
-    const int k = kc_lo + tid;
-    kd = P.dk[k];
-    kge = P.gend[k];
-    if (MODEL == 1) {
-      kg = P.Gk[k];
-      kgf = P.Gkff[k];
-    }
-  }
-  pdl_wait();
-
-  // ------------------ every load of this kernel's inputs, in one round trip
-  // (thread 0 also reads the control line: stop flag and the scalars of j)
-  LineView lv;
-  if (tid == 0) {
-    lv = load_line(ctl, c);
-    s_stopped = lv.stop;
-  }
-  const uint64_t* agg = P.agg;
-  // warp of this thread's group end (relative to the CTA); the pass kernel
-  // stored each warp's offset inside the CTA in wt
-  const int wl = (one_end && tid < nends) ? (int)((kge >> 5) / P.wpw) - c * WPC : (tid < WPC ? tid : 0);
-  uint64_t v0[M], v1[M], wbv[M];
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    v0[m] = tid < G ? __ldcg(agg + (size_t)m * G + tid) : 0ull;
-    v1[m] = tid + NT < G ? __ldcg(agg + (size_t)m * G + tid + NT) : 0ull;
-    wbv[m] = ((one_end && tid < nends) || (!one_end && tid < WPC))
-                 ? __ldcg(P.wt + (size_t)m * P.nwarps + c * WPC + wl)
-                 : 0ull;
-  }
-  const A* rec = reinterpret_cast<const A*>(P.rec);
-  A kr[M];
-  if (one_end && tid < nends)
-#pragma unroll
-    for (int m = 0; m < M; ++m) kr[m] = rec[(size_t)(kc_lo + tid) * M + m];
-
-  // ------------------- per-warp sums of the aggregates of CTAs before c
-  {
-    A r[NA];
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const A x0 = unpack8<A>(v0[m]), x1 = unpack8<A>(v1[m]);
-      acc_zero(r[m]);
-      if (tid < c) r[m] = x0;
-      if (tid + NT < c) r[m] = acc_add(r[m], x1);
-      if (MODEL == 1 && m >= 3) r[M + m - 3] = acc_add(x0, x1);
-    }
-    for (int qc = tid + 2 * NT; qc < G; qc += NT)  // grids above 512 CTAs
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const A x = unpack8<A>(__ldcg(agg + (size_t)m * G + qc));
-        if (qc < c) r[m] = acc_add(r[m], x);
-        if (MODEL == 1 && m >= 3) r[M + m - 3] = acc_add(r[M + m - 3], x);
-      }
-    warp_sum_n<NA>(r);
-    if (lane == 0)
-#pragma unroll
-      for (int i = 0; i < NA; ++i) s_wp[w][i] = r[i];
-  }
-  __syncthreads();
-  if (BATCH && s_stopped) return;  // this fit has stopped (the others go on)
-  // prefix before CTA c and (Fine-Gray) grand totals: thread i sums value i
-  // over the warps in a fixed order, once for the CTA
-  if (tid < NA) {
-    A t = s_wp[0][tid];
-#pragma unroll 1
-    for (int qw = 1; qw < kTransWarps; ++qw) t = acc_add(t, s_wp[qw][tid]);
-    s_tc[tid] = t;
-  }
-  __syncthreads();
-  A T_c[M], tot[M];
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    T_c[m] = s_tc[m];
-    if (MODEL == 1 && m >= 3) tot[m] = s_tc[M + m - 3];
-    else acc_zero(tot[m]);
-  }
-
-  // ---------------------------------------------- steps 3-4
-  A fg1, fg2;
-  acc_zero(fg1);
-  acc_zero(fg2);
-  double pl = 0.0;
-  auto end_terms = [&](int d, const A (&Pm)[M], double g, float2 gf) {
-    A den = Pm[0], num1 = Pm[1], num2 = Pm[2];
-    if (MODEL == 1) {
-      const A gg = acc_base<A>(g, ff{gf.x, gf.y});
-      den = acc_add(den, acc_mul(gg, acc_add(tot[3 % M], acc_neg(Pm[3 % M]))));
-      num1 = acc_add(num1, acc_mul(gg, acc_add(tot[4 % M], acc_neg(Pm[4 % M]))));
-      num2 = acc_add(num2, acc_mul(gg, acc_add(tot[5 % M], acc_neg(Pm[5 % M]))));
-    }
-    const A inv = acc_recip(den);
-    const A Gr = acc_mul(num1, inv);
-    const A H = acc_mul(num2, inv);
-    fg1 = acc_add(fg1, acc_scale(Gr, d));
-    fg2 = acc_add(fg2, acc_scale(acc_add(H, acc_neg(acc_mul(Gr, Gr))), d));
-    if (eval) pl += (double)d * log(acc_to_d(den));
-  };
-  if (one_end) {
-    if (kd != 0) {
-      // prefix at the end: CTAs before, the CTA's warps before, the warp's rows
-      A Pm[M];
-#pragma unroll
-      for (int m = 0; m < M; ++m) Pm[m] = acc_add(acc_add(T_c[m], unpack8<A>(wbv[m])), kr[m]);
-      end_terms(kd, Pm, kg, kgf);
-    }
-  } else {
-    if (tid < WPC)
-#pragma unroll
-      for (int m = 0; m < M; ++m) s_base[tid][m] = acc_add(T_c[m], unpack8<A>(wbv[m]));
-    __syncthreads();
-    for (int k = kc_lo + tid; k < kc_hi; k += NT) {
-      const int d = P.dk[k];
-      if (d == 0) continue;
-      const int wl = (int)((P.gend[k] >> 5) / P.wpw) - c * WPC;
-      A Pm[M];
-#pragma unroll
-      for (int m = 0; m < M; ++m) Pm[m] = acc_add(s_base[wl][m], rec[(size_t)k * M + m]);
-      end_terms(d, Pm, MODEL == 1 ? P.Gk[k] : 0.0, MODEL == 1 ? P.Gkff[k] : make_float2(0.f, 0.f));
-    }
-  }
-
-  // ------------------------------------------- CTA partials, fixed order
-  {
-    A r[3] = {fg1, fg2, eval ? acc_from_d(pl, (A*)nullptr) : A{}};
-    warp_sum_n<3>(r);
-    if (lane == 0)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) s_red[w][i] = r[i];
-  }
-  __syncthreads();
-  uint64_t* part = reinterpret_cast<uint64_t*>(P.slot_part);
-  if (tid == 0) {
-    A a[3] = {s_red[0][0], s_red[0][1], s_red[0][2]};
-#pragma unroll 1
-    for (int qw = 1; qw < kTransWarps; ++qw)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) a[i] = acc_add(a[i], s_red[qw][i]);
-    if (lv.stop) {
-      s_last = 0;  // the fit has stopped: nothing to publish
-    } else {
-      part[c] = pack8(a[0]);
-      part[G + c] = pack8(a[1]);
-      part[2 * G + c] = pack8(a[2]);
-      // release: the partials above are visible to whoever sees the count
-      unsigned prev;
-      asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&ctl->ticket) : "memory");
-      s_last = prev == (unsigned)(G - 1);
-    }
-  }
-  pdl_launch_dependents();
-  __syncthreads();
-  if (!s_last) return;
-
-  // ------------------------------- last CTA: the step of coordinate j
-  if (w < 3) {
-    // warp m sums partial vector m over the CTAs in a fixed order (acquire:
-    // every other CTA released its partials before its count)
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    A acc;
-    acc_zero(acc);
-    for (int q0 = 0; q0 < G; q0 += 32 * 10) {
-      uint64_t v[10];
-#pragma unroll
-      for (int u = 0; u < 10; ++u) {
-        const int qc = q0 + 32 * u + lane;
-        v[u] = qc < G ? __ldcg(part + (size_t)w * G + qc) : 0ull;
-      }
-#pragma unroll
-      for (int u = 0; u < 10; ++u) acc = acc_add(acc, unpack8<A>(v[u]));
-    }
-    A r[1] = {acc};
-    warp_sum_n<1>(r);
-    if (lane == 0) s_red[0][w] = r[0];
-  } else if (w == 3 && eval) {
-    // objective pieces at the current beta (every earlier step is stored)
-    double lin, pen;
-    warp_lin_pen(P, -1, 0.0, lin, pen);
-    if (lane == 0) {
-      s_lin[0] = lin;
-      s_lin[1] = pen;
-    }
-  } else if (w == 4 && lane == 0) {
-    // scalars of the next coordinate, for the control line
-    const int jn = j + 1 < P.p ? j + 1 : 0;
-    s_next[0] = __ldcg(P.beta + jn);
-    s_next[1] = __ldcg(P.width + jn);
-    s_next[2] = P.pen[jn];
-    s_next[3] = P.dTx[jn];
-  }
-  __syncthreads();
-  if (w == 0)
-    publish_step(P, j, lv, lv.dtx - acc_to_d(s_red[0][0]), -acc_to_d(s_red[0][1]), eval, s_lin[0],
-                 s_lin[1], acc_to_d(s_red[0][2]), s_next);
-}
-
-// Transform of single fits with the work spread evenly: every CTA scans the
+// The transform, its work spread evenly: every CTA scans the
 // pass CTAs' aggregates (one per thread, two-level warp scans in shared
 // memory; Fine-Gray also takes the grand totals of the suffix components)
-// and takes an even share of the group ends, about one a thread.  The
-// per-CTA range split of k_trans gave the CTAs holding the first rows (many
-// small tie groups) most of the work.  It reads the control line and its
+// and takes an even share of the group ends, about one a thread (batched fits:
+// about four).  A split by pass CTA gave the CTAs holding the first rows (many
+// small tie groups) most of the work; and with a CTA per pass CTA and one end
+// a thread, the reductions of 200 batched fits cost more than their ends (50
+// us of a coordinate's 280 at n = 10^6).  It reads the control line and its
 // first end's group table entries before the wait: the line was written by
 // the previous coordinate's transform, which finished before this
 // coordinate's pass kernel passed its own wait.
@@ -435,11 +196,11 @@ __global__ void __launch_bounds__(kTransThreads) k_trans(const __grid_constant__
 // 128 threads on every SM walk 16 ends each).
 constexpr int kBtSmall = 128, kBtLarge = 512;
 constexpr int kBtMaxG = 384;   // pass CTAs
-constexpr int kBtMaxCtas = 152;
+constexpr int kBtMaxCtas = kMaxTransCtas;
 inline int btrans_threads(int K) { return K <= kBtSmall * kBtMaxCtas ? kBtSmall : kBtLarge; }
 
-template <int MODEL, int LAYOUT, typename T, int kBtNT>
-__global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ CcdParams P, int j) {
+template <int MODEL, int LAYOUT, typename T, int kBtNT, bool BATCH = false>
+__global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ CcdParams P0, int j) {
   using A = typename AccOf<T>::type;
   constexpr int M = MODEL == 0 ? 3 : 6;
   constexpr int kBtWarps = kBtNT / 32, kAgg = kBtNT == kBtSmall ? 3 : 1;
@@ -450,6 +211,9 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
   __shared__ int s_last, s_stop;
   __shared__ double s_lin[2];
   __shared__ double s_next[4];
+  __shared__ CcdParams s_fit;
+  if (BATCH) load_fit(s_fit, P0);
+  const CcdParams& P = BATCH ? s_fit : P0;
   GraphCtl* ctl = P.gctl;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int WPC = P.wpc, G = P.G, G2 = gridDim.x, c2 = blockIdx.x;
@@ -484,7 +248,7 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
     }
   }
   __syncthreads();
-  if (s_stop) {  // the same value in every CTA
+  if (s_stop) {  // the same value in every CTA of the fit
     pdl_wait();
     return;
   }
@@ -601,6 +365,10 @@ inline int btrans_ctas(int K) {
   const int nt = btrans_threads(K);
   return std::max(4, std::min(kBtMaxCtas, (K + nt - 1) / nt));
 }
+// Per fit of a batch: about four ends a thread (kBtSmall threads).
+inline int btrans_ctas_batch(int K) {
+  return std::max(1, std::min(kBtMaxCtas, (K + 4 * kBtSmall - 1) / (4 * kBtSmall)));
+}
 
 // Grid of the pass kernel: as many CTAs per SM (up to MINB) as fit.
 template <int MODEL, int LAYOUT, typename T>
@@ -622,6 +390,7 @@ cudaError_t grid_graph(int* G, int* wpc) {
 template <int MODEL, int LAYOUT, typename T>
 cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGraph_t* g) {
   using GC = GCfg<MODEL, LAYOUT>;
+  if (P.G > kBtMaxG) return cudaErrorInvalidValue;   // the transform scans three aggregates a thread at most
   cudaError_t st = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (st != cudaSuccess) return st;
   cudaLaunchAttribute attr[1];
@@ -634,7 +403,6 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   cp.attrs = attr;
   cp.numAttrs = 1;
   cudaLaunchConfig_t ct = cp;
-  ct.blockDim = dim3(kTransThreads);
   // batched fits: Cox only (the censoring weights of Fine-Gray would have
   // to be re-estimated on each training set)
   // The many-ends form of the row pass where warps hold two group ends or
@@ -647,7 +415,9 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps;
   const bool few_rows = P.nfit == 0 && P.wpw <= 16 && (Cfg<MODEL, LAYOUT, T>::ND > 1 || sizeof(T) == 8);
   auto kp = k_pass<MODEL, LAYOUT, T, false, false>;
-  auto kt = k_trans<MODEL, LAYOUT, T, false>;
+  auto kt = btrans_threads(P.K) == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;
+  ct.gridDim = dim3(btrans_ctas(P.K));
+  ct.blockDim = dim3(btrans_threads(P.K));
   if constexpr (MODEL == 0) {
     const bool multi = P.pass_form == 2 || (P.pass_form == 0 && (many || few_rows));
     if (P.nfit > 0) {
@@ -659,7 +429,9 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
         if (P.tile_form == 2)
           kp = multi ? k_pass<MODEL, LAYOUT, T, true, true, 2> : k_pass<MODEL, LAYOUT, T, true, false, 2>;
       }
-      kt = k_trans<MODEL, LAYOUT, T, true>;
+      kt = k_btrans<MODEL, LAYOUT, T, kBtSmall, true>;
+      ct.gridDim = dim3(btrans_ctas_batch(P.K), P.nfit);
+      ct.blockDim = dim3(kBtSmall);
     } else if (multi) {
       kp = k_pass<MODEL, LAYOUT, T, false, true>;
     }
@@ -671,12 +443,6 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
       if (junk) cudaGraphDestroy(junk);
       return cudaErrorInvalidValue;
     }
-  }
-  // single fits: the balanced transform (up to kBtMaxG pass CTAs)
-  if (P.nfit == 0 && P.G <= kBtMaxG) {
-    kt = btrans_threads(P.K) == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;
-    ct.gridDim = dim3(btrans_ctas(P.K));
-    ct.blockDim = dim3(btrans_threads(P.K));
   }
   cudaError_t lst = cudaSuccess;
   for (int j = 0; j < P.p && lst == cudaSuccess; ++j) {

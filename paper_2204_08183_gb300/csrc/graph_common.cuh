@@ -62,7 +62,7 @@ __device__ __forceinline__ void scan_aggregates(const uint64_t* agg, int G, A (*
 #pragma unroll
     for (int a = 1; a < AGG; ++a) t[m] = acc_add(t[m], v[a][m]);
   }
-  warp_scan_n<NV>(t, lane);
+  if (w * 32 * AGG < G) warp_scan_n<NV>(t, lane);   // (the other warps hold zeros)
   if (lane == 31)
 #pragma unroll
     for (int m = 0; m < NV; ++m) s_w[w][m] = t[m];

@@ -100,6 +100,7 @@ struct CcdParams {
 // a kernel reads line c % kRep once, so no line has more than a handful of
 // readers.
 constexpr int kRep = 32;
+constexpr int kMaxTransCtas = 152;   // CTAs of a transform (a partial sum each)
 struct alignas(128) CtlLine {
   int32_t stop;          // the fit has stopped: every later kernel returns
   int32_t nevals;        // objective evaluations so far (one per sweep)
