@@ -97,6 +97,40 @@ def test_columns_of_every_length(lib, values):
     _against_oracle("cox", d, X, values, "csc", range(len(lengths)))
 
 
+# four entries a load, and columns that start and end inside one: a fault is
+# found at every place
+@pytest.mark.parametrize("values", [None, "ones", "real"])
+@pytest.mark.parametrize("first", [0, 1, 3, 4])
+def test_faults_at_every_entry(lib, first, values):
+    rng = np.random.default_rng(first)
+    n, k = 300, 22
+    time = np.arange(n, 0, -1).astype(np.int32)
+    status = (rng.random(n) < 0.6).astype(np.int8)
+    rows = np.concatenate([np.sort(rng.choice(n, m, replace=False)) for m in (first, k, 5)]).astype(np.int32)
+    col_ptr = np.array([0, first, first + k, first + k + 5], dtype=np.int64)
+    vals = None if values is None else (np.ones(len(rows)) if values == "ones" else rng.normal(size=len(rows)))
+
+    def code(rows, vals):
+        d = binding.SurvData(time, status, col_ptr=col_ptr, row_idx=rows, values=vals, n=n, p=3)
+        try:
+            binding.cox_lambda_max(d)
+        except binding.SurvError as e:
+            return e.code
+        return 0
+
+    assert code(rows, vals) == 0
+    for i in range(first, first + k):
+        for bad in ([-1, n] if i == first else [-1, n, rows[i - 1]]):
+            r = rows.copy()
+            r[i] = bad
+            assert code(r, vals) == binding.SURV_E_INDEX, (i, bad)
+        if vals is not None:
+            for bad in (np.nan, np.inf):
+                v = vals.copy()
+                v[i] = bad
+                assert code(rows, v) == binding.SURV_E_NONFINITE, (i, bad)
+
+
 @pytest.mark.parametrize("n", [1, 5, 127, 4095, 4097, 8193, 20003])
 def test_dense_and_weights_at_block_edges(lib, n):
     from paper_2204_08183_gb300 import synth
