@@ -196,10 +196,19 @@ __global__ void __launch_bounds__(GCfg<MODEL, LAYOUT>::NT, GCfg<MODEL, LAYOUT>::
 // 128 threads on every SM walk 16 ends each).
 constexpr int kBtSmall = 128, kBtLarge = 512;
 constexpr int kBtMaxG = 384;   // pass CTAs
+
+// Up to 4096 ends a single fit's transform is one cluster of at most 16 CTAs
+// (two ends a thread), whose partial sums meet in the first CTA's shared
+// memory at a cluster barrier: the fence, the ticket and the way through L2
+// that other transforms end with take 1 us longer (ms a fit with the ticket
+// and the cluster: 10.02 and 9.76 for Fine-Gray at 5 x 10^6 x 50,
+// 1000 ends; 2.32 and 2.25 for dense Cox at 500,009 x 24, 3650 ends).
+constexpr int kBtCluster = 16;
+inline bool btrans_one_cluster(int K) { return K <= 2 * kBtSmall * kBtCluster; }
 constexpr int kBtMaxCtas = kMaxTransCtas;
 inline int btrans_threads(int K) { return K <= kBtSmall * kBtMaxCtas ? kBtSmall : kBtLarge; }
 
-template <int MODEL, int LAYOUT, typename T, int kBtNT, bool BATCH = false>
+template <int MODEL, int LAYOUT, typename T, int kBtNT, bool BATCH = false, bool CLUSTER = false>
 __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ CcdParams P0, int j) {
   using A = typename AccOf<T>::type;
   constexpr int M = MODEL == 0 ? 3 : 6;
@@ -211,7 +220,9 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
   __shared__ int s_last, s_stop;
   __shared__ double s_lin[2];
   __shared__ double s_next[4];
+  __shared__ uint64_t s_part[CLUSTER ? 3 * kBtCluster : 1];   // the CTAs' partials (in the first CTA)
   __shared__ CcdParams s_fit;
+  if (CLUSTER) cluster_arrive();   // this CTA has started
   if (BATCH) load_fit(s_fit, P0);
   const CcdParams& P = BATCH ? s_fit : P0;
   GraphCtl* ctl = P.gctl;
@@ -248,6 +259,7 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
     }
   }
   __syncthreads();
+  if (CLUSTER) cluster_wait();
   if (s_stop) {  // the same value in every CTA of the fit
     pdl_wait();
     return;
@@ -319,25 +331,37 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
     A a = s_red[0][tid];
 #pragma unroll 1
     for (int qw = 1; qw < kBtWarps; ++qw) a = acc_add(a, s_red[qw][tid]);
-    part[(size_t)tid * G2 + c2] = pack8(a);
+    if (CLUSTER) store_remote(&s_part[tid * kBtCluster + c2], 0, pack8(a));
+    else part[(size_t)tid * G2 + c2] = pack8(a);
   }
-  __syncthreads();
-  if (tid == 0) {
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    unsigned prev;
-    asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&ctl->ticket) : "memory");
-    s_last = prev == (unsigned)(G2 - 1);
+  if (CLUSTER) {
+    cluster_arrive();
+    pdl_launch_dependents();
+    cluster_wait();
+    if (c2 != 0) return;
+  } else {
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      unsigned prev;
+      asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&ctl->ticket) : "memory");
+      s_last = prev == (unsigned)(G2 - 1);
+    }
+    pdl_launch_dependents();
+    __syncthreads();
+    if (!s_last) return;
   }
-  pdl_launch_dependents();
-  __syncthreads();
-  if (!s_last) return;
 
   // ------------------------------- last CTA: the step of coordinate j
   if (w < 3) {
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
     A acc;
     acc_zero(acc);
-    for (int qc = lane; qc < G2; qc += 32) acc = acc_add(acc, unpack8<A>(__ldcg(part + (size_t)w * G2 + qc)));
+    if (CLUSTER) {
+      if (lane < G2) acc = acc_add(acc, unpack8<A>(s_part[w * kBtCluster + lane]));
+    } else {
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      for (int qc = lane; qc < G2; qc += 32) acc = acc_add(acc, unpack8<A>(__ldcg(part + (size_t)w * G2 + qc)));
+    }
     A r[1] = {acc};
     warp_sum_n<1>(r);
     if (lane == 0) s_red[0][w] = r[0];
@@ -391,11 +415,15 @@ template <int MODEL, int LAYOUT, typename T>
 cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGraph_t* g) {
   using GC = GCfg<MODEL, LAYOUT>;
   if (P.G > kBtMaxG) return cudaErrorInvalidValue;   // the transform scans three aggregates a thread at most
-  cudaError_t st = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-  if (st != cudaSuccess) return st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+  const unsigned cl = (unsigned)std::min(kBtCluster, btrans_ctas(P.K));
+  cudaLaunchAttribute attr_cl[2];
+  const bool cluster = P.nfit == 0 && btrans_one_cluster(P.K) &&
+                       cluster_launch(k_btrans<MODEL, LAYOUT, T, kBtSmall, false, true>, cl, kBtSmall, attr[0], attr_cl);
+  cudaError_t st = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+  if (st != cudaSuccess) return st;
   cudaLaunchConfig_t cp = {};
   cp.gridDim = dim3(P.G, P.nfit > 0 ? P.nfit : 1);
   cp.blockDim = dim3(GC::NT);
@@ -418,6 +446,12 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   auto kt = btrans_threads(P.K) == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;
   ct.gridDim = dim3(btrans_ctas(P.K));
   ct.blockDim = dim3(btrans_threads(P.K));
+  if (cluster) {
+    kt = k_btrans<MODEL, LAYOUT, T, kBtSmall, false, true>;
+    ct.gridDim = dim3(cl);
+    ct.attrs = attr_cl;
+    ct.numAttrs = 2;
+  }
   if constexpr (MODEL == 0) {
     const bool multi = P.pass_form == 2 || (P.pass_form == 0 && (many || few_rows));
     if (P.nfit > 0) {

@@ -116,6 +116,24 @@ __device__ __forceinline__ void load_fit(CcdParams& dst, const CcdParams& P0) {
   __syncthreads();
 }
 
+// Thread-block clusters.
+// (.aligned: the lanes of a warp arrive and wait together)
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// store an 8-byte accumulator at the address that `local` has in CTA `rank`
+__device__ __forceinline__ void store_remote(const void* local, unsigned rank, uint64_t v) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(local);
+  uint32_t ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(ra), "l"(v) : "memory");
+}
+
 // The step of coordinate j, taken by warp 0 of the kernel's last CTA
 // (Section 2.4): lane 0 gets l' (grad) and l'' (hess); on an evaluation pass
 // (eval, j = 0) the objective f = lin - sum_dlog + pen at the start of the
@@ -208,6 +226,26 @@ __device__ __forceinline__ void publish_step(const CcdParams& P, int j, const Li
   }
 }
 
+
+// Attributes of a launch of k as one cluster of `ctas` CTAs beside the launch's
+// own attribute; false where the device cannot place such a cluster.
+template <typename K>
+bool cluster_launch(K k, unsigned ctas, unsigned threads, const cudaLaunchAttribute& own, cudaLaunchAttribute (&at)[2]) {
+  at[0] = own;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim = {ctas, 1, 1};
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(ctas);
+  c.blockDim = dim3(threads);
+  c.attrs = at + 1;
+  c.numAttrs = 1;
+  int num = 0;
+  if ((ctas <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+      cudaOccupancyMaxActiveClusters(&num, k, &c) == cudaSuccess)
+    return num >= 1;
+  cudaGetLastError();
+  return false;
+}
 
 }  // namespace ccdk
 }  // namespace survgpu
