@@ -81,13 +81,12 @@ def parse():
 # kernels as committed: per row pass of the headline batches (k_ipass<4> +
 # k_itrans<4>), per coordinate of the one-coordinate Cox schedule (k_pass +
 # k_btrans) and of the Fine-Gray fit (k_pass + k_btrans).
-TRAFFIC_IND_ROW_PASS = 17179904
-TRAFFIC_ONE_COORD = 2435456
-TRAFFIC_FG_COORD = 71040486
-# DRAM bytes of one autograd step's four big kernels at N = 2^20, p = 256,
-# 64 columns (k_xb_tc 764.5 MB, k_nll_scan 275.1 MB, k_nll_grad 490.0 MB,
-# k_xtg_tc 805.9 MB; one ncu capture each, cold caches)
-TRAFFIC_AG_STEP_N20 = 2335500000
+TRAFFIC_IND_ROW_PASS = 17028000
+TRAFFIC_ONE_COORD = 2439000
+TRAFFIC_FG_COORD = 72352000
+# DRAM bytes of one autograd step's two big kernels at N = 2^20, p = 256,
+# 64 columns (k_nll_fwd 563.4 MB, k_nll_bwd 545.7 MB)
+TRAFFIC_AG_STEP_N20 = 1109130000
 
 
 def workload(n, p):
@@ -348,7 +347,7 @@ def run_gpu(args, rank, world):
     value = sweeps_all / (t_max / 1e3)
 
     # Roofline of the dominant kernel.  The unit of work is one coordinate:
-    # the k_pass + k_trans pair (graph schedule) that reads e over all N rows
+    # the k_pass + k_btrans pair (graph schedule) that reads e over all N rows
     # and the column's CSC slice; its duration is the fit's CCD device time
     # (all graph replays, kernel gaps included) divided by the coordinate
     # passes.  Eta updates after nonzero steps are counted in the bytes.
@@ -556,14 +555,9 @@ def run_autograd(args, rank, world):
         torch.distributed.all_reduce(tt, op=torch.distributed.ReduceOp.MAX)
         t_max = float(tt.item())
     value = world * 1e3 / t_max
-    # minimal bytes: X read by both products, eta written by the forward and
-    # read by the backward
-    alg = 2 * (2 * n * p) + 2 * (4 * n * C)
-    # as implemented: X B reads X and writes eta; the forward scan reads eta;
-    # the backward reads eta, writes G (bf16, 2 Cp columns) and X^T G reads
-    # X and G
-    Cp = max(32, (C + 15) // 16 * 16)
-    moved = (2 * n * p + 4 * n * C) + 4 * n * C + (4 * n * C + 2 * n * 2 * Cp) + (2 * n * p + 2 * n * 2 * Cp)
+    # minimal bytes, and those of the implementation: X read once in each
+    # direction; eta and G stay on the chip
+    alg = moved = 2 * (2 * n * p)
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
@@ -576,21 +570,20 @@ def run_autograd(args, rank, world):
            "vs_baseline": None, "dtype": "bf16 X, f32 B/eta, f64 logs", "data": "synthetic",
            "config": {"workload": "cox_nll_autograd_n%d_p256_c64" % n, "n": n, "p": p, "columns": C,
                       "time_grid": 5000, "censoring": 0.3,
-                      "l2": "inputs larger than L2 (X 2 GiB, eta 1 GiB)"},
+                      "l2": "inputs larger than L2 (X 2 GiB)"},
            "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                         "frac": round(achieved / peak, 4),
-                        # DRAM bytes of k_xb_tc + k_nll_scan + k_nll_grad + k_xtg_tc
-                        # in one ncu capture at N = 2^20 (the products and the
-                        # scans move bytes in proportion to N), times 4; see
-                        # profiles/tcgen05_products_cox_nll_p256_c64.md and
-                        # profiles/k_nll_scan_k_nll_grad_n1m_c64.md
+                        # DRAM bytes of k_nll_fwd + k_nll_bwd in one ncu
+                        # capture at N = 2^20 (both move bytes in proportion
+                        # to N), times 4; see
+                        # profiles/k_nll_fwd_k_nll_bwd_n1m_c64.md
                         "traffic": (TRAFFIC_AG_STEP_N20 * n // (1 << 20)) if p == 256 and C == 64 else None,
                         "traffic_note": "bytes per step, ncu capture at N=2^20 scaled by N",
                         "algorithmic_bytes_per_step": alg, "implementation_bytes_per_step": moved,
                         "forward_ms": round(fwd_ms, 3), "backward_ms": round(t_max - fwd_ms, 3),
-                        "kernel": "tcgen05 products k_xb_tc (X B) and k_xtg_tc (X^T G), TMA + TMEM, "
-                                  "+ k_nll_scan/finish/lambda/grad"},
-           "clocks": clk, "gpu_launches": args.steps * 14}
+                        "kernel": "tcgen05 k_nll_fwd (X B, risk-set scan) and k_nll_bwd (X B, G, X^T G), TMA + TMEM, "
+                                  "+ k_nll_finish/lambda, k_xtg_reduce"},
+           "clocks": clk, "gpu_launches": args.steps * 8}
     if not args.no_e2e:
         # autograd function, inputs copied from pinned host memory every step
         hX = X.cpu().pin_memory()
@@ -738,7 +731,7 @@ def run_cv(args, rank, world):
                       "l2": "inputs larger than L2 (e + eta of 200 fits: 2.4 GB)"},
            "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                         "frac": round(achieved / peak, 4), "traffic": None,
-                        "traffic_note": "not a whole-path figure: a capture of early launches (all 200 fits active, most passes streaming e) read 440-540 MB and wrote 56-78 MB a launch; see profiles/k_pass_batched_cv_n1e6.md",
+                        "traffic_note": "not a whole-path figure: a capture of early launches (all 200 fits active, most passes streaming e) read 441-541 MB and wrote 56-79 MB a launch; see profiles/k_pass_batched_cv_n1e6.md",
                         "unit_of_work": "one coordinate of one active fit (batched row pass)",
                         "algorithmic_bytes_per_coordinate": round(alg / max(passes, 1)),
                         "coordinate_passes_per_step": passes / len(infos),
@@ -746,7 +739,7 @@ def run_cv(args, rank, world):
                         "ccd_ms_per_step": round(kern_ms / len(infos), 3),
                         "heldout_ms_per_step": round(sum(i["heldout_ms"] for i in infos) / len(infos), 3),
                         "graph_replays": infos[-1]["graph_replays"],
-                        "kernel": "k_pass + k_trans <cox,csc,f32,batched>, grid (ctas_per_fit, 200)"},
+                        "kernel": "k_pass + k_btrans <cox,csc,f32,batched>, grid (ctas_per_fit, 200)"},
            "clocks": clk, "gpu_launches": int(sum(i["kernel_launches"] for i in infos)),
            "cv": {"best_lambda": infos[-1]["best_lambda"], "sweeps_max": int(sweeps.max()),
                   "sweeps_mean": float(sweeps.mean()), "fits_converged": infos[-1]["fits_converged"],

@@ -114,7 +114,9 @@ typedef struct surv_opts {
   double wait_limit_s;           /* bound on every device-side wait of the grid-wide
                                     exchange; <= 0 selects 2 seconds                */
   void *stream;                  /* cudaStream_t, or NULL for the default stream    */
-  surv_workspace *workspace;     /* reusable workspace, or NULL (allocate per call) */
+  surv_workspace *workspace;     /* reusable workspace, or NULL (the call takes its
+                                    buffers from a stream-ordered pool of the device
+                                    that keeps at most 256 MiB between calls)       */
 } surv_opts;
 
 /* Test only: one CTA of the CCD kernel never announces its first exchange,
@@ -320,8 +322,9 @@ typedef struct surv_nll_data {
   const void *X;                 /* [n][p] bfloat16, row-major                       */
 } surv_nll_data;
 
-/* nll[C] (device doubles) at B [p][C] (device floats).  Keeps eta and the
- * risk-set sums in the workspace `ws` (required) for cox_nll_backward.
+/* nll[C] (device doubles) at B [p][C] (device floats).  Keeps the split
+ * B, the risk-set sums and, for more than 256 covariates, eta in the workspace
+ * `ws` (required) for cox_nll_backward, which reads X again.
  * Errors: SURV_E_INVALID (null, sizes, host pointers), SURV_E_UNSORTED,
  * SURV_E_STATUS, SURV_E_NOMEM, SURV_E_CUDA; SURV_E_DEVICE_TIMEOUT when a
  * bounded wait inside the tensor-core kernels of an earlier forward or

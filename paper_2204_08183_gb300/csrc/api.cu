@@ -529,8 +529,9 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   // the FP32 mode): 4 columns per row pass, the fastest measured at N = 10^7
   // (8 columns: SURV_FLAG_SPEC_B8, for comparison).  Not when the tie groups
   // outnumber twice the warps: the transform of 4 columns at ~10^6 group
-  // ends costs more than the passes saved (measured 107 against 68 ms per
-  // fit at N = 2 x 10^6 with unique times).
+  // ends costs more than the passes saved (107 against 68 ms per fit
+  // at N = 2 x 10^6 with unique times when both walked their ends one after
+  // another; one coordinate per pass takes 29 ms now).
   int spec_b = 0;
   if (!(o.flags & SURV_FLAG_ONE_COORDINATE) && graph && !sn && model == SURV_COX && layout == SURV_CSC &&
       prec == 0 && p >= 2 && (int64_t)K < 2 * (int64_t)nwarps) {
