@@ -89,7 +89,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
   int nevals = L->nevals, stop = L->stop;
   double f_prev = L->f_prev;
   long long passes = L->passes, eta_updates = L->eta_updates;
-  bool dirty = passes == 0;   // the first pass of a fit
+  // The first pass of a launch forms every component: the warp totals of an
+  // unchanged e are kept in shared memory, which a launch finds undefined.
+  bool fresh = true;
   if (stop) return;   // the same in every CTA
   // the group end that thread tid takes first
   int d1 = 0, wl1 = 0;
@@ -113,8 +115,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
   __syncthreads();
   cluster_arrive();   // every CTA of the cluster has started: its shared memory may be written
   cluster_wait();
-  if (dirty && rows) {
-    // eta = X beta and e on the warp's own rows, a column at a time (a launch
+  if (passes == 0 && rows) {
+    // a fit's first launch: eta = X beta and e on the warp's own rows, a column at a time (a launch
     // per nonzero coefficient outside cost more than the evaluation it prepared)
     using E = typename std::conditional<sizeof(T) == 4, float2, double>::type;
     for (int64_t r = row_lo + lane; r < row_hi; r += 32) {
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
   for (int sw = 0; sw < sweeps && !stop;) {
     const int q = j == 0 ? p - 1 : j - 1;
     const bool eval = j == 0 || single;
-    const bool dense = LAYOUT == 1 || applied != 0.0 || dirty;
+    const bool dense = LAYOUT == 1 || applied != 0.0 || fresh;
     // ------------------------------------------------ steps 1-2, own rows
     if (rows) {
       if (applied != 0.0 && !kFuse) warp_update<LAYOUT, T>(P, q, gw, row_lo, row_hi, applied, delta);
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
     applied = s_applied;
     delta = {s_delta[0], s_delta[1]};
     stop = s_stop;
-    dirty = false;
+    fresh = false;
     if (!stop && jn == 0) ++sw;
     if (!stop) j = jn;
   }
