@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
     A fg1, fg2;
     acc_zero(fg1);
     acc_zero(fg2);
-    double pl = 0.0;
+    double pg1 = 0.0, pg2 = 0.0, pl = 0.0;
     for (int k = kc_lo + tid; k < kc_hi; k += kClThreads) {
       int d = d1, wl = wl1;
       double g = g1;
@@ -204,6 +204,23 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
       A Pm[M];
 #pragma unroll
       for (int m = 0; m < M; ++m) Pm[m] = acc_add(s_base[wl][m], rec[(size_t)k * M + m]);
+      if (sizeof(T) == 4 && single) {
+        // A single evaluation takes its ends in FP64, as the persistent kernel
+        // does with an end a thread: H - G^2 cancels where a covariate varies
+        // little against its mean, and float-float has 9 bits fewer for it.
+        double den = acc_to_d(Pm[0]), num1 = acc_to_d(Pm[1]), num2 = acc_to_d(Pm[2]);
+        if (MODEL == 1) {
+          den += g * (acc_to_d(s_tot[0]) - acc_to_d(Pm[3 % M]));
+          num1 += g * (acc_to_d(s_tot[1]) - acc_to_d(Pm[4 % M]));
+          num2 += g * (acc_to_d(s_tot[2]) - acc_to_d(Pm[5 % M]));
+        }
+        const double inv = 1.0 / den;
+        const double Gr = num1 * inv, H = num2 * inv;
+        pg1 += d * Gr;
+        pg2 += d * (H - Gr * Gr);
+        pl += d * log(den);
+        continue;
+      }
       A den = Pm[0], num1 = Pm[1], num2 = Pm[2];
       if (MODEL == 1) {
         const A gg = acc_base<A>(g, ff{gf.x, gf.y});
@@ -217,6 +234,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
       fg1 = acc_add(fg1, acc_scale(Gr, d));
       fg2 = acc_add(fg2, acc_scale(acc_add(H, acc_neg(acc_mul(Gr, Gr))), d));
       if (eval) pl += (double)d * log(acc_to_d(den));
+    }
+    if (sizeof(T) == 4 && single) {
+      fg1 = acc_from_d(pg1, (A*)nullptr);
+      fg2 = acc_from_d(pg2, (A*)nullptr);
     }
     const int nred = min((kc_hi - kc_lo + 31) >> 5, kClWarps);   // warps that had ends
     if (w < nred) {
