@@ -205,8 +205,8 @@ int device_view(surv_workspace* ws, int id, const void* src, size_t bytes, cudaS
   return SURV_OK;
 }
 
-// Pageable host memory: the runtime's copies from and to it are complete when
-// they return, so it needs none of them.
+// Pageable host memory, which the host reads and writes itself once the stream's
+// earlier work is done.
 bool is_pageable(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -216,10 +216,13 @@ bool is_pageable(const void* p) {
   return a.type == cudaMemoryTypeUnregistered;
 }
 
-// Copy a caller array (host or device) into host memory.
+// Copy a caller array (host or device) into host memory, in the order of the
+// call's stream: earlier work on it may write the array (a host function, or a
+// kernel where the device reaches pageable memory).
 int to_host(const void* src, size_t bytes, void* dst, cudaStream_t s) {
   if (bytes == 0) return SURV_OK;
   if (is_pageable(src)) {
+    CUDA_TRY(cudaStreamSynchronize(s));
     std::memcpy(dst, src, bytes);
     return SURV_OK;
   }
