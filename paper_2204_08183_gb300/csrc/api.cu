@@ -67,8 +67,9 @@ namespace {
 // call (ordering, tie groups, lambda_max, fits without a workspace).  Allocating
 // and freeing their buffers with cudaMalloc / cudaFree was most of such a call:
 // ordering 10^7 times spent 0.2 ms on the GPU of 0.42 ms.  The pool may be used
-// by any thread and stream; at most kPoolKeep bytes stay in it while it is idle,
-// and an allocation of this library that fails returns them first.
+// by any thread and stream; a call whose buffers took it above kPoolKeep bytes
+// gives the rest back before it returns (pool_give_back), and an allocation of
+// this library that fails returns all that is idle first.
 constexpr uint64_t kPoolKeep = 256ull << 20;
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
@@ -97,6 +98,17 @@ cudaMemPool_t scratch_pool(int dev) {
     }
   }
   return g_pool[dev];
+}
+
+// After the frees of a call: what the pool holds above kPoolKeep goes back to
+// the device.  The pool's own threshold takes effect only when somebody
+// synchronises again: 60 million times to order left 672 MiB reserved.
+void pool_give_back(surv_workspace* ws) {
+  uint64_t held = 0;
+  if (cudaMemPoolGetAttribute(ws->pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess && held > kPoolKeep &&
+      cudaStreamSynchronize(ws->pool_stream) == cudaSuccess)
+    cudaMemPoolTrimTo(ws->pool, kPoolKeep);
+  cudaGetLastError();
 }
 
 cudaError_t buf_free(surv_workspace* ws, void* p) {
@@ -167,6 +179,7 @@ void free_all(surv_workspace* ws) {
     b.p = nullptr;
     b.cap = 0;
   }
+  if (ws->pool) pool_give_back(ws);
 }
 
 // Memory the kernels may read in place: device memory of the current device
