@@ -359,10 +359,25 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
   }
 }
 
+// Form of the row pass: the many-ends form where warps hold two group ends or
+// more on average, and where fewer crowd into the warps of the latest times,
+// whose way through them one after another is then the pass: always in FP64,
+// and in FP32 from 96 ends if a warp has a whole tile of rows (with fewer rows a
+// lane's FP32 sums would be longer than the 4 rows of the other form).  us a
+// coordinate, ends one after another and the many-ends form: FP64 dense
+// Cox 22.9 and 20.3 for 60 ends of 16,384 rows, 55.9 and 21.1 for 359
+// (Fine-Gray 97.5 and 32.2); FP32 dense Fine-Gray 17.9 and 18.4 for 60 ends of
+// 70,000 rows, 21.2 and 20.4 for 100, 40.2 and 22.6 for 365; sparse Cox 12.9
+// and 13.7 for 60 ends of 300,000 rows, 15.0 and 14.7 for 100, 26.2 and 15.9
+// for 365.
+bool many_ends(int prec, int64_t K, int64_t nwarps, int64_t wpw) {
+  return prec == 1 || K >= 2 * nwarps || (K >= 96 && wpw >= 8);
+}
+
 template <int MODEL, int LAYOUT, typename T>
 cudaError_t cluster_size_of(int* G) {
   static_assert(kClWarps <= 32 && kClMax <= 32, "one lane per warp and per CTA");
-  auto k = k_cluster<MODEL, LAYOUT, T, false>;
+  auto k = k_cluster<MODEL, LAYOUT, T, true>;
   *G = 0;
   cudaError_t st = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (st != cudaSuccess) return st;
@@ -388,8 +403,9 @@ cudaError_t cluster_size_of(int* G) {
 
 template <int MODEL, int LAYOUT, typename T>
 cudaError_t launch_cluster(const CcdParams& P, int sweeps, cudaStream_t s) {
-  const bool multi = (int64_t)P.K >= 2 * (int64_t)P.nwarps;
-  auto k = multi ? k_cluster<MODEL, LAYOUT, T, true> : k_cluster<MODEL, LAYOUT, T, false>;
+  auto k = k_cluster<MODEL, LAYOUT, T, true>;
+  if constexpr (sizeof(T) == 4)
+    if (!many_ends(0, P.K, P.nwarps, P.wpw)) k = k_cluster<MODEL, LAYOUT, T, false>;
   cudaError_t st = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (st != cudaSuccess) return st;
   cudaLaunchAttribute at[1];
