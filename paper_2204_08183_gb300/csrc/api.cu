@@ -520,7 +520,18 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
                                &cols_nb)))
     return rc;
   if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
-  if (cluster && K > survgpu::kClusterMaxEnds) {   // too many group ends for a few SMs: the warps' rows change
+  // Default fits of sparse Cox data in the FP32 mode: batches (see below) where
+  // the group ends do not outnumber twice the warps of a full grid.
+  const bool sparse_cox = model == SURV_COX && layout == SURV_CSC && prec == 0 && p >= 2;
+  auto few_ends = [&](int64_t warps) { return (int64_t)K < 2 * warps; };
+  bool stay = cluster && K <= survgpu::kClusterMaxEnds;
+  if (stay && single_j < 0) {
+    int g = 0, w = 0;
+    CUDA_TRY(survgpu::graph_grid_size(model, layout, prec, &g, &w));
+    stay = survgpu::cluster_is_faster(model, layout, prec, n, K, (double)stg.nnz / (double)p, stg.vals != nullptr,
+                                      sparse_cox && few_ends((int64_t)g * w));
+  }
+  if (cluster && !stay) {   // too much for a few SMs: the warps' rows change
     if ((rc = partition(false))) return rc;
     if (layout == SURV_CSC) {
       if ((rc = ensure(ws, W::WOFF, 4 * (size_t)p * (nwarps + 1), &woff))) return rc;
@@ -549,8 +560,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   // at N = 2 x 10^6 with unique times when both walked their ends one after
   // another; one coordinate per pass takes 29 ms now).
   int spec_b = 0;
-  if (!(o.flags & SURV_FLAG_ONE_COORDINATE) && graph && !sn && model == SURV_COX && layout == SURV_CSC &&
-      prec == 0 && p >= 2 && (int64_t)K < 2 * (int64_t)nwarps) {
+  if (!(o.flags & SURV_FLAG_ONE_COORDINATE) && graph && !sn && sparse_cox && few_ends(nwarps)) {
     spec_b = (o.flags & SURV_FLAG_SPEC_B8) ? 8 : 4;
   }
   const int R = spec_b ? 1 + 2 * spec_b : M;  // record / aggregate components

@@ -23,6 +23,7 @@
 // sweeps; the state goes back to the control line, and the host launches
 // again until the fit reports its stop.
 #include <algorithm>
+#include <cmath>
 
 #include "graph_common.cuh"
 
@@ -434,19 +435,45 @@ cudaError_t launch_cluster(const CcdParams& P, int sweeps, cudaStream_t s) {
     return cudaErrorInvalidValue;                                                          \
   } while (0)
 
-// Largest cohorts for which a fit in one cluster was the faster (whole calls,
-// ms, cluster and kernel pair).  FP64 is bound by the FP64 pipes of the 16
-// SMs beyond two words a warp: 0.83 and 1.37 at 10,000 x 10 dense, 2.06 and
-// 1.37 at 20,000.  FP32: sparse Cox (against batches) 4.65 and 5.89 at 200,000
-// x 100, 5.79 and 5.16 at 400,000; dense Cox 1.73 and 1.98 at 100,000 x 24,
-// 2.27 and 2.0 at 200,000; sparse Fine-Gray 3.92 and 4.27 at 200,003 x 40, 5.35
-// and 4.3 at 400,000; dense Fine-Gray 4.69 and 4.85 at 100,000 x 50, 6.74 and
-// 5.0 at 200,000.  By group ends (kClusterMaxEnds): sparse Cox with hardly any
-// ties 4.93 and 5.64 at 20,000 x 80, 7.3 and 6.5 at 50,000.
-int64_t cluster_rows(int model, int layout, int prec) {
-  if (prec == 1) return 2 * 32 * kClMax * kClWarps;   // 16,384
-  if (layout == 0) return model == 0 ? 300000 : 262144;
-  return model == 0 ? 131072 : 100000;
+// us a coordinate of a fit in one cluster,
+//   fixed + row n/10^5 + many n/10^5 (the many-ends form) + end E/1000
+//         + serial (K - 50)/100 (the other form) + (entry + entry_end min(1, K/300)) nnz/10^4,
+// nnz the stored entries of a column and E the group ends of its busiest CTA
+// (the first of 16: 0.4 K of exponential times, at most its rows), and of the
+// kernel pair on the whole chip, other + other_log log2 K, where n hardly counts.
+// Least squares over 1,500 fits of 300 to 300,000 rows, 40 to 33,000 ends and
+// 0.5 to 45 % density (6 to 9 % rms).  The choice between them costs 0.4 % on
+// average against the faster one, and at most a sixth more than the schedule
+// that stood before the cluster.  Limits on n and on K alone lost where both
+// were near them or columns dense (ms a fit, cluster and pair: 7.6 and 1.6 for
+// sparse Cox at 300,000 x 60 with half of the entries stored, 9.8 and 8.7 at 5 %
+// with 27,000 ends; 7.5 and 4.3 for sparse Fine-Gray at 262,000 x 40).
+struct FitCost {
+  double fixed, row, many, end, serial, entry, entry_end, other, other_log;
+};
+constexpr FitCost kFitCost[2][2][2] = {   // model, layout, precision
+    {{{9.4, 1.0, 0.6, 2.9, 4.0, 0.3, 1.6, 5.0, 1.1}, {12.2, 20.0, 0.0, 6.1, 0.0, 3.7, 1.5, 21.0, 0.65}},
+     {{9.4, 2.3, 2.7, 3.4, 4.0, 0.0, 0.0, 11.4, 0.62}, {10.5, 65.5, 0.0, 5.7, 0.0, 0.0, 0.0, 22.0, 0.65}}},
+    {{{14.0, 1.0, 1.6, 4.9, 7.0, 0.5, 2.6, 15.1, 0.92}, {16.6, 42.5, 0.0, 9.1, 0.0, 4.6, 3.4, 32.0, 0.95}},
+     {{13.5, 2.6, 5.8, 5.7, 7.0, 0.0, 0.0, 13.0, 0.95}, {14.9, 107.5, 0.0, 8.8, 0.0, 0.0, 0.0, 32.5, 0.95}}}};
+
+// The same of one row pass of a batch of four coordinates (sparse Cox, FP32):
+// its warps walk their ends one after another, the more of them the larger K
+// against the spread of the rows (10 % rms, real values 15 %).
+double batch_pass_us(double n, double K, double nnz, bool values) {
+  const double v = std::log2(1.0 + K / std::sqrt(n)) * (0.7 + std::sqrt(nnz / n));
+  return values ? 31.0 + 13.0 * v : 16.5 + 6.0 * v;
+}
+
+// Rows up to which the figures above hold.
+int64_t cluster_rows(int prec) { return prec == 1 ? 40000 : 300000; }
+
+// Row words a warp and row warps of a cluster of G CTAs: no more warps than the
+// words need, so that the rows are spread evenly over the CTAs.
+void cluster_partition(int64_t n, int G, int64_t* wpw, int* wpc) {
+  const int64_t nwords = (n + 31) / 32, most = (int64_t)G * kClWarps;
+  *wpw = (nwords + most - 1) / most;
+  *wpc = (int)(((nwords + *wpw - 1) / *wpw + G - 1) / G);
 }
 
 }  // namespace
@@ -454,15 +481,24 @@ int64_t cluster_rows(int model, int layout, int prec) {
 cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc) {
   *G = 0;
   *wpc = 0;
-  if (n > cluster_rows(model, layout, prec) || p > kClMaxP) return cudaSuccess;
+  if (n > cluster_rows(prec) || p > kClMaxP) return cudaSuccess;
   cudaError_t st = [&] { SURV_DISPATCH_CL(cluster_size_of, G); }();
   if (st != cudaSuccess || *G == 0) return st;
-  // no more row warps than the words need, so that the rows are spread evenly
-  // over the CTAs
-  const int64_t nwords = (n + 31) / 32, most = (int64_t)*G * kClWarps;
-  const int64_t wpw = (nwords + most - 1) / most, used = (nwords + wpw - 1) / wpw;
-  *wpc = (int)((used + *G - 1) / *G);
+  int64_t wpw = 0;
+  cluster_partition(n, *G, &wpw, wpc);
   return cudaSuccess;
+}
+
+bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches) {
+  const FitCost& c = kFitCost[model][layout][prec];
+  int64_t wpw = 0;
+  int wpc = 0;
+  cluster_partition(n, kClMax, &wpw, &wpc);
+  const double rows = (double)n * 1e-5;
+  double us = c.fixed + c.row * rows + (c.entry + c.entry_end * std::min(1.0, K / 300.0)) * nnz * 1e-4;
+  if (many_ends(prec, K, (int64_t)kClMax * wpc, wpw)) us += c.many * rows + c.end * 1e-3 * std::min(0.4 * K, n / 16.0);
+  else us += c.serial * 0.01 * std::max(0, K - 50);
+  return us < (batches ? batch_pass_us((double)n, K, nnz, values) : c.other + c.other_log * std::log2(std::max(2, K)));
 }
 
 cudaError_t run_cluster(int model, int layout, int prec, const CcdParams& P, int sweeps, cudaStream_t s) {

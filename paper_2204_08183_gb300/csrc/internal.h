@@ -204,6 +204,10 @@ cudaError_t replay_until_stop(const CcdParams& P, cudaStream_t s, GraphCache* gc
 // which is for cohorts of at most kClusterMaxEnds tie groups (known later).
 constexpr int32_t kClusterMaxEnds = 32768;
 cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc);
+// Whether a fit of such a cohort (K tie groups; CSC: nnz stored entries a
+// column on average, with values or ones) is faster there than on the kernel
+// pair or, with `batches`, than in batches of four coordinates.
+bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches);
 // Up to `sweeps` sweeps of a fit (or the evaluation of P.single_j) in one
 // launch; *P.gctl zeroed before the first, which also sets eta = X beta and e.
 // P.gctl->done tells the stop.
