@@ -53,7 +53,11 @@ struct ClCfg {
   static constexpr int SR = 4;
 };
 
-template <int MODEL, int LAYOUT, typename T, bool MULTI>
+// ONE: a single evaluation, which takes its group ends in FP64 (FP32 mode), as
+// the persistent kernel does: H - G^2 cancels where a covariate varies little
+// against its mean, and float-float has 9 bits fewer for it.  (A kernel of its
+// own: as a branch it cost fits of dense Fine-Gray 5 %.)
+template <int MODEL, int LAYOUT, typename T, bool MULTI, bool ONE>
 __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant__ CcdParams P, int sweeps) {
   using A = typename AccOf<T>::type;
   using C = Cfg<MODEL, LAYOUT, T>;
@@ -205,10 +209,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
       A Pm[M];
 #pragma unroll
       for (int m = 0; m < M; ++m) Pm[m] = acc_add(s_base[wl][m], rec[(size_t)k * M + m]);
-      if (sizeof(T) == 4 && single) {
-        // A single evaluation takes its ends in FP64, as the persistent kernel
-        // does with an end a thread: H - G^2 cancels where a covariate varies
-        // little against its mean, and float-float has 9 bits fewer for it.
+      if constexpr (ONE) {
         double den = acc_to_d(Pm[0]), num1 = acc_to_d(Pm[1]), num2 = acc_to_d(Pm[2]);
         if (MODEL == 1) {
           den += g * (acc_to_d(s_tot[0]) - acc_to_d(Pm[3 % M]));
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(const __grid_constant
       fg2 = acc_add(fg2, acc_scale(acc_add(H, acc_neg(acc_mul(Gr, Gr))), d));
       if (eval) pl += (double)d * log(acc_to_d(den));
     }
-    if (sizeof(T) == 4 && single) {
+    if constexpr (ONE) {
       fg1 = acc_from_d(pg1, (A*)nullptr);
       fg2 = acc_from_d(pg2, (A*)nullptr);
     }
@@ -378,7 +379,7 @@ bool many_ends(int prec, int64_t K, int64_t nwarps, int64_t wpw) {
 template <int MODEL, int LAYOUT, typename T>
 cudaError_t cluster_size_of(int* G) {
   static_assert(kClWarps <= 32 && kClMax <= 32, "one lane per warp and per CTA");
-  auto k = k_cluster<MODEL, LAYOUT, T, true>;
+  auto k = k_cluster<MODEL, LAYOUT, T, true, false>;
   *G = 0;
   cudaError_t st = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (st != cudaSuccess) return st;
@@ -404,9 +405,12 @@ cudaError_t cluster_size_of(int* G) {
 
 template <int MODEL, int LAYOUT, typename T>
 cudaError_t launch_cluster(const CcdParams& P, int sweeps, cudaStream_t s) {
-  auto k = k_cluster<MODEL, LAYOUT, T, true>;
-  if constexpr (sizeof(T) == 4)
-    if (!many_ends(0, P.K, P.nwarps, P.wpw)) k = k_cluster<MODEL, LAYOUT, T, false>;
+  auto k = k_cluster<MODEL, LAYOUT, T, true, false>;
+  if constexpr (sizeof(T) == 4) {
+    const bool many = many_ends(0, P.K, P.nwarps, P.wpw);
+    if (P.single_j >= 0) k = many ? k_cluster<MODEL, LAYOUT, T, true, true> : k_cluster<MODEL, LAYOUT, T, false, true>;
+    else if (!many) k = k_cluster<MODEL, LAYOUT, T, false, false>;
+  }
   cudaError_t st = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (st != cudaSuccess) return st;
   cudaLaunchAttribute at[1];
