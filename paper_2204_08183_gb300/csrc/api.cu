@@ -524,12 +524,63 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   // the group ends do not outnumber twice the warps of a full grid.
   const bool sparse_cox = model == SURV_COX && layout == SURV_CSC && prec == 0 && p >= 2;
   auto few_ends = [&](int64_t warps) { return (int64_t)K < 2 * warps; };
+  void *gend, *dk, *ck;
+  if ((rc = ensure(ws, W::GEND, 4 * (size_t)K, &gend))) return rc;
+  if ((rc = ensure(ws, W::DK, 4 * (size_t)K, &dk))) return rc;
+  if ((rc = ensure(ws, W::CK, 4 * (size_t)K, &ck))) return rc;
+  survgpu::RowMasks masks;
+  if ((rc = row_masks(ws, n, &masks))) return rc;
+  bool grouped = false;   // the group tables are written
+  auto write_groups = [&]() -> int {
+    if ((rc = ensure(ws, W::WK0, 4 * (size_t)(nwarps + 1), &wk0))) return rc;
+    if (grouped)
+      CUDA_TRY(survgpu::prep_warp_groups(static_cast<int32_t*>(gend), K, n, nwarps, rows_per_warp,
+                                         static_cast<int32_t*>(wk0), s));
+    else
+      CUDA_TRY(survgpu::prep_group_write(time_p, status_p, n, cnt, K, static_cast<int32_t*>(gend),
+                                         static_cast<int32_t*>(dk), static_cast<int32_t*>(ck), nwarps, rows_per_warp,
+                                         static_cast<int32_t*>(wk0), s, &masks));
+    ++launches;
+    grouped = true;
+    return SURV_OK;
+  };
   bool stay = cluster && K <= survgpu::kClusterMaxEnds;
   if (stay && single_j < 0) {
     int g = 0, w = 0;
     CUDA_TRY(survgpu::graph_grid_size(model, layout, prec, &g, &w));
-    stay = survgpu::cluster_is_faster(model, layout, prec, n, K, (double)stg.nnz / (double)p, stg.vals != nullptr,
-                                      sparse_cox && few_ends((int64_t)g * w));
+    const bool batches = sparse_cox && few_ends((int64_t)g * w);
+    auto faster = [&](double moving) {
+      return survgpu::cluster_is_faster(model, layout, prec, n, K, (double)stg.nnz / (double)p, stg.vals != nullptr,
+                                        batches, moving);
+    };
+    stay = faster(1.0);
+    // An L1 fit may move few of its coordinates, and batches then take several a
+    // row pass.  Which way it goes shows at the start: the nonzeros of a warm
+    // beta, or at beta = 0 the gradients beyond their strengths (five small
+    // kernels and one wait, 40 us; not for 8 coordinates or fewer, where a fit is
+    // not longer than that).  Sparse Cox at 200,000 x 60, of which 20 move: 1.41
+    // ms in batches, 2.33 on the cluster.
+    if (batches && o.penalty == SURV_PEN_L1 && p > 8 && faster(0.0) != stay) {
+      int64_t moving = 0;
+      for (double b : beta_h) moving += b != 0.0;
+      if (moving == 0) {
+        void *lam, *r, *grad;
+        if ((rc = ensure(ws, W::LM_LAM, 8 * (size_t)K, &lam))) return rc;
+        if ((rc = ensure(ws, W::LM_R, 8 * (size_t)n, &r))) return rc;
+        if ((rc = ensure(ws, W::LM_G, 8 * (size_t)(p + 1), &grad))) return rc;
+        if ((rc = write_groups())) return rc;
+        CUDA_TRY(survgpu::null_gradient(layout, prec, stg.colptr, stg.rowidx, stg.vals, stg.ld, n, p, status_p,
+                                        static_cast<int32_t*>(gend), static_cast<int32_t*>(dk), K,
+                                        static_cast<double*>(lam), static_cast<double*>(r),
+                                        static_cast<double*>(grad), s));
+        launches += 4;
+        std::vector<double> grad_h(p);
+        CUDA_TRY(cudaMemcpyAsync(grad_h.data(), grad, 8 * (size_t)p, cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(cudaStreamSynchronize(s));
+        for (int64_t j = 0; j < p; ++j) moving += std::fabs(grad_h[j]) > pen_h[j];
+      }
+      stay = faster((double)moving / (double)p);
+    }
   }
   if (cluster && !stay) {   // too much for a few SMs: the warps' rows change
     if ((rc = partition(false))) return rc;
@@ -540,15 +591,14 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
       ++launches;
     }
   }
+  if (!grouped || !cluster)
+    if ((rc = write_groups())) return rc;
   const void* vals_d = stg.vals;  // null for indicator CSC data (all values 1)
   DevCtrl hc;
 
   // ---------------------------------------------------------- tables
-  void *gend, *dk, *ck, *Gk, *rec, *e, *eta, *w2 = nullptr, *dTx, *beta, *width, *pen, *slots;
+  void *Gk, *rec, *e, *eta, *w2 = nullptr, *dTx, *beta, *width, *pen, *slots;
   constexpr size_t accsz = 8;  // an accumulator: ff (2 floats) or double
-  if ((rc = ensure(ws, W::GEND, 4 * (size_t)K, &gend))) return rc;
-  if ((rc = ensure(ws, W::DK, 4 * (size_t)K, &dk))) return rc;
-  if ((rc = ensure(ws, W::CK, 4 * (size_t)K, &ck))) return rc;
   if ((rc = ensure(ws, W::GK, 8 * (size_t)K, &Gk))) return rc;
   void* Gkff = nullptr;
   if ((rc = ensure(ws, W::GKFF, 8 * (size_t)K, &Gkff))) return rc;
@@ -568,7 +618,6 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   if ((rc = ensure(ws, W::E, tsz * (size_t)n, &e))) return rc;
   if ((rc = ensure(ws, W::ETA, 8 * (size_t)n, &eta))) return rc;
   if (model == SURV_FG && (rc = ensure(ws, W::W2, tsz * (size_t)n, &w2))) return rc;
-  if ((rc = ensure(ws, W::WK0, 4 * (size_t)(nwarps + 1), &wk0))) return rc;
   if ((rc = ensure(ws, W::DTX, 8 * (size_t)p, &dTx))) return rc;
   if ((rc = ensure(ws, W::BETA, 8 * (size_t)p, &beta))) return rc;
   if ((rc = ensure(ws, W::WIDTH, 8 * (size_t)p, &width))) return rc;
@@ -609,12 +658,6 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     S.multi = (int64_t)K >= 2 * (int64_t)nwarps ? 1 : 0;
   }
 
-  survgpu::RowMasks masks;
-  if ((rc = row_masks(ws, n, &masks))) return rc;
-  CUDA_TRY(survgpu::prep_group_write(time_p, status_p, n, cnt, K, static_cast<int32_t*>(gend),
-                                     static_cast<int32_t*>(dk), static_cast<int32_t*>(ck), nwarps, rows_per_warp,
-                                     static_cast<int32_t*>(wk0), s, &masks));
-  ++launches;
   if (model == SURV_FG) {
     CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), s));
     // the records are not in use yet: scratch for 1 / G

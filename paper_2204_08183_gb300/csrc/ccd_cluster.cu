@@ -461,12 +461,15 @@ constexpr FitCost kFitCost[2][2][2] = {   // model, layout, precision
     {{{14.0, 1.0, 1.6, 4.9, 7.0, 0.5, 2.6, 15.1, 0.92}, {16.6, 42.5, 0.0, 9.1, 0.0, 4.6, 3.4, 32.0, 0.95}},
      {{13.5, 2.6, 5.8, 5.7, 7.0, 0.0, 0.0, 13.0, 0.95}, {14.9, 107.5, 0.0, 8.8, 0.0, 0.0, 0.0, 32.5, 0.95}}}};
 
-// The same of one row pass of a batch of four coordinates (sparse Cox, FP32):
-// its warps walk their ends one after another, the more of them the larger K
-// against the spread of the rows (10 % rms, real values 15 %).
-double batch_pass_us(double n, double K, double nnz, bool values) {
-  const double v = std::log2(1.0 + K / std::sqrt(n)) * (0.7 + std::sqrt(nnz / n));
-  return values ? 31.0 + 13.0 * v : 16.5 + 6.0 * v;
+// The same in batches of four coordinates (sparse Cox, FP32).  A row pass (10 %
+// rms, real values 15 %): its warps walk their ends one after another, the more
+// of them the larger K against the spread of the rows, and stream e only after
+// a step.  It serves the coordinates up to the first that steps, so with a share
+// `moving` of them 1 / moving (1 - (1 - moving)^4), four where none does.
+double batch_us(double n, double K, double nnz, bool values, double moving) {
+  const double v = std::log2(1.0 + K / std::sqrt(n)) * (0.7 + std::sqrt(nnz / n)) * (0.5 + 0.5 * std::min(1.0, 3.0 * moving));
+  const double pass = values ? 31.0 + 13.0 * v : 16.5 + 6.0 * v;
+  return pass * (moving > 0.0 ? moving / (1.0 - std::pow(1.0 - moving, 4)) : 0.25);
 }
 
 // Rows up to which the figures above hold.
@@ -493,7 +496,8 @@ cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_
   return cudaSuccess;
 }
 
-bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches) {
+bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches,
+                       double moving) {
   const FitCost& c = kFitCost[model][layout][prec];
   int64_t wpw = 0;
   int wpc = 0;
@@ -502,7 +506,8 @@ bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, do
   double us = c.fixed + c.row * rows + (c.entry + c.entry_end * std::min(1.0, K / 300.0)) * nnz * 1e-4;
   if (many_ends(prec, K, (int64_t)kClMax * wpc, wpw)) us += c.many * rows + c.end * 1e-3 * std::min(0.4 * K, n / 16.0);
   else us += c.serial * 0.01 * std::max(0, K - 50);
-  return us < (batches ? batch_pass_us((double)n, K, nnz, values) : c.other + c.other_log * std::log2(std::max(2, K)));
+  if (!batches) return us < c.other + c.other_log * std::log2(std::max(2, K));
+  return us - 1.8 * (1.0 - moving) < batch_us((double)n, K, nnz, values, moving);   // (no update, no walk of e)
 }
 
 cudaError_t run_cluster(int model, int layout, int prec, const CcdParams& P, int sweeps, cudaStream_t s) {

@@ -407,10 +407,9 @@ cudaError_t cv_select(const double* heldout, int nlambda, int nfolds, double* cv
   return cudaGetLastError();
 }
 
-cudaError_t lambda_max_device(int layout, int prec, const int64_t* col_ptr, const int32_t* row_idx,
-                              const void* values, int64_t ld, int64_t n, int64_t p, const int8_t* status,
-                              const int32_t* gend, const int32_t* dk, int32_t K, const double* pf, double* lam,
-                              double* r, double* g, double* out, cudaStream_t s) {
+cudaError_t null_gradient(int layout, int prec, const int64_t* col_ptr, const int32_t* row_idx, const void* values,
+                          int64_t ld, int64_t n, int64_t p, const int8_t* status, const int32_t* gend,
+                          const int32_t* dk, int32_t K, double* lam, double* r, double* g, cudaStream_t s) {
   k_lmax_terms<<<grid_for(K, kCvThreads, 1024), kCvThreads, 0, s>>>(gend, dk, K, lam);
   k_lmax_lambda<<<1, kScanThreads, 0, s>>>(K, lam);
   k_lmax_resid<<<grid_for(n, kCvThreads, 8192), kCvThreads, 0, s>>>(gend, K, status, lam, n, r);
@@ -421,6 +420,16 @@ cudaError_t lambda_max_device(int layout, int prec, const int64_t* col_ptr, cons
     if (prec == 0) k_lmax_grad_dense<float><<<(unsigned)p, 1024, 0, s>>>((const float*)values, ld, n, r, g);
     else k_lmax_grad_dense<double><<<(unsigned)p, 1024, 0, s>>>((const double*)values, ld, n, r, g);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t lambda_max_device(int layout, int prec, const int64_t* col_ptr, const int32_t* row_idx,
+                              const void* values, int64_t ld, int64_t n, int64_t p, const int8_t* status,
+                              const int32_t* gend, const int32_t* dk, int32_t K, const double* pf, double* lam,
+                              double* r, double* g, double* out, cudaStream_t s) {
+  const cudaError_t st =
+      null_gradient(layout, prec, col_ptr, row_idx, values, ld, n, p, status, gend, dk, K, lam, r, g, s);
+  if (st != cudaSuccess) return st;
   k_lmax_max<<<1, 1024, 0, s>>>(g, pf, p, out);
   return cudaGetLastError();
 }

@@ -206,8 +206,10 @@ constexpr int32_t kClusterMaxEnds = 32768;
 cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc);
 // Whether a fit of such a cohort (K tie groups; CSC: nnz stored entries a
 // column on average, with values or ones) is faster there than on the kernel
-// pair or, with `batches`, than in batches of four coordinates.
-bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches);
+// pair or, with `batches`, than in batches of four coordinates, of which a share
+// `moving` steps in a sweep.
+bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches,
+                       double moving);
 // Up to `sweeps` sweeps of a fit (or the evaluation of P.single_j) in one
 // launch; *P.gctl zeroed before the first, which also sets eta = X beta and e.
 // P.gctl->done tells the stop.
@@ -333,6 +335,10 @@ cudaError_t cv_heldout(int prec, int64_t n, int64_t fit_n, const int32_t* time, 
 cudaError_t cv_select(const double* heldout, int nlambda, int nfolds, double* cv_mean, int32_t* best,
                       cudaStream_t s);
 // *out (device) = max_j |l'_j(0)| / pf_j for Cox; lam [K], r [n], g [p] scratch
+// Gradient of the Cox log-likelihood at beta = 0, FP64 (lam [K], r [n]: scratch).
+cudaError_t null_gradient(int layout, int prec, const int64_t* col_ptr, const int32_t* row_idx, const void* values,
+                          int64_t ld, int64_t n, int64_t p, const int8_t* status, const int32_t* gend,
+                          const int32_t* dk, int32_t K, double* lam, double* r, double* g, cudaStream_t s);
 cudaError_t lambda_max_device(int layout, int prec, const int64_t* col_ptr, const int32_t* row_idx,
                               const void* values, int64_t ld, int64_t n, int64_t p, const int8_t* status,
                               const int32_t* gend, const int32_t* dk, int32_t K, const double* pf, double* lam,
