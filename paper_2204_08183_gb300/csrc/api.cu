@@ -39,7 +39,7 @@ struct DevCtrl {
   int32_t total_events;
   unsigned counters[2];
   unsigned ticket;       // blocks of k_group_count done
-  unsigned pad;
+  int32_t crowd;         // most group ends among 32 rows (where asked for)
   double out[survgpu::OUT_COUNT];
   unsigned long long timing[survgpu::PH_COUNT];
   survgpu::GraphCtl gctl;
@@ -365,7 +365,8 @@ int row_masks(surv_workspace* ws, int64_t n, survgpu::RowMasks* m) {
 // again.
 int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, Staged& st, DevCtrl* ctrl,
                        surv_workspace* ws, cudaStream_t s, void** cnt, int32_t* K, int32_t* events,
-                       int64_t* launches, survgpu::PrepColumns* cols = nullptr, int* cols_nb = nullptr) {
+                       int64_t* launches, survgpu::PrepColumns* cols = nullptr, int* cols_nb = nullptr,
+                       int32_t* crowd = nullptr) {
   CUDA_TRY(cudaMemsetAsync(ctrl, 0, sizeof(DevCtrl), s));
   int rc;
   if ((rc = ensure(ws, surv_workspace::BLOCKCNT, survgpu::prep_count_bytes(n), cnt))) return rc;
@@ -376,7 +377,7 @@ int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, St
     cols->event = event = static_cast<uint32_t*>(ev);
   }
   CUDA_TRY(survgpu::prep_group_count(st.time, st.status, n, model, *cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events,
-                                     &ctrl->ticket, s, event));
+                                     &ctrl->ticket, s, event, crowd ? &ctrl->crowd : nullptr));
   ++*launches;
   int64_t longest = n;
   if (layout == SURV_CSC) {
@@ -399,6 +400,7 @@ int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, St
   if ((rc = map_prep_error(hc.perr))) return rc;
   *K = hc.K;
   *events = hc.total_events;
+  if (crowd) *crowd = hc.crowd;
   if (layout == SURV_CSC && st.vals && !(hc.perr & survgpu::PREP_VALUES_NOT_ONE)) st.vals = nullptr;
   return SURV_OK;
 }
@@ -505,7 +507,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   const int32_t* time_p = stg.time;
   const int8_t* status_p = stg.status;
   void* cnt = nullptr;
-  int32_t K = 0, events = 0;
+  int32_t K = 0, events = 0, crowd = 0;
   survgpu::PrepColumns cols;
   int cols_nb = 0;
   void *woff = nullptr, *wk0 = nullptr;
@@ -517,7 +519,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     cols.woff = static_cast<int32_t*>(woff);
   }
   if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches, &cols,
-                               &cols_nb)))
+                               &cols_nb, cluster && single_j < 0 ? &crowd : nullptr)))
     return rc;
   if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   // Default fits of sparse Cox data in the FP32 mode: batches (see below) where
@@ -549,10 +551,9 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     int g = 0, w = 0;
     CUDA_TRY(survgpu::graph_grid_size(model, layout, prec, &g, &w));
     const bool batches = sparse_cox && few_ends((int64_t)g * w);
-    auto faster = [&](double moving) {
-      return survgpu::cluster_is_faster(model, layout, prec, n, K, (double)stg.nnz / (double)p, stg.vals != nullptr,
-                                        batches, moving);
-    };
+    const survgpu::FitShape shape = {n, K, crowd, (double)stg.nnz / (double)p, stg.vals != nullptr,
+                                     batches ? (int64_t)g * w : 0};
+    auto faster = [&](double moving) { return survgpu::cluster_is_faster(model, layout, prec, shape, moving); };
     stay = faster(1.0);
     // An L1 fit may move few of its coordinates, and batches then take several a
     // row pass.  Which way it goes shows at the start: the nonzeros of a warm

@@ -440,35 +440,41 @@ cudaError_t launch_cluster(const CcdParams& P, int sweeps, cudaStream_t s) {
   } while (0)
 
 // us a coordinate of a fit in one cluster,
-//   fixed + row n/10^5 + many n/10^5 (the many-ends form) + end E/1000
-//         + serial (K - 50)/100 (the other form) + (entry + entry_end min(1, K/300)) nnz/10^4,
-// nnz the stored entries of a column and E the group ends of its busiest CTA
-// (the first of 16: 0.4 K of exponential times, at most its rows), and of the
-// kernel pair on the whole chip, other + other_log log2 K, where n hardly counts.
-// Least squares over 1,500 fits of 300 to 300,000 rows, 40 to 33,000 ends and
-// 0.5 to 45 % density (6 to 9 % rms).  The choice between them costs 0.4 % on
-// average against the faster one, and at most a sixth more than the schedule
-// that stood before the cluster.  Limits on n and on K alone lost where both
-// were near them or columns dense (ms a fit, cluster and pair: 7.6 and 1.6 for
-// sparse Cox at 300,000 x 60 with half of the entries stored, 9.8 and 8.7 at 5 %
-// with 27,000 ends; 7.5 and 4.3 for sparse Fine-Gray at 262,000 x 40).
+//   fixed + row n/10^5 + many n/10^5 + end E/1000          (the many-ends form)
+//         + serial max(0, W - 5)/10                         (the other form)
+//         + (entry + entry_end f) nnz/10^4,                 (CSC)
+// E the group ends of its busiest CTA and W of its busiest warp, both bounded by
+// the rows, by K (0.4 and 0.12 of it for exponential times) and by `crowd`, the
+// most ends among 32 rows; f = min(1, K/300) min(1, (crowd + 1)/3) the share of
+// entry rounds with an end.  Of the kernel pair on the whole chip:
+// other + other_log log2 K, where n hardly counts.  Least squares over 4,600
+// fits of 300 to 300,000 rows with exponential, censored and uniform times, 40 to
+// 39,000 ends and 0.5 to 50 % density: 4 to 9 % rms.  The choice between the two
+// costs 0.3 to 1 % on average against the faster one, and at most 12 % more than
+// the schedule that stood before the cluster.  Limits on n and on K alone lost
+// where both were near them or columns dense (ms a fit, cluster and pair: 7.6
+// and 1.6 for sparse Cox at 300,000 x 60 with half of the entries stored, 9.8
+// and 8.7 at 5 % with 27,000 ends; 7.5 and 4.3 for sparse Fine-Gray at 262,000 x
+// 40 with half of the entries).
 struct FitCost {
   double fixed, row, many, end, serial, entry, entry_end, other, other_log;
 };
 constexpr FitCost kFitCost[2][2][2] = {   // model, layout, precision
-    {{{9.4, 1.0, 0.6, 2.9, 4.0, 0.3, 1.6, 5.0, 1.1}, {12.2, 20.0, 0.0, 6.1, 0.0, 3.7, 1.5, 21.0, 0.65}},
-     {{9.4, 2.3, 2.7, 3.4, 4.0, 0.0, 0.0, 11.4, 0.62}, {10.5, 65.5, 0.0, 5.7, 0.0, 0.0, 0.0, 22.0, 0.65}}},
-    {{{14.0, 1.0, 1.6, 4.9, 7.0, 0.5, 2.6, 15.1, 0.92}, {16.6, 42.5, 0.0, 9.1, 0.0, 4.6, 3.4, 32.0, 0.95}},
-     {{13.5, 2.6, 5.8, 5.7, 7.0, 0.0, 0.0, 13.0, 0.95}, {14.9, 107.5, 0.0, 8.8, 0.0, 0.0, 0.0, 32.5, 0.95}}}};
+    {{{9.6, 0.8, 0.4, 2.4, 5.0, 0.3, 1.75, 4.0, 1.16}, {12.3, 19.0, 0.0, 6.0, 0.0, 3.0, 2.0, 21.5, 0.65}},
+     {{9.7, 0.8, 3.6, 3.0, 5.0, 0.0, 0.0, 11.0, 0.64}, {10.7, 60.0, 0.0, 5.9, 0.0, 0.0, 0.0, 22.8, 0.62}}},
+    {{{14.0, 0.3, 1.8, 4.4, 8.2, 0.3, 2.8, 14.6, 0.94}, {16.8, 38.0, 0.0, 8.5, 0.0, 4.5, 5.0, 33.0, 0.95}},
+     {{13.7, 0.5, 6.8, 5.1, 9.0, 0.0, 0.0, 12.8, 0.95}, {15.1, 98.0, 0.0, 8.9, 0.0, 0.0, 0.0, 33.3, 0.9}}}};
 
-// The same in batches of four coordinates (sparse Cox, FP32).  A row pass (10 %
-// rms, real values 15 %): its warps walk their ends one after another, the more
-// of them the larger K against the spread of the rows, and stream e only after
-// a step.  It serves the coordinates up to the first that steps, so with a share
-// `moving` of them 1 / moving (1 - (1 - moving)^4), four where none does.
-double batch_us(double n, double K, double nnz, bool values, double moving) {
-  const double v = std::log2(1.0 + K / std::sqrt(n)) * (0.7 + std::sqrt(nnz / n)) * (0.5 + 0.5 * std::min(1.0, 3.0 * moving));
-  const double pass = values ? 31.0 + 13.0 * v : 16.5 + 6.0 * v;
+// The same in batches of four coordinates (sparse Cox, FP32).  A row pass (6 %
+// rms, real values 8 %): its busiest warp walks its ends one after another, and
+// streams e only after a step.  It serves the coordinates up to the first that
+// steps, so with a share `moving` of them 1 / moving (1 - (1 - moving)^4), four
+// where none does.
+double batch_us(const FitShape& f, double moving) {
+  const int64_t nwords = (f.n + 31) / 32, wpw = (nwords + f.batch_warps - 1) / f.batch_warps;
+  const double dens = std::min(0.5, std::sqrt(f.nnz / (double)f.n));
+  const double walk = 0.1 * (double)(f.crowd * wpw) * (0.5 + 0.5 * std::min(1.0, 3.0 * moving));
+  const double pass = f.values ? 29.0 + walk * (13.0 + 26.0 * dens) : 17.6 + walk * (5.3 + 14.5 * dens);
   return pass * (moving > 0.0 ? moving / (1.0 - std::pow(1.0 - moving, 4)) : 0.25);
 }
 
@@ -496,18 +502,20 @@ cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_
   return cudaSuccess;
 }
 
-bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches,
-                       double moving) {
+bool cluster_is_faster(int model, int layout, int prec, const FitShape& f, double moving) {
   const FitCost& c = kFitCost[model][layout][prec];
   int64_t wpw = 0;
   int wpc = 0;
-  cluster_partition(n, kClMax, &wpw, &wpc);
-  const double rows = (double)n * 1e-5;
-  double us = c.fixed + c.row * rows + (c.entry + c.entry_end * std::min(1.0, K / 300.0)) * nnz * 1e-4;
-  if (many_ends(prec, K, (int64_t)kClMax * wpc, wpw)) us += c.many * rows + c.end * 1e-3 * std::min(0.4 * K, n / 16.0);
-  else us += c.serial * 0.01 * std::max(0, K - 50);
-  if (!batches) return us < c.other + c.other_log * std::log2(std::max(2, K));
-  return us - 1.8 * (1.0 - moving) < batch_us((double)n, K, nnz, values, moving);   // (no update, no walk of e)
+  cluster_partition(f.n, kClMax, &wpw, &wpc);
+  const double rows = (double)f.n * 1e-5, K = f.K, crowd = f.crowd;
+  double us = c.fixed + c.row * rows +
+              (c.entry + c.entry_end * std::min(1.0, K / 300.0) * std::min(1.0, (crowd + 1.0) / 3.0)) * f.nnz * 1e-4;
+  if (many_ends(prec, f.K, (int64_t)kClMax * wpc, wpw))
+    us += c.many * rows + c.end * 1e-3 * std::min(std::min(0.4 * K, (double)f.n / 16.0), crowd * (double)f.n / 512.0);
+  else
+    us += c.serial * 0.1 * std::max(0.0, std::min(crowd * (double)wpw, 0.12 * K) - 5.0);
+  if (f.batch_warps == 0) return us < c.other + c.other_log * std::log2(std::max(2.0, K));
+  return us - 1.8 * (1.0 - moving) < batch_us(f, moving);   // (a zero step: no update, no walk of e)
 }
 
 cudaError_t run_cluster(int model, int layout, int prec, const CcdParams& P, int sweeps, cudaStream_t s) {

@@ -204,12 +204,17 @@ cudaError_t replay_until_stop(const CcdParams& P, cudaStream_t s, GraphCache* gc
 // which is for cohorts of at most kClusterMaxEnds tie groups (known later).
 constexpr int32_t kClusterMaxEnds = 32768;
 cudaError_t cluster_grid_size(int model, int layout, int prec, int64_t n, int64_t p, int* G, int* wpc);
-// Whether a fit of such a cohort (K tie groups; CSC: nnz stored entries a
-// column on average, with values or ones) is faster there than on the kernel
-// pair or, with `batches`, than in batches of four coordinates, of which a share
-// `moving` steps in a sweep.
-bool cluster_is_faster(int model, int layout, int prec, int64_t n, int32_t K, double nnz, bool values, bool batches,
-                       double moving);
+// Whether such a fit is faster there than on the kernel pair or, with
+// batch_warps (the warps of a full grid), than in batches of four coordinates, of
+// which a share `moving` steps in a sweep.
+struct FitShape {
+  int64_t n;
+  int32_t K, crowd;      // group ends, and the most of them among 32 rows
+  double nnz;            // CSC: stored entries of a column on average,
+  bool values;           //   with values (else all 1)
+  int64_t batch_warps;   // 0: no batches
+};
+bool cluster_is_faster(int model, int layout, int prec, const FitShape& f, double moving);
 // Up to `sweeps` sweeps of a fit (or the evaluation of P.single_j) in one
 // launch; *P.gctl zeroed before the first, which also sets eta = X beta and e.
 // P.gctl->done tells the stop.
@@ -276,7 +281,8 @@ cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr
 // Tie groups.  prep_group_count checks times and status codes (*perr) and
 // writes *K, *total_events (subjects with status 1), its block counts into cnt
 // (prep_count_bytes(n) bytes) and, with event [ceil(n / 32)], the events (bit r
-// of word w: row 32 w + r has status 1); *ticket is a zeroed word.
+// of word w: row 32 w + r has status 1); with crowd (zeroed before), the most
+// group ends among the 32 rows of a word; *ticket is a zeroed word.
 // prep_group_write then fills gend, dk and ck (ck may be null), with wk0 the
 // first group of each warp's rows, and with masks those of every 32 rows.
 struct RowMasks {              // [ceil(n / 32)] each
@@ -286,7 +292,7 @@ struct RowMasks {              // [ceil(n / 32)] each
 size_t prep_count_bytes(int64_t n);
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
                              unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s,
-                             uint32_t* event = nullptr);
+                             uint32_t* event = nullptr, int32_t* crowd = nullptr);
 cudaError_t prep_group_write(const int32_t* time, const int8_t* status, int64_t n, const void* cnt, int32_t K,
                              int32_t* gend, int32_t* dk, int32_t* ck, int32_t nwarps, int64_t rows_per_warp,
                              int32_t* wk0, cudaStream_t s, const RowMasks* masks = nullptr);

@@ -374,14 +374,14 @@ __device__ __forceinline__ bool quad_aligned(const int32_t* time, const int8_t* 
 __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time, const int8_t* status, int64_t n,
                                                              int model, int64_t nb, int32_t* cnt, unsigned* perr,
                                                              int32_t* K, int32_t* total_events, unsigned* ticket,
-                                                             uint32_t* event) {
+                                                             uint32_t* event, int32_t* crowd) {
   __shared__ unsigned s_w[kGrpThreads / 32];
   __shared__ int32_t s_p[3][kGrpThreads / 32];
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const bool vec = quad_aligned(time, status);
   const int64_t r0 = (int64_t)blockIdx.x * kGrpRows + w * (128 * kGrpRounds) + lane * 4;
-  unsigned c = 0, bad = 0;
+  unsigned c = 0, bad = 0, most = 0;
   RawQuad raw[kGrpRounds];
 #pragma unroll
   for (int it = 0; it < kGrpRounds; ++it) raw[it] = load_raw(time, status, n, r0 + 128 * it, vec);
@@ -394,6 +394,11 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
       const uint32_t ev = word_of(q.ev);
       if ((lane & 7) == 0 && r0 + 128 * it < n) event[(r0 + 128 * it) >> 5] = ev;
     }
+    if (crowd) most = max(most, (unsigned)__popc(word_of(q.end)));
+  }
+  if (crowd) {
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) atomicMax(crowd, (int32_t)most);
   }
   if (bad) atomicOr(perr, bad);
   c = __reduce_add_sync(0xffffffffu, c);
@@ -906,11 +911,11 @@ size_t prep_count_bytes(int64_t n) { return 3 * sizeof(int32_t) * (size_t)((n + 
 
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
                              unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s,
-                             uint32_t* event) {
+                             uint32_t* event, int32_t* crowd) {
   if (n <= 0) return cudaSuccess;
   const int64_t nb = (n + kGrpRows - 1) / kGrpRows;
   k_group_count<<<(unsigned)nb, kGrpThreads, 0, s>>>(time, status, n, model, nb, static_cast<int32_t*>(cnt), perr, K,
-                                                     total_events, ticket, event);
+                                                     total_events, ticket, event, crowd);
   return cudaGetLastError();
 }
 

@@ -26,9 +26,9 @@ def _cohort(model, layout, n, p, K, density, seed=5):
 
 
 @pytest.mark.parametrize("model,layout,n,K,density,one_cluster", [
-    ("cox", "csc", 50_000, 3650, 0.05, True), ("cox", "csc", 300_000, 3650, 0.5, False),
+    ("cox", "csc", 50_000, 3650, 0.05, True), ("cox", "csc", 300_000, 1000, 0.5, False),
     ("cox", "csc", 150_000, 40_000, 0.05, False), ("cox", "csc", 20_000, 40_000, 0.01, True),
-    ("fg", "csc", 100_000, 60, 0.02, True), ("fg", "csc", 200_000, 1000, 0.5, False),
+    ("fg", "csc", 100_000, 1000, 0.02, True), ("fg", "csc", 200_000, 1000, 0.5, False),
     ("cox", "dense", 30_000, 365, 1.0, False), ("cox", "dense", 8_000, 3650, 1.0, True),
     ("fg", "dense", 100_000, 10_000, 1.0, False), ("fg", "dense", 10_000, 1000, 1.0, True)])
 def test_route_of_a_fit(lib, model, layout, n, K, density, one_cluster):
