@@ -206,7 +206,16 @@ constexpr int kBtMaxG = 384;   // pass CTAs
 constexpr int kBtCluster = 16;
 inline bool btrans_one_cluster(int K) { return K <= 2 * kBtSmall * kBtCluster; }
 constexpr int kBtMaxCtas = kMaxTransCtas;
-inline int btrans_threads(int K) { return K <= kBtSmall * kBtMaxCtas ? kBtSmall : kBtLarge; }
+// Sparse Cox data in FP32, whose pass is the shortest, wants the larger blocks
+// from 8192 ends on: at 10,000 to 19,000 of them 79 to 148 small blocks start
+// later behind the pass than 20 to 38 large ones (us a coordinate at 3 x 10^6
+// rows, 128 and 512 threads: 26.4 and 23.5; dense and Fine-Gray data 0 to 5 % the
+// other way).
+template <int MODEL, int LAYOUT, typename T>
+inline int btrans_threads(int K) {
+  constexpr int most = MODEL == 0 && LAYOUT == 0 && sizeof(T) == 4 ? 8192 : kBtSmall * kBtMaxCtas;
+  return K <= most ? kBtSmall : kBtLarge;
+}
 
 template <int MODEL, int LAYOUT, typename T, int kBtNT, bool BATCH = false, bool CLUSTER = false>
 __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ CcdParams P0, int j) {
@@ -385,8 +394,7 @@ __global__ void __launch_bounds__(kBtNT, 1) k_btrans(const __grid_constant__ Ccd
 }
 
 // CTAs of the balanced transform: about one group end a thread.
-inline int btrans_ctas(int K) {
-  const int nt = btrans_threads(K);
+inline int btrans_ctas(int K, int nt) {
   return std::max(4, std::min(kBtMaxCtas, (K + nt - 1) / nt));
 }
 // Per fit of a batch: about four ends a thread (kBtSmall threads).
@@ -418,7 +426,8 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
-  const unsigned cl = (unsigned)std::min(kBtCluster, btrans_ctas(P.K));
+  const int bt = btrans_threads<MODEL, LAYOUT, T>(P.K);
+  const unsigned cl = (unsigned)std::min(kBtCluster, btrans_ctas(P.K, bt));
   cudaLaunchAttribute attr_cl[2];
   const bool cluster = P.nfit == 0 && btrans_one_cluster(P.K) &&
                        cluster_launch(k_btrans<MODEL, LAYOUT, T, kBtSmall, false, true>, cl, kBtSmall, attr[0], attr_cl);
@@ -443,9 +452,9 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps;
   const bool few_rows = P.nfit == 0 && P.wpw <= 16 && (Cfg<MODEL, LAYOUT, T>::ND > 1 || sizeof(T) == 8);
   auto kp = k_pass<MODEL, LAYOUT, T, false, false>;
-  auto kt = btrans_threads(P.K) == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;
-  ct.gridDim = dim3(btrans_ctas(P.K));
-  ct.blockDim = dim3(btrans_threads(P.K));
+  auto kt = bt == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;
+  ct.gridDim = dim3(btrans_ctas(P.K, bt));
+  ct.blockDim = dim3(bt);
   if (cluster) {
     kt = k_btrans<MODEL, LAYOUT, T, kBtSmall, false, true>;
     ct.gridDim = dim3(cl);
