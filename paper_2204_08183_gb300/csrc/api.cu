@@ -39,7 +39,8 @@ struct DevCtrl {
   int32_t total_events;
   unsigned counters[2];
   unsigned ticket;       // blocks of k_group_count done
-  int32_t crowd;         // most group ends among 32 rows (where asked for)
+  int32_t crowd[2];      // most group ends among 32 and 4096 rows (where asked for)
+  unsigned pad;
   double out[survgpu::OUT_COUNT];
   unsigned long long timing[survgpu::PH_COUNT];
   survgpu::GraphCtl gctl;
@@ -377,7 +378,7 @@ int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, St
     cols->event = event = static_cast<uint32_t*>(ev);
   }
   CUDA_TRY(survgpu::prep_group_count(st.time, st.status, n, model, *cnt, &ctrl->perr, &ctrl->K, &ctrl->total_events,
-                                     &ctrl->ticket, s, event, crowd ? &ctrl->crowd : nullptr));
+                                     &ctrl->ticket, s, event, crowd ? ctrl->crowd : nullptr));
   ++*launches;
   int64_t longest = n;
   if (layout == SURV_CSC) {
@@ -400,7 +401,7 @@ int validate_and_count(int model, int layout, int prec, int64_t n, int64_t p, St
   if ((rc = map_prep_error(hc.perr))) return rc;
   *K = hc.K;
   *events = hc.total_events;
-  if (crowd) *crowd = hc.crowd;
+  if (crowd) std::memcpy(crowd, hc.crowd, sizeof(hc.crowd));
   if (layout == SURV_CSC && st.vals && !(hc.perr & survgpu::PREP_VALUES_NOT_ONE)) st.vals = nullptr;
   return SURV_OK;
 }
@@ -507,7 +508,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   const int32_t* time_p = stg.time;
   const int8_t* status_p = stg.status;
   void* cnt = nullptr;
-  int32_t K = 0, events = 0, crowd = 0;
+  int32_t K = 0, events = 0, crowd[2] = {0, 0};
   survgpu::PrepColumns cols;
   int cols_nb = 0;
   void *woff = nullptr, *wk0 = nullptr;
@@ -519,7 +520,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     cols.woff = static_cast<int32_t*>(woff);
   }
   if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches, &cols,
-                               &cols_nb, cluster && single_j < 0 ? &crowd : nullptr)))
+                               &cols_nb, single_j < 0 ? crowd : nullptr)))
     return rc;
   if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   // Default fits of sparse Cox data in the FP32 mode: batches (see below) where
@@ -551,7 +552,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     int g = 0, w = 0;
     CUDA_TRY(survgpu::graph_grid_size(model, layout, prec, &g, &w));
     const bool batches = sparse_cox && few_ends((int64_t)g * w);
-    const survgpu::FitShape shape = {n, K, crowd, (double)stg.nnz / (double)p, stg.vals != nullptr,
+    const survgpu::FitShape shape = {n, K, crowd[0], (double)stg.nnz / (double)p, stg.vals != nullptr,
                                      batches ? (int64_t)g * w : 0};
     auto faster = [&](double moving) { return survgpu::cluster_is_faster(model, layout, prec, shape, moving); };
     stay = faster(1.0);
@@ -718,6 +719,8 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   P.Gk = static_cast<const double*>(Gk);
   P.Gkff = static_cast<const float2*>(Gkff);
   P.wk0 = static_cast<const int32_t*>(wk0);
+  P.warp_ends = (int32_t)((double)crowd[1] * (double)rows_per_warp /
+                              (double)std::min<int64_t>(n, survgpu::kGroupRows) + 0.5);
   P.endw = masks.end;
   P.wordk = masks.first;
   P.col_ptr = static_cast<const int64_t*>(colptr_d);

@@ -449,7 +449,13 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   // coordinate, the plain and the many-ends form: 20.9 and 18.2 at 500,009 x
   // 24 dense Cox, 31.8 and 26.7 at 200,003 x 40 sparse Fine-Gray; at 5 x 10^6
   // x 50 dense Fine-Gray the plain form, 49.0 against 52.4).
-  const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps;
+  // Not for Fine-Gray in FP32 where the ends are spread evenly, two to four a
+  // warp: its six (dense) or two components pay for the scan of each tile (us a
+  // coordinate at 3 x 10^6 rows with 10,000 even ends, the many-ends and the
+  // plain form: 54.2 and 44.1 dense, 43.9 and 39.0 at 10 % density; 57.6 and 65
+  // dense with 30,000).
+  constexpr int kEven = MODEL == 1 && sizeof(T) == 4 ? (LAYOUT == 1 ? 5 : 4) : 0;
+  const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps && (P.nfit > 0 || P.warp_ends >= kEven);
   const bool few_rows = P.nfit == 0 && P.wpw <= 16 && (Cfg<MODEL, LAYOUT, T>::ND > 1 || sizeof(T) == 8);
   auto kp = k_pass<MODEL, LAYOUT, T, false, false>;
   auto kt = bt == kBtSmall ? k_btrans<MODEL, LAYOUT, T, kBtSmall> : k_btrans<MODEL, LAYOUT, T, kBtLarge>;

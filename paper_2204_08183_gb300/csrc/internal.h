@@ -37,6 +37,8 @@ struct CcdParams {
   const double* Gk;      // [K] Kaplan-Meier censoring survival at t_k (FG)
   const float2* Gkff;    // [K] the same as float-float (hi, lo)
   const int32_t* wk0;    // [nwarps+1] first group index whose end is in warp w
+  int32_t warp_ends;     // about the most group ends of a warp (single fits)
+  int32_t unused;
   const uint32_t* endw;  // [ceil(n/32)] group ends among 32 rows (bit per row) and
   const int32_t* wordk;  //   group ends before them (many-ends form of the row pass)
 
@@ -281,14 +283,16 @@ cudaError_t prep_check_finite_f64(const double* v, int64_t count, unsigned* perr
 // Tie groups.  prep_group_count checks times and status codes (*perr) and
 // writes *K, *total_events (subjects with status 1), its block counts into cnt
 // (prep_count_bytes(n) bytes) and, with event [ceil(n / 32)], the events (bit r
-// of word w: row 32 w + r has status 1); with crowd (zeroed before), the most
-// group ends among the 32 rows of a word; *ticket is a zeroed word.
+// of word w: row 32 w + r has status 1); with crowd (two zeroed words), the most
+// group ends among the 32 rows of a word and among kGroupRows rows; *ticket is a zeroed
+// word.
 // prep_group_write then fills gend, dk and ck (ck may be null), with wk0 the
 // first group of each warp's rows, and with masks those of every 32 rows.
 struct RowMasks {              // [ceil(n / 32)] each
   uint32_t* end = nullptr;     // bit r: row 32 w + r ends a group
   int32_t* first = nullptr;    // group ends before row 32 w
 };
+constexpr int kGroupRows = 4096;   // subjects a block of the count
 size_t prep_count_bytes(int64_t n);
 cudaError_t prep_group_count(const int32_t* time, const int8_t* status, int64_t n, int model, void* cnt,
                              unsigned* perr, int32_t* K, int32_t* total_events, unsigned* ticket, cudaStream_t s,

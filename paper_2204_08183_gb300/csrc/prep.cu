@@ -305,6 +305,7 @@ __global__ void k_check_finite(const double* v, int64_t count, unsigned* perr) {
 constexpr int kGrpThreads = 256;
 constexpr int kGrpRounds = 4;
 constexpr int kGrpRows = kGrpThreads * 4 * kGrpRounds;
+static_assert(kGrpRows == kGroupRows, "rows of a block");
 
 struct RowQuad {
   unsigned end, ev, ce, bad;   // 4-bit masks of the quad's rows; prep error bits
@@ -370,7 +371,8 @@ __device__ __forceinline__ bool quad_aligned(const int32_t* time, const int8_t* 
 }
 
 // cnt [3][nb]: exclusive prefixes over the blocks of ends, events and
-// censored on exit.  *ticket is zero on entry and on exit.
+// censored on exit.  *ticket is zero on entry and on exit.  crowd (if given):
+// the most ends among 32 and among kGrpRows rows.
 __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time, const int8_t* status, int64_t n,
                                                              int model, int64_t nb, int32_t* cnt, unsigned* perr,
                                                              int32_t* K, int32_t* total_events, unsigned* ticket,
@@ -434,6 +436,14 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
   for (int64_t b = lo + kKeep; b < hi; ++b)
 #pragma unroll
     for (int m = 0; m < 3; ++m) sum[m] += __ldcg(cnt + m * nb + b);
+  if (crowd) {   // the most ends of a block
+    int32_t top = 0;
+#pragma unroll
+    for (int q = 0; q < kKeep; ++q) top = max(top, keep[0][q]);
+    for (int64_t b = lo + kKeep; b < hi; ++b) top = max(top, __ldcg(cnt + b));
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) atomicMax(crowd + 1, top);
+  }
   int32_t inc[3] = {sum[0], sum[1], sum[2]};
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1)
