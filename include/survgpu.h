@@ -128,7 +128,8 @@ typedef struct surv_opts {
  * kernels per coordinate replayed as a CUDA graph, one replay per sweep.
  * Both schedules compute the same quantities in the same order of
  * coordinates; this flag exists to compare them.  (Without flags, cohorts
- * that one thread-block cluster holds run in one launch on that cluster;
+ * for which one thread-block cluster is the fastest, by rows, group ends and
+ * stored entries, run there, in launches of up to 8192 coordinates;
  * loglik_grad_hess uses it too, and the persistent kernel for larger ones.) */
 #define SURV_FLAG_PERSISTENT 2
 /* cox_cv_path only, with ctas_per_fit = 0: time one sweep of the batched

@@ -8,7 +8,7 @@
 // exchange through distributed shared memory and the hardware's cluster
 // barrier, and every CTA takes the Newton step itself from the same numbers in
 // the same order, so a coordinate needs two cluster barriers and nothing else
-// (11 to 23 us; its row pass, on 16 SMs instead of 152, is the longest part,
+// (8 to 25 us, in FP64 11 to 45; its row pass, on 16 SMs instead of 152, is the longest part,
 // the two barriers take 1 us):
 //
 //   rows     each warp updates and passes over its own rows (warp_pass, the

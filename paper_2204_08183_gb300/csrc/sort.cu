@@ -21,7 +21,8 @@
 // Four passes of 8 bits, with one block scanning the whole count table (8.6
 // ms of it) and scatters straight from registers, took 9.3 ms of device time
 // at n = 10^7 and days 1..3650; ordering and grouping such records takes
-// 1.34 instead of 10.45 ms in all.
+// 0.88 instead of 10.35 ms in all (with the tie-group table in two passes and the
+// scratch pool).
 #include <algorithm>
 #include <cstdint>
 

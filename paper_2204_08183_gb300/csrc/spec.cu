@@ -532,7 +532,6 @@ struct IpCfg {
 // threads on more CTAs: 15 % more than with 512).
 constexpr int kItNT = 512;
 constexpr int kItWarps = kItNT / 32;
-constexpr int kItAgg = 1;
 
 // Position of the warp's group end k (k warp-uniform): lane registers for
 // the first 32, a broadcast load beyond.
@@ -726,7 +725,7 @@ __global__ void __launch_bounds__(kSpNT, 2) k_ipass(const __grid_constant__ CcdP
 template <int B>
 __global__ void __launch_bounds__(kItNT, 1) k_itrans(const __grid_constant__ CcdParams P, int slot) {
   constexpr int R = IpCfg<B>::R, NP = IpCfg<B>::NP, NPP = IpCfg<B>::NPP;
-  __shared__ ff s_T[kItNT * kItAgg][R];       // exclusive prefix of the pass CTAs' aggregates
+  __shared__ ff s_T[kItNT][R];           // exclusive prefix of the pass CTAs' aggregates
   __shared__ ff s_w[kItWarps][R];
   __shared__ ff s_red[kItWarps][NP];
   __shared__ ff s_tot[NP];
@@ -770,7 +769,7 @@ __global__ void __launch_bounds__(kItNT, 1) k_itrans(const __grid_constant__ Ccd
   pdl_wait();
 
   // prefixes of the pass CTAs' aggregates
-  scan_aggregates<kItNT, kItAgg, R, ff>(P.agg, G, s_T, s_w, nullptr);
+  scan_aggregates<kItNT, 1, R, ff>(P.agg, G, s_T, s_w, nullptr);
   __syncthreads();
 
   // G_k of the batch's columns at the group ends (steps 3-4); column 0's
@@ -884,7 +883,7 @@ cudaError_t capture_spec(const CcdParams& P, int S, bool pdl, cudaStream_t cs, c
   // indicator columns: the lockstep walks and the ranged transform
   const bool ind = P.values == nullptr;
   if (ind) {
-    if (P.G > kItNT * kItAgg) return cudaErrorInvalidValue;   // the transform scans kItAgg aggregates a thread
+    if (P.G > kItNT) return cudaErrorInvalidValue;   // the transform scans one aggregate a thread
     ct.gridDim = dim3(itrans_ctas(P.K, B));
     ct.blockDim = dim3(kItNT);
   }
