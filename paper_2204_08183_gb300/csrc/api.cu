@@ -509,7 +509,8 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   const int32_t* time_p = stg.time;
   const int8_t* status_p = stg.status;
   void* cnt = nullptr;
-  int32_t K = 0, events = 0, crowd[2] = {0, 0};
+  int32_t K = 0, events = 0, crowd[2] = {0, 0};   // (for the cluster's rule and Fine-Gray's row pass)
+  const bool wants_crowd = single_j < 0 && (cluster || (graph && model == SURV_FG && prec == 0));
   survgpu::PrepColumns cols;
   int cols_nb = 0;
   void *woff = nullptr, *wk0 = nullptr;
@@ -521,7 +522,7 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     cols.woff = static_cast<int32_t*>(woff);
   }
   if ((rc = validate_and_count(model, layout, prec, n, p, stg, ctrl, ws, s, &cnt, &K, &events, &launches, &cols,
-                               &cols_nb, single_j < 0 ? crowd : nullptr)))
+                               &cols_nb, wants_crowd ? crowd : nullptr)))
     return rc;
   if (events <= 0) { set_error("no events"); return SURV_E_NO_EVENTS; }
   // Default fits of sparse Cox data in the FP32 mode: batches (see below) where

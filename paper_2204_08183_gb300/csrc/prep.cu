@@ -398,14 +398,18 @@ __global__ void __launch_bounds__(kGrpThreads) k_group_count(const int32_t* time
     }
     if (crowd) most = max(most, (unsigned)__popc(word_of(q.end)));
   }
-  if (crowd) {
-    most = __reduce_max_sync(0xffffffffu, most);
-    if (lane == 0) atomicMax(crowd, (int32_t)most);
-  }
   if (bad) atomicOr(perr, bad);
   c = __reduce_add_sync(0xffffffffu, c);
-  if (lane == 0) s_w[w] = c;
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 0) {
+    s_w[w] = c;
+    s_p[0][w] = (int32_t)most;
+  }
   __syncthreads();
+  if (crowd && tid == 32) {
+    for (int q = 0; q < kGrpThreads / 32; ++q) most = max(most, (unsigned)s_p[0][q]);
+    atomicMax(crowd, (int32_t)most);
+  }
   if (tid < 3) {
     int32_t v = 0;
     for (int q = 0; q < kGrpThreads / 32; ++q) v += (int32_t)(s_w[q] >> (10 * tid) & 1023u);
