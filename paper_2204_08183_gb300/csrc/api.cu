@@ -484,16 +484,16 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   if ((rc = partition(o.flags == 0))) return rc;
 
   // ---------------------------------------------------------- staging
+  // host copies of beta and penalty factors (p values each), before the call's
+  // own work is on the stream that they wait for
+  std::vector<double> beta_h(p), pf_h(p, 1.0), pen_h(p);
+  if ((rc = to_host(beta_inout, 8 * (size_t)p, beta_h.data(), s))) return rc;
+  if (o.penalty_factor && (rc = to_host(o.penalty_factor, 8 * (size_t)p, pf_h.data(), s))) return rc;
   Staged stg;
   if ((rc = stage_data(d, prec, ws, s, &stg, &launches))) return rc;
   const void *colptr_d = stg.colptr, *rowidx_d = stg.rowidx;
   const int64_t ld = stg.ld;
   const std::vector<int64_t>& colptr_h = stg.colptr_h;
-
-  // host copies of beta and penalty factors (p values each)
-  std::vector<double> beta_h(p), pf_h(p, 1.0), pen_h(p);
-  if ((rc = to_host(beta_inout, 8 * (size_t)p, beta_h.data(), s))) return rc;
-  if (o.penalty_factor && (rc = to_host(o.penalty_factor, 8 * (size_t)p, pf_h.data(), s))) return rc;
   for (int64_t j = 0; j < p; ++j) {
     if (!std::isfinite(beta_h[j]) || !std::isfinite(pf_h[j]) || pf_h[j] < 0.0) {
       set_error("non-finite beta or invalid penalty factor at %lld", (long long)j);
@@ -534,10 +534,10 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
   if ((rc = ensure(ws, W::DK, 4 * (size_t)K, &dk))) return rc;
   if ((rc = ensure(ws, W::CK, 4 * (size_t)K, &ck))) return rc;
   survgpu::RowMasks masks;
-  if ((rc = row_masks(ws, n, &masks))) return rc;
   bool grouped = false;   // the group tables are written
   auto write_groups = [&]() -> int {
     if ((rc = ensure(ws, W::WK0, 4 * (size_t)(nwarps + 1), &wk0))) return rc;
+    if ((rc = row_masks(ws, n, &masks))) return rc;
     if (grouped)
       CUDA_TRY(survgpu::prep_warp_groups(static_cast<int32_t*>(gend), K, n, nwarps, rows_per_warp,
                                          static_cast<int32_t*>(wk0), s));
@@ -595,8 +595,6 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
       ++launches;
     }
   }
-  if (!grouped || !cluster)
-    if ((rc = write_groups())) return rc;
   const void* vals_d = stg.vals;  // null for indicator CSC data (all values 1)
   DevCtrl hc;
 
@@ -662,6 +660,8 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     S.multi = (int64_t)K >= 2 * (int64_t)nwarps ? 1 : 0;
   }
 
+  if (!grouped || !cluster)   // (a cluster's, written for its rule, stand)
+    if ((rc = write_groups())) return rc;
   if (model == SURV_FG) {
     CUDA_TRY(survgpu::prep_km(static_cast<int32_t*>(gend), static_cast<int32_t*>(ck), K, static_cast<double*>(Gk), s));
     // the records are not in use yet: scratch for 1 / G

@@ -352,46 +352,47 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
         // acc_dirty is false) and an exclusive lane scan of the lanes' totals in
         // twice the working precision, and a lane walks its rows up to each end.
         // One component at a time: the scans of a tile need few registers.
-        const unsigned who = __ballot_sync(0xffffffffu, nib != 0u);
-        const bool any = who != 0u;
-        if (sizeof(T) == 8 && any && (who & (who - 1u)) == 0u &&
-            !__any_sync(0xffffffffu, (nib & (nib - 1u)) != 0u)) {
-          // One end in an FP64 tile: a tree over the partials and the rows up to it
-          // instead of the sum and the scan, which is most of the pass there (us a
-          // coordinate, dense Fine-Gray at 10^6 rows with 10,000 even ends: 157 with
-          // the scan, 121 with the tree; in FP32 the tree gained nothing).
-          A pref[ND];
+        if constexpr (sizeof(T) == 8) {
+          const unsigned who = __ballot_sync(0xffffffffu, nib != 0u);
+          if (who != 0u && (who & (who - 1u)) == 0u && !__any_sync(0xffffffffu, (nib & (nib - 1u)) != 0u)) {
+            // One end in an FP64 tile: a tree over the partials and the rows up to it
+            // instead of the sum and the scan, which is most of the pass there (us a
+            // coordinate, dense Fine-Gray at 10^6 rows with 10,000 even ends: 157 with
+            // the scan, 121 with the tree; in FP32 the tree gained nothing).
+            A pref[ND];
 #pragma unroll
-          for (int d = 0; d < ND; ++d) {
-            T part = T(0);
+            for (int d = 0; d < ND; ++d) {
+              T part = T(0);
 #pragma unroll
-            for (int u = 0; u < U; ++u)
+              for (int u = 0; u < U; ++u)
 #pragma unroll
-              for (int q = 0; q < VEC; ++q) {
-                const T v = dense_comp<MODEL, LAYOUT, T>(d, ev[u][q], xv[u][q], wv[u][q]);
-                // the rows before the end's lane, and those up to the end in it
-                if (who >> lane > 1u || (nib >> (u * VEC + q)) != 0u) part += v;
-              }
-            pref[d] = acc_add_v(acc[d], part);
-            T su[U];
+                for (int q = 0; q < VEC; ++q) {
+                  const T v = dense_comp<MODEL, LAYOUT, T>(d, ev[u][q], xv[u][q], wv[u][q]);
+                  // the rows before the end's lane, and those up to the end in it
+                  if (who >> lane > 1u || (nib >> (u * VEC + q)) != 0u) part += v;
+                }
+              pref[d] = acc_add_v(acc[d], part);
+              T su[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) su[u] = chunk_sum(d, ev, xv, wv, u);
+              for (int u = 0; u < U; ++u) su[u] = chunk_sum(d, ev, xv, wv, u);
 #pragma unroll
-            for (int s = 1; s < U; s <<= 1)
+              for (int s = 1; s < U; s <<= 1)
 #pragma unroll
-              for (int u = 0; u + s < U; u += 2 * s) su[u] += su[u + s];
-            acc[d] = acc_add_v(acc[d], su[0]);
+                for (int u = 0; u + s < U; u += 2 * s) su[u] += su[u + s];
+              acc[d] = acc_add_v(acc[d], su[0]);
+            }
+            warp_sum_set<ND, WIDE>(pref);
+            if (nib) {
+              const int64_t r = row_of(t0, 0);
+              const int k = P.wordk[r >> 5] + __popc(P.endw[r >> 5] & ((1u << (r & 31)) - 1u));
+#pragma unroll
+              for (int d = 0; d < ND; ++d) rec[(size_t)k * M + C::dmap(d)] = pref[d];
+            }
+            acc_dirty = true;
+            return;
           }
-          warp_sum_set<ND, WIDE>(pref);
-          if (nib) {
-            const int64_t r = row_of(t0, 0);
-            const int k = P.wordk[r >> 5] + __popc(P.endw[r >> 5] & ((1u << (r & 31)) - 1u));
-#pragma unroll
-            for (int d = 0; d < ND; ++d) rec[(size_t)k * M + C::dmap(d)] = pref[d];
-          }
-          acc_dirty = true;
-          return;
         }
+        const bool any = __any_sync(0xffffffffu, nib != 0u);
         if (any && acc_dirty) warp_sum_set<ND, WIDE>(acc);
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
