@@ -560,10 +560,10 @@ int fit_common(int model, const surv_data* d, const surv_opts* o_in, double* bet
     stay = faster(1.0);
     // An L1 fit may move few of its coordinates, and batches then take several a
     // row pass.  Which way it goes shows at the start: the nonzeros of a warm
-    // beta, or at beta = 0 the gradients beyond their strengths (five small
-    // kernels and one wait, 40 us; not for 8 coordinates or fewer, where a fit is
-    // not longer than that).  Sparse Cox at 200,000 x 60, of which 20 move: 1.41
-    // ms in batches, 2.33 on the cluster.
+    // beta, or at beta = 0 the gradients beyond their strengths (a few
+    // small kernels and one wait, 46 us; not for 8 coordinates or fewer, where a
+    // fit is hardly longer).  Four sweeps of sparse Cox at 200,000 x 60, 5 %, 7
+    // coordinates in the end: 2.56 ms in batches, 3.70 on the cluster.
     if (batches && o.penalty == SURV_PEN_L1 && p > 8 && faster(0.0) != stay) {
       int64_t moving = 0;
       for (double b : beta_h) moving += b != 0.0;

@@ -447,11 +447,13 @@ cudaError_t launch_cluster(const CcdParams& P, int sweeps, cudaStream_t s) {
 // the rows, by K (0.4 and 0.12 of it for exponential times) and by `crowd`, the
 // most ends among 32 rows; f = min(1, K/300) min(1, (crowd + 1)/3) the share of
 // entry rounds with an end.  Of the kernel pair on the whole chip:
-// other + other_log log2 K, where n hardly counts.  Least squares over 4,600
+// other + other_log log2 K, where n hardly counts.  Least squares over 5,100
 // fits of 300 to 300,000 rows with exponential, censored and uniform times, 40 to
-// 39,000 ends and 0.5 to 50 % density: 4 to 9 % rms.  The choice between the two
-// costs 0.3 to 1 % on average against the faster one, and at most 12 % more than
-// the schedule that stood before the cluster.  Limits on n and on K alone lost
+// 39,000 ends and 0.5 to 50 % density: 4 to 9 % rms (the cluster on sparse data in
+// FP32 14 to 15, the pair on sparse Fine-Gray 11).  The choice between the two
+// costs 0 to 1.1 % on average against the faster one (up to 56 % for single fits
+// next to the line), and at most 12 % more than the schedule that stood before
+// the cluster (20 fits more than 5 %).  Limits on n and on K alone lost
 // where both were near them or columns dense (ms a fit, cluster and pair: 7.6
 // and 1.6 for sparse Cox at 300,000 x 60 with half of the entries stored, 9.8
 // and 8.7 at 5 % with 27,000 ends; 7.5 and 4.3 for sparse Fine-Gray at 262,000 x

@@ -358,7 +358,7 @@ __device__ __forceinline__ void warp_pass(const CcdParams& P, int j, int64_t row
             // One end in an FP64 tile: a tree over the partials and the rows up to it
             // instead of the sum and the scan, which is most of the pass there (us a
             // coordinate, dense Fine-Gray at 10^6 rows with 10,000 even ends: 157 with
-            // the scan, 121 with the tree; in FP32 the tree gained nothing).
+            // the scan, 131 with the tree; in FP32 the tree gained nothing).
             A pref[ND];
 #pragma unroll
             for (int d = 0; d < ND; ++d) {

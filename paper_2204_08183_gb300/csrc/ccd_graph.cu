@@ -209,8 +209,8 @@ constexpr int kBtMaxCtas = kMaxTransCtas;
 // Sparse Cox data in FP32, whose pass is the shortest, wants the larger blocks
 // from 8192 ends on: at 10,000 to 19,000 of them 79 to 148 small blocks start
 // later behind the pass than 20 to 38 large ones (us a coordinate at 3 x 10^6
-// rows, 128 and 512 threads: 26.4 and 23.5; dense and Fine-Gray data 0 to 5 % the
-// other way).
+// rows, 128 and 512 threads: 26.4 and 24.1; 6 % on average over even, 2 % over
+// exponential times; other data between 1 % this and 6 % the other way).
 template <int MODEL, int LAYOUT, typename T>
 inline int btrans_threads(int K) {
   constexpr int most = MODEL == 0 && LAYOUT == 0 && sizeof(T) == 4 ? 8192 : kBtSmall * kBtMaxCtas;
@@ -452,7 +452,7 @@ cudaError_t capture_sweep(const CcdParams& P, bool pdl, cudaStream_t cs, cudaGra
   // Not for Fine-Gray in FP32 where the ends are spread evenly, two to four a
   // warp: its six (dense) or two components pay for the scan of each tile (us a
   // coordinate at 3 x 10^6 rows with 10,000 even ends, the many-ends and the
-  // plain form: 54.2 and 44.1 dense, 43.9 and 39.0 at 10 % density; 57.6 and 65
+  // plain form: 54.3 and 44.1 dense, 44.4 and 39.0 at 10 % density; 57.6 and 63.1
   // dense with 30,000).
   constexpr int kEven = MODEL == 1 && sizeof(T) == 4 ? (LAYOUT == 1 ? 5 : 4) : 0;
   const bool many = (int64_t)P.K >= 2 * (int64_t)P.nwarps && (P.nfit > 0 || P.warp_ends >= kEven);
